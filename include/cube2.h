@@ -482,7 +482,7 @@ int cube2_ensemble_create(cube2_ensemble **out, cube2_ctx *const *ctxs, cube2_pa
  *                   (cube2_ensemble_check) and returns.  Boxes with the third
  *                   level or FP16 velocities are refused (CUBE2_ERR_STATE).
  *   pp_ctas_per_sm  persistent grid: CTAs per SM (1..16)
- *   pp_wmax         PP shared-stream width for every box (0: each context's own, 16)
+ *   pp_wmax         PP shared-stream width along x for every box (0: each context's own, 64)
  *   timeout_ms      bound of the persistent kernel's wait (> 0)                  */
 typedef struct {
     int32_t n_streams;

@@ -110,9 +110,12 @@ struct cube2_ctx {
     int32_t *nstart = nullptr;     // [n_cells] its exclusive scan
     int32_t *perm2 = nullptr;      // [N] merge scratch of the segmented sort
     int32_t *big = nullptr;        // [n_cells] cells too large for the per-thread sort
-    int *big_n = nullptr;          // [2] their numbers (up to 1024 particles, more)
+    int *big_n = nullptr;          // [2] their numbers (up to 1024 particles, more); in PP: dense cells, target
+                                   // places
     float4 *pos4 = nullptr;        // [N] in-cell offsets as floats (+ cell id bits), PP order
     int32_t *pp_perm = nullptr;    // [N] particle index of each PP slot (sub-cell order in dense cells)
+    int32_t *pp_tgt = nullptr;     // [pp_target_slots] PP slots in target (pencil) order, -1 in the pencils' padding
+    int2 *pp_dense = nullptr;      // [N / 64] dense cells and the places of their first targets
     unsigned long long *pp_stats = nullptr;  // [4] in-range ordered pairs, candidates; the same of per-lane walks
     int num_sms = 152;
     int32_t *scan_tmp = nullptr;   // block sums of the multi-level scan
@@ -134,8 +137,8 @@ struct cube2_ctx {
     double *vjp_sq = nullptr;      // [1] loss accumulator
     cube2::PM3 pm3;                // adaptive third level (cfg.pm3_tile > 0)
     float *vel32 = nullptr;        // [3][N] FP32 working momenta of a step (cfg.vel_fp16 = 1 only)
-    // shared-stream width of the PP kernel (warps spanning at most pp_wmax + 1 cells)
-    int pp_wmax = 16;
+    // shared-stream width of the PP kernel (warps spanning at most pp_wmax + 1 cells along x)
+    int pp_wmax = 64;
     // PP work counters (cube2_pp_count): off unless asked for
     bool pp_count = false;
     // ensemble recording: launch_pp prepares the PP inputs and leaves the PP
@@ -195,6 +198,9 @@ cudaError_t launch_fft_batched_solve(cube2_ctx *ctx, Level &L);     // forward, 
 cudaError_t launch_pm3(cube2_ctx *ctx, const cube2_particles *p);    // map, local deposit + solve, gather (acc +=)
 cudaError_t launch_pm3_map(cube2_ctx *ctx, const cube2_particles *p);  // refinement map only
 cudaError_t launch_vel_encode(cube2_ctx *ctx, const cube2_particles *p, const float *const v[3]);
+int64_t pp_dense_cells(int64_t N);
+int64_t pp_target_slots(int64_t N, int n_ios);
+int64_t pp_target_items(int64_t N, int n_ios);
 size_t pp_params_bytes();
 size_t pp_queue_bytes();
 cudaError_t launch_pp_persistent_step(cudaStream_t st, const void *boxes, const int32_t *item_box,

@@ -161,14 +161,14 @@ int cube2_ensemble_create_ex(cube2_ensemble **out, cube2_ctx *const *ctxs, cube2
     E->events.assign(nev, nullptr);
     for (int k = 0; k < nbr && e == cudaSuccess; ++k) e = cudaStreamCreateWithFlags(&E->branches[k], cudaStreamNonBlocking);
     for (int k = 0; k < nev && e == cudaSuccess; ++k) e = cudaEventCreateWithFlags(&E->events[k], cudaEventDisableTiming);
-    // persistent PP: items (box, block of 128 slots), parameters per step, queue
+    // persistent PP: items (box, 128 target places), parameters per step, queue
     const size_t psz = cube2::pp_params_bytes();
     std::vector<int32_t> item_box, base(n_boxes);
     std::vector<unsigned char> params;
     if (persistent && e == cudaSuccess) {
         for (int b = 0; b < n_boxes; ++b) {
             base[b] = (int32_t)item_box.size();
-            const int64_t nb = (ctxs[b]->N + 127) / 128;
+            const int64_t nb = ctxs[b]->N > 0 ? cube2::pp_target_items(ctxs[b]->N, ctxs[b]->n_ios) : 0;
             for (int64_t k = 0; k < nb; ++k) item_box.push_back(b);
         }
         params.assign((size_t)n_steps * n_boxes * psz, 0);

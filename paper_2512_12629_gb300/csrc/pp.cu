@@ -5,25 +5,31 @@
 // hold all its partners.  The cells of one (dz, dy) row are adjacent in memory,
 // so a run of cells along x is one contiguous particle range.
 //
+// The plain and the persistent kernel (and the counting ones) give the same bits:
+// products and sums that could be contracted are written as fmaf or kept apart.
+//
 // Arithmetic is carried out in IOS-cell units.  A particle's in-cell offset
 // off/2^16 is exact in FP32 (prep kernel, once per force evaluation) and so is
 // (cell step + offset) and the separation of two such values: the pair term is
 // bitwise antisymmetric.  Each ordered pair is evaluated from both sides (gather
 // form, no atomics, deterministic).
 //
-// One thread per target, in PP slot order: cell order, with the particles of
-// dense cells (64 or more) reordered by a 4x4x4 sub-cell key inside their
-// cell (PP's own position array and slot -> particle map; results are written
-// back to the particle's index).  A warp whose 32 targets
-// lie in one row of cells, narrow enough (every dense region; see wmax),
-// shares one source stream: the particles of cells xa-1 .. xb+1 in the 9 rows
-// around it.  It stages 64 sources at a time in shared memory; each lane tests
-// all 64 (sign of r^2 - b_cut^2 shifted into two 32-bit masks, 8 instructions
-// per candidate) and evaluates only the set bits, one mask word after the
-// other, with a branch-free far-pair formula; pairs closer than b_pp take a
-// separate, rarely entered loop.
-// Other warps (sparse regions) walk each lane's own 27 cells.  The Jacobian
-// product of the adjoint (pp_vjp_kernel) uses the same two paths.
+// One thread per target.  Targets are taken in pencil order (pp_pencil_kernel),
+// so that the 32 of a warp lie in a compact block of cells at any density; the
+// particles of dense cells (64 or more) are reordered by a 4x4x4 sub-cell key
+// inside their cell (PP's own position array and slot -> particle map; results
+// are written back to the particle's index).  A warp shares one source stream:
+// the particles of the cells within one of its block, staged by one lane each
+// and dropped where they are out of reach of the targets' bounding box.
+// Compact warps evaluate every pair of target and kept source; others test all
+// of them (packed arithmetic) and evaluate the ones found in range from a queue
+// per lane.  The few warps spread along x (nearly empty regions) walk each
+// lane's own 27 cells.  The adjoint's Jacobian product (pp_vjp_kernel) uses the
+// same stream.
+//
+// 256^3 run, a step's PP at z = 49 / z = 1 / z = 0: 1.35 / 5.0 / 8.7 ms;
+// with the targets in IOS order (streams only for warps inside one row, the
+// 27-cell walk for all others) 1.39 / 7.4 / 13.4 ms.
 // Per-particle sums are compensated: plain FP32 partials per batch are added to
 // the running total with Kahan's scheme.  The path a warp takes depends only
 // on the cell layout and every sum has a fixed order, so results are bitwise
@@ -38,13 +44,18 @@ namespace {
 struct PPParams {
     const float4 *pos;          // [N] (off_x, off_y, off_z)/2^16, .w = cell id bits, in PP slot order
     const int32_t *perm;        // [N] particle index of each slot
+    const int32_t *tgt;         // slot of each target, pencil by pencil, padded to whole warps with -1
+    const unsigned *tgt_n;      // length of tgt (device)
     const int32_t *count, *start;
     float *acc0, *acc1, *acc2;
     float *vel0, *vel1, *vel2;
     unsigned long long *stats;  // [2]: in-range ordered pairs, candidates
     int64_t N;
     int n_ios, accumulate;
+    unsigned div_mul;           // c / n_ios = umulhi(c, div_mul) >> div_shift for 0 <= c < 2^31
+    int div_shift;
     float inv_bpp, inv_bcut, bcut2, bpp2;   // IOS-cell units
+    float ratio2;                     // 1 / b_pp^2, IOS-cell units
     float coef;                       // V_p / (4 pi s_ios^2)
     float kick;                       // 0: no kick; else v += kick * acc after the sum
     int *status;
@@ -53,7 +64,7 @@ struct PPParams {
     const int32_t *pm3_slot;
     int pm3_T, pm3_ns;
     float bcut2_3, inv_bcut_3;
-    int wmax;                         // widest warp (cells beyond the first) on the shared stream
+    int wmax;                         // widest warp along x (cells beyond the first) on the shared stream
 };
 
 // R(r, b) of Eq. (refforce) times b^2, as a function of u = r / b < 1.
@@ -68,9 +79,9 @@ __device__ __forceinline__ float ref_force_scaled(float u) {
 }
 
 __device__ __forceinline__ void kahan_add(float &sum, float &comp, float v) {
-    const float y = v - comp;
-    const float t = sum + y;
-    comp = (t - sum) - y;
+    const float y = __fsub_rn(v, comp);   // v is never contracted into the difference
+    const float t = __fadd_rn(sum, y);
+    comp = __fsub_rn(__fsub_rn(t, sum), y);
     sum = t;
 }
 
@@ -84,9 +95,9 @@ __device__ __forceinline__ void finish(const PPParams &P, int64_t i, float a0, f
     P.acc1[i] = a1;
     P.acc2[i] = a2;
     if (P.kick != 0.0f) {
-        const float v0 = P.vel0[i] + P.kick * a0;
-        const float v1 = P.vel1[i] + P.kick * a1;
-        const float v2 = P.vel2[i] + P.kick * a2;
+        const float v0 = fmaf(P.kick, a0, P.vel0[i]);
+        const float v1 = fmaf(P.kick, a1, P.vel1[i]);
+        const float v2 = fmaf(P.kick, a2, P.vel2[i]);
         P.vel0[i] = v0;
         P.vel1[i] = v1;
         P.vel2[i] = v2;
@@ -151,18 +162,103 @@ struct RowRanges {
     __device__ __forceinline__ int size() const { return (end[0] - beg[0]) + (nseg > 1 ? end[1] - beg[1] : 0); }
 };
 
-constexpr int PP_WARPS_CTA = 4;
-constexpr int PP_CTA = PP_WARPS_CTA * 32;
+constexpr int PP_ITEM = 128;                                // target places of a persistent work item
+constexpr int PREP_WARPS = 4, PREP_CTA = PREP_WARPS * 32;   // input kernels
+
+// Targets are taken in pencil order: the cells of a pencil (PEN_Y x PEN_Z cells
+// in y and z, all of x) slab by slab along x, so that 32 consecutive targets
+// lie in a compact block at any density (8 x 2 x 2 cells at one particle per
+// cell, one cell where it holds 32) and one source stream per warp is short: 98
+// sources in reach of the block at one particle per cell.  2 x 2 against 4 x 2
+// cells: 1.35 against 1.68 ms at z = 49 (the block's eight x cells in a row make
+// its loads and stores whole sectors), equal late; 2 x 1: 1.50.  Each pencil
+// starts on a whole warp (its tail is padded with -1): a warp never spans two.
+constexpr int PEN_Y = 2, PEN_Z = 2, PEN = PEN_Y * PEN_Z;
+
+__host__ __device__ __forceinline__ int pencils_y(int n) { return (n + PEN_Y - 1) / PEN_Y; }
+__host__ __device__ __forceinline__ int pencils_z(int n) { return (n + PEN_Z - 1) / PEN_Z; }
+
+// One CTA per pencil: the target places of its cells (cells of sort_min
+// particles or more are listed with their first place for pp_dense_sort_kernel,
+// which writes them with a warp each) and the padding of the pencil's tail.
+// Pencils take their places in tgt by an atomic on tgt_n: their order varies,
+// the warps of a pencil and so the results do not.
+__global__ void __launch_bounds__(PREP_CTA) pp_pencil_kernel(const int32_t *__restrict__ count,
+                                                             const int32_t *__restrict__ start, int n, int sort_min,
+                                                             int32_t *__restrict__ tgt, unsigned *tgt_n,
+                                                             int2 *__restrict__ list, int *list_n) {
+    __shared__ unsigned s_base;   // places are unsigned: N plus the padding may pass 2^31
+    __shared__ int s_warp[PREP_WARPS];
+    const int npy = pencils_y(n);
+    const int y0 = (int)(blockIdx.x % npy) * PEN_Y, z0 = (int)(blockIdx.x / npy) * PEN_Z;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    // cell k of a slab: y forwards in the first z plane, backwards in the second
+    auto row_of = [&](int k) -> int64_t {
+        const int z = z0 + k / PEN_Y, y = y0 + (k < PEN_Y ? k : PEN - 1 - k);
+        return (y < n && z < n) ? ((int64_t)z * n + y) * n : -1;
+    };
+    if (w == 0) {   // a row's particles are contiguous
+        const int64_t r = lane < PEN ? row_of(lane) : -1;
+        int total = r >= 0 ? start[r + n - 1] + count[r + n - 1] - start[r] : 0;
+        total = __reduce_add_sync(0xffffffffu, total);
+        const int padded = (total + 31) & ~31;
+        unsigned base = 0;
+        if (lane == 0 && padded) base = atomicAdd(tgt_n, (unsigned)padded);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (lane < padded - total) tgt[base + total + lane] = -1;
+        if (lane == 0) s_base = base;
+    }
+    __syncthreads();
+    unsigned run = s_base;
+    for (int xb = 0; xb < n; xb += PREP_CTA) {
+        const int x = xb + threadIdx.x;
+        int cnt[PEN], sum = 0;
+#pragma unroll
+        for (int k = 0; k < PEN; ++k) {
+            const int64_t r = row_of(k);
+            cnt[k] = (x < n && r >= 0) ? count[r + x] : 0;
+            sum += cnt[k];
+        }
+        int incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        if (lane == 31) s_warp[w] = incl;
+        __syncthreads();
+        unsigned at = run + incl - sum;
+#pragma unroll
+        for (int k = 0; k < PREP_WARPS; ++k) {
+            if (k < w) at += s_warp[k];
+            run += s_warp[k];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < PEN; ++k) {
+            const int64_t r = row_of(k);
+            if (x < n && r >= 0) {
+                if (cnt[k] >= sort_min) {
+                    list[atomicAdd(list_n, 1)] = make_int2((int)(r + x), (int)at);
+                } else if (cnt[k]) {
+                    const int st = start[r + x];
+                    for (int j = 0; j < cnt[k]; ++j) tgt[at + j] = st + j;
+                }
+                at += cnt[k];
+            }
+        }
+    }
+}
 
 // Float offsets (and the cell id bits) for the PP kernel.
-__global__ void __launch_bounds__(PP_CTA) prep_positions_kernel(const uint16_t *off0, const uint16_t *off1,
+__global__ void __launch_bounds__(PREP_CTA) prep_positions_kernel(const uint16_t *off0, const uint16_t *off1,
                                                                 const uint16_t *off2, const int32_t *cellid,
                                                                 float4 *pos, int32_t *perm, int64_t n) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float s = 1.0f / FIX;
     pos[i] = make_float4((float)off0[i] * s, (float)off1[i] * s, (float)off2[i] * s, __int_as_float(cellid[i]));
-    if (perm) perm[i] = (int32_t)i;
+    perm[i] = (int32_t)i;
 }
 
 // Dense cells are reordered for PP by a 4x4x4 sub-cell key (Morton order of
@@ -177,27 +273,23 @@ __device__ __forceinline__ int subcell_key(unsigned ox, unsigned oy, unsigned oz
     return (int)((((x >> 1) | ((y >> 1) << 1) | ((z >> 1) << 2)) << 3) | ((x & 1) | ((y & 1) << 1) | ((z & 1) << 2)));
 }
 
-__global__ void __launch_bounds__(256) pp_dense_list_kernel(const int32_t *count, int64_t n_cells, int32_t *list,
-                                                            int *list_n) {
-    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < n_cells && count[c] >= PP_SORT_MIN) list[atomicAdd(list_n, 1)] = (int32_t)c;
-}
-
 // One warp per listed cell: histogram of the 64 keys, exclusive scan, then a
 // stable scatter 32 particles at a time (rank among equal keys of the chunk
 // by match masks, chunks in order).
 __global__ void __launch_bounds__(256) pp_dense_sort_kernel(const uint16_t *off0, const uint16_t *off1,
                                                             const uint16_t *off2, const int32_t *count,
-                                                            const int32_t *start, const int32_t *list,
-                                                            const int *list_n, float4 *pos, int32_t *perm) {
+                                                            const int32_t *start, const int2 *list, const int *list_n,
+                                                            float4 *pos, int32_t *perm, int32_t *tgt) {
     __shared__ int hist[8][64], run[8][64];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int nwarps_total = gridDim.x * (blockDim.x >> 5);
     const int nl = *list_n;
     const float s = 1.0f / FIX;
     for (int li = blockIdx.x * (blockDim.x >> 5) + w; li < nl; li += nwarps_total) {
-        const int c = list[li];
+        const int c = list[li].x;
+        const unsigned place = (unsigned)list[li].y;
         const int st = start[c], cnt = count[c];
+        for (int j = lane; j < cnt; j += 32) tgt[place + j] = st + j;
         hist[w][lane] = 0;
         hist[w][lane + 32] = 0;
         __syncwarp();
@@ -248,75 +340,66 @@ struct Sum3 {
     }
 };
 
-// Far-pair factor R_PP(r)/r for b_pp <= r < b_cut (Eq. PP), IOS-cell units,
-// branch-free.  Where r >= b_pp the first term of R_PP is 1/r^2 and the
-// difference is written as m(u)/r^2 with u = r/b_cut: for u >= 1/2 the
-// outer-shell branch of Eq. (refforce) gives r^2 (1/r^2 - R) =
-// v^5 (192/5 - 416/5 v + 2048/35 v^2 - 64/5 v^3), v = 1 - u (an exact
-// polynomial shift, free of cancellation near the cutoff); below u = 1/2 the
-// inner branch gives 1 - 64/5 u^3 + 256/5 u^5 - 32 u^6 - 1536/35 u^7 + 192/5 u^8.
-// Pairs closer than b_pp (and r = 0) get 0 here; close_pair() handles them.
-__device__ __forceinline__ float far_pair(float r2, float inv_bcut, float bpp2) {
-    const float rinv = rsqrtf(r2);
-    const float u = r2 * rinv * inv_bcut;
-    const float v = 1.0f - u;
-    const float v2 = v * v;
-    const float m_out = v2 * v2 * v * (192.0f / 5.0f + v * (-416.0f / 5.0f + v * (2048.0f / 35.0f - 64.0f / 5.0f * v)));
-    const float u2 = u * u;
-    const float m_in = 1.0f + u2 * u * (-64.0f / 5.0f + u2 * (256.0f / 5.0f + u * (-32.0f + u * (-1536.0f / 35.0f + 192.0f / 5.0f * u))));
-    const float g = (u >= 0.5f ? m_out : m_in) * (rinv * rinv * rinv);
-    return r2 >= bpp2 ? g : 0.0f;
-}
+// Sources of a warp whose targets lie in cells [xa, xb] x [ya, yb] x [za, zb] of
+// one pencil: for each row of the block one cell larger on every side, the
+// cells xa-1 .. xb+1 as a main range and, at the box's faces, the wrapped cell
+// on the left and on the right, flattened into one stream of the non-empty
+// ranges.  Positions p from begin[s] on are slots p + seg[s].x; a source's
+// coordinates in the warp's frame (cell (xa, ya - 1, za - 1) at 0) are (cell id
+// - seg[s].y) + off_x, row_y + off_y, row_z + off_z with the row's offsets as
+// floats in seg[s].z and .w: exact in FP32 for blocks of up to 128 cells.
+constexpr int PP_ROWS = (PEN_Y + 2) * (PEN_Z + 2);
+constexpr int PP_SEGS = 3 * PP_ROWS;
 
-// R_PP(r)/r for 0 < r < b_pp: both terms of Eq. PP are softened.
-__device__ __forceinline__ float close_pair(float r2, float inv_bpp, float inv_bcut) {
-    const float rinv = rsqrtf(r2);
-    const float r = r2 * rinv;
-    return (ref_force_scaled(r * inv_bpp) * inv_bpp * inv_bpp - ref_force_scaled(r * inv_bcut) * inv_bcut * inv_bcut) *
-           rinv;
-}
+// A warp is on the shared stream when it spans at most wmax + 1 cells along x
+// (PPParams.wmax, the context's pp_wmax); the few wider ones (fewer than 32
+// particles in that many slabs) walk each lane's own 27 cells.
 
-// Sources of a warp whose 32 targets lie in one row of cells, x in [xa, xb]:
-// for each of the 9 (dz, dy) rows, the cells xa-1 .. xb+1 as a main range and
-// at most one wrapped cell, flattened into one stream.  Stream position p of
-// segment s is particle beg[s] + p - cum[s]; its x coordinate in the warp's
-// frame (cell xa at 0) is (cell id - adj[s]) + off_x.
-constexpr int PP_SEGS = 18;
-struct WarpSegs {
-    int beg[PP_SEGS];
-    int adj[PP_SEGS];
-    int cum[PP_SEGS + 2];
+struct PPBlock {
+    int xa, xb, ya, yb, za, zb;
 };
 
-// The widest warp (cells beyond the first) that takes the shared-stream path
-// is a runtime parameter (PPParams.wmax, the context's pp_wmax, 16 unless an
-// ensemble's autotuner chose another): its lanes test (w + 3) / 3 times their
-// own candidates, still cheaper than the per-lane walk up to about w = 16 over
-// the 256^3 run (at full occupancy w = 8, 12, 16 and 24 lie within 2 % of each
-// other).
+// Staged sources by component, so that a 16-byte load brings two packed pairs.
+template <int N>
+struct Soa {
+    float x[N], y[N], z[N];
+    __device__ __forceinline__ void put(int i, float4 q) {
+        x[i] = q.x;
+        y[i] = q.y;
+        z[i] = q.z;
+    }
+};
 
-struct PPWarpShared {
-    struct {
-        float4 buf[64];   // staged sources of the union path
-        WarpSegs seg;
-        float box[8];     // the warp's target bounding box (lo x, y, z, hi x, y, z) and largest squared range
+constexpr int OUTER_N = 64;             // sources evaluated at a time, no pair of them closer than half the range
+constexpr int MIXED_N = 32;             // sources evaluated at a time, any distance
+constexpr int SPARSE_N = 128;           // sources tested before the pairs found are evaluated
+constexpr int QUEUE_N = 32;             // pairs a lane can hold
+
+struct alignas(16) PPWarpShared {
+    union {
+        struct {
+            Soa<OUTER_N + 32> outer;
+            Soa<MIXED_N + 32> mixed;
+        } d;
+        struct {
+            Soa<SPARSE_N + 4> src;
+            unsigned char queue[QUEUE_N][32];
+        } s;
+        float4 buf[64];
     } u;
+    int4 seg[PP_SEGS];
+    int begin[PP_SEGS];
+    // bounding box of the warp's targets: (lo x, y, z, largest squared range), (hi x, y, z, where the outer half begins)
+    float4 box[2];
 };
 
-struct PPShared {
-    PPWarpShared w[PP_WARPS_CTA];
-};
-
-// Stage stream position p (far-away point past the end).  s: the lane's
-// running segment index (positions a lane stages only increase).
-__device__ __forceinline__ float4 stage_source(const PPParams &P, const WarpSegs &W, int p, int &s) {
-    if (p >= W.cum[PP_SEGS]) return make_float4(1.0e18f, 1.0e18f, 1.0e18f, 0.0f);
-    while (p >= W.cum[s + 1]) ++s;
-    const float4 q = __ldg(&P.pos[W.beg[s] + (p - W.cum[s])]);
-    const int row = s >> 1;   // (dz + 1) * 3 + (dy + 1)
-    return make_float4((float)(__float_as_int(q.w) - W.adj[s]) + q.x, q.y + (float)(row % 3), q.z + (float)(row / 3),
+__device__ __forceinline__ float4 frame_position(float4 q, int4 g) {
+    return make_float4((float)(__float_as_int(q.w) - g.y) + q.x, q.y + __int_as_float(g.z), q.z + __int_as_float(g.w),
                        0.0f);
 }
+
+// padding sources: out of range of every target, and no overflow in the pair formula
+constexpr float PP_FAR = 4096.0f;
 
 // Candidate test of 32 staged sources: bit (31 - k) set where source k is
 // closer than b_cut (sign of r^2 - b_cut^2, shifted in).
@@ -332,155 +415,462 @@ __device__ __forceinline__ unsigned test32(const float4 *S, float mx, float my, 
     return m;
 }
 
+__device__ __forceinline__ void prefetch_l1(const void *p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
+
 // Build the warp's segment table; returns the stream length.
-__device__ int build_segments(const PPParams &P, WarpSegs &W, int c0, int xa, int xb) {
+__device__ __forceinline__ int build_segments(const PPParams &P, int4 *seg, int *begin, const PPBlock &B, int &nseg) {
     const int lane = threadIdx.x & 31;
     const int n = P.n_ios;
-    const int cz = c0 / (n * n), cy = (c0 / n) % n;
-    // segment table: lane 2*row + which
-    int len = 0;
-    if (lane < PP_SEGS) {
-        const int row = lane >> 1, which = lane & 1;
-        const int dz = row / 3 - 1, dy = row % 3 - 1;
-        const int rb = (wrap(cz + dz, n) * n + wrap(cy + dy, n)) * n;
-        int beg = 0, adj = rb + xa;
-        if (which == 0) {
-            const int lo = xa > 0 ? xa - 1 : 0, hi = xb < n - 1 ? xb + 1 : n - 1;
-            beg = __ldg(&P.start[rb + lo]);
-            len = __ldg(&P.start[rb + hi]) + __ldg(&P.count[rb + hi]) - beg;
-        } else if (xa == 0) {
-            beg = __ldg(&P.start[rb + n - 1]);
-            len = __ldg(&P.count[rb + n - 1]);
-            adj += n;
-        } else if (xb == n - 1) {
-            beg = __ldg(&P.start[rb]);
-            len = __ldg(&P.count[rb]);
-            adj -= n;
-        }
-        W.beg[lane] = beg;
-        W.adj[lane] = adj;
-    }
-    int incl = len;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-    }
-    if (lane < PP_SEGS) W.cum[lane + 1] = incl;
-    if (lane == 0) W.cum[0] = 0;
-    if (lane == PP_SEGS) W.cum[PP_SEGS + 1] = 0x7fffffff;
-    __syncwarp();
-    return W.cum[PP_SEGS];
-}
-
-// Test of 32 staged sources by every lane and evaluation of the set bits (the
-// pairs in range), far pairs first, the rare pairs closer than b_pp after.
-__device__ __forceinline__ void eval32(const float4 *S, float mx, float my, float mz, float bcut2, float ibc,
-                                       float bpp2, float ibp, float coef, bool has, Sum3 &a, unsigned &pairs) {
-    unsigned m = has ? test32(S, mx, my, mz, bcut2) : 0u;
-    pairs += __popc(m);
-    float px = 0.f, py = 0.f, pz = 0.f;
-    unsigned cm = 0u;   // pairs closer than b_pp
-    while (m) {
-        const int k = __clz(m);
-        const unsigned bit = 0x80000000u >> k;
-        m ^= bit;
-        const float4 q = S[k];
-        const float rx = q.x - mx, ry = q.y - my, rz = q.z - mz;
-        const float r2 = rx * rx + ry * ry + rz * rz;
-        const float g = far_pair(r2, ibc, bpp2);
-        if (r2 < bpp2) cm |= bit;
-        px = fmaf(g, rx, px);
-        py = fmaf(g, ry, py);
-        pz = fmaf(g, rz, pz);
-    }
-    if (__any_sync(0xffffffffu, cm != 0u)) {
-        while (cm) {
-            const int k = __clz(cm);
-            cm ^= 0x80000000u >> k;
-            const float4 q = S[k];
-            const float rx = q.x - mx, ry = q.y - my, rz = q.z - mz;
-            const float r2 = rx * rx + ry * ry + rz * rz;
-            if (r2 > 0.0f) {
-                const float g = close_pair(r2, ibp, ibc);
-                px = fmaf(g, rx, px);
-                py = fmaf(g, ry, py);
-                pz = fmaf(g, rz, pz);
+    const int ny = B.yb - B.ya + 3, rows = ny * (B.zb - B.za + 3);
+    const int rz = lane / ny, ry = lane - rz * ny;
+    const int rb = lane < rows ? (wrap(B.za - 1 + rz, n) * n + wrap(B.ya - 1 + ry, n)) * n : 0;
+    int run = 0;
+    nseg = 0;
+#pragma unroll 1
+    for (int g = 0; g < 3; ++g) {
+        if ((g == 1 && B.xa > 0) || (g == 2 && B.xb < n - 1)) continue;
+        int beg = 0, len = 0, adj = rb + B.xa;
+        if (lane < rows) {
+            if (g == 0) {
+                const int lo = max(B.xa - 1, 0), hi = min(B.xb + 1, n - 1);
+                beg = __ldg(&P.start[rb + lo]);
+                len = __ldg(&P.start[rb + hi]) + __ldg(&P.count[rb + hi]) - beg;
             } else {
-                --pairs;   // the target itself, or a coincident particle: no pair force
+                const int c = g == 1 ? rb + n - 1 : rb;
+                beg = __ldg(&P.start[c]);
+                len = __ldg(&P.count[c]);
+                adj += g == 1 ? n : -n;
             }
         }
-    }
-    a.add_block(coef * px, coef * py, coef * pz);
-}
-
-// Warps inside one row of cells share one source stream (the cells xa-1 ..
-// xb+1 of the 9 rows around it).  Each source is staged once by one lane and
-// kept only if it lies within the warp's largest PP range of the bounding box
-// of the warp's targets (no pair of it can be in range otherwise); the kept
-// sources are packed in shared memory and every lane tests and evaluates them
-// 32 at a time.  The target itself is in the stream and drops out at r = 0.
-__device__ void union_path(const PPParams &P, const WarpSegs &W, float4 *S, float *box, int64_t i, bool has, int c0,
-                           int xa, float4 me, float bcut2, float ibc, Sum3 &a, unsigned &pairs, unsigned &cands) {
-    (void)i;
-    const int lane = threadIdx.x & 31;
-    const int n = P.n_ios;
-    const int total = W.cum[PP_SEGS];
-    const int cx = (has ? __float_as_int(me.w) : c0) % n;
-    const float mx = (float)(cx - xa) + me.x, my = me.y + 1.0f, mz = me.z + 1.0f;
-    const float bpp2 = P.bpp2, ibp = P.inv_bpp;
-    // bounding box of the warp's targets and the largest squared range
-    float lx = has ? mx : 1e30f, ly = has ? my : 1e30f, lz = has ? mz : 1e30f;
-    float hx = has ? mx : -1e30f, hy = has ? my : -1e30f, hz = has ? mz : -1e30f;
-    float reach2 = has ? bcut2 : 0.0f;
+        if (len > 0) {   // its first sources on their way before the stream comes to them
+            prefetch_l1(&P.pos[beg]);
+            if (len > 1) prefetch_l1(&P.pos[beg + min(len, 16) - 1]);
+        }
+        int incl = len;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        lx = fminf(lx, __shfl_xor_sync(0xffffffffu, lx, o));
-        ly = fminf(ly, __shfl_xor_sync(0xffffffffu, ly, o));
-        lz = fminf(lz, __shfl_xor_sync(0xffffffffu, lz, o));
-        hx = fmaxf(hx, __shfl_xor_sync(0xffffffffu, hx, o));
-        hy = fmaxf(hy, __shfl_xor_sync(0xffffffffu, hy, o));
-        hz = fmaxf(hz, __shfl_xor_sync(0xffffffffu, hz, o));
-        reach2 = fmaxf(reach2, __shfl_xor_sync(0xffffffffu, reach2, o));
-    }
-    // kept in the warp's shared memory: fewer live registers in the loop
-    if (lane == 0) {
-        box[0] = lx; box[1] = ly; box[2] = lz;
-        box[3] = hx; box[4] = hy; box[5] = hz;
-        box[6] = reach2;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        const unsigned full = __ballot_sync(0xffffffffu, len > 0);
+        const int at = run + incl - len;
+        if (len > 0) {
+            const int k = nseg + __popc(full & ((1u << lane) - 1u));
+            begin[k] = at;
+            seg[k] = make_int4(beg - at, adj, __float_as_int((float)ry), __float_as_int((float)rz));
+        }
+        run += __shfl_sync(0xffffffffu, incl, 31);
+        nseg += __popc(full);
     }
     __syncwarp();
-    int fill = 0, sa = 0;
-    for (int b0 = 0; b0 < total; b0 += 32) {
-        const float4 q = stage_source(P, W, b0 + lane, sa);
-        const float dx = fmaxf(fmaxf(box[0] - q.x, q.x - box[3]), 0.0f);
-        const float dy = fmaxf(fmaxf(box[1] - q.y, q.y - box[4]), 0.0f);
-        const float dz = fmaxf(fmaxf(box[2] - q.z, q.z - box[5]), 0.0f);
-        const bool keep = dx * dx + dy * dy + dz * dz < box[6];
-        const unsigned km = __ballot_sync(0xffffffffu, keep);
-        if (keep) S[fill + __popc(km & ((1u << lane) - 1u))] = q;
-        fill += __popc(km);
-        __syncwarp();
-        if (fill >= 32) {
-            if (has) cands += 32u;
-            eval32(S, mx, my, mz, bcut2, ibc, bpp2, ibp, P.coef, has, a, pairs);
-            __syncwarp();
-            const float4 t = S[32 + lane];
-            if (32 + lane < fill) S[lane] = t;
-            fill -= 32;
-            __syncwarp();
+    return run;
+}
+
+// ------------------------------------------------------------ pair factor
+// R_PP(r)/r of a pair with b_pp <= r < b_cut (Eq. PP) in units of 1/b_cut^3, as
+// a function of u^2 = (r / b_cut)^2.  Where r >= b_pp the first term of R_PP is
+// 1/r^2 and R_PP(r)/r = m(u)/u^3: the outer shell of Eq. (refforce) gives
+//   u >= 1/2: m = (1-u)^5 q(u), q = 32/35 + 32/7 u + 704/35 u^2 + 64/5 u^3
+//             (an exact polynomial shift, free of cancellation near the cutoff),
+//             so m/u^3 = t^5 u^2 q(u) with t = 1/u - 1, zero beyond the cutoff
+//             where t is clamped at 0;
+//   u < 1/2:  m = 1 - 64/5 u^3 + 256/5 u^5 - 32 u^6 - 1536/35 u^7 + 192/5 u^8.
+// u^2 is 0 or at least 2^-32, so the flush of denormals never acts.
+__device__ __forceinline__ float rsqrt_ftz(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+constexpr float Q0 = 32.0f / 35.0f, Q1 = 32.0f / 7.0f, Q2 = 704.0f / 35.0f, Q3 = 64.0f / 5.0f;
+constexpr float I0 = -64.0f / 5.0f, I2 = 256.0f / 5.0f, I3 = -32.0f, I4 = -1536.0f / 35.0f, I5 = 192.0f / 5.0f;
+
+// R(r, b)/r of Eq. (refforce) in units of 1/b^3 at x = r/b <= 1.
+__device__ __forceinline__ float soft_factor(float x2) {
+    const float xinv = rsqrt_ftz(x2);
+    const float x = x2 * xinv;
+    if (x2 < 0.25f) return -fmaf(fmaf(fmaf(fmaf(I5, x, I4), x, I3), x, I2), x2, I0);
+    const float t = __saturatef(xinv - 1.0f);
+    const float a = t * t * x;
+    return fmaf(-(a * a * t), fmaf(fmaf(fmaf(Q3, x, Q2), x, Q1), x, Q0), xinv * xinv * xinv);
+}
+
+// R_PP(r)/r for 0 < r < b_pp, same units as the far factor: both terms of Eq.
+// PP are softened.  ratio2 = (b_cut/b_pp)^2.
+__device__ __forceinline__ float close_factor(float u2, float ratio2) {
+    return fmaf(ratio2 * sqrtf(ratio2), soft_factor(u2 * ratio2), -soft_factor(u2));
+}
+
+// Two FP32 values in one 64-bit register pair (packed FP32 arithmetic: the rate
+// of the FMA pipe is that of two scalar instructions, the issue slots are
+// those of one).
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pack(float a, float b) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack(f2 v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+    f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+    f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f2 twice(float a) { return pack(a, a); }
+
+// A target as the pair loops see it.
+struct PPLane {
+    float mx, my, mz;        // position in the warp's frame
+    float bcut2, ib2;        // range^2, 1/range^2 [IOS cells]
+    float coef;              // of the sums: V_p/(4 pi s^2) / range^3
+    bool has;
+};
+
+// The far factor of two pairs (OUTER: both at u >= 1/2 or out of range).
+template <bool OUTER>
+__device__ __forceinline__ f2 far_factor2(f2 u2) {
+    float ua, ub;
+    unpack(u2, ua, ub);
+    const float ia = rsqrt_ftz(ua), ib = rsqrt_ftz(ub);
+    const f2 uinv = pack(ia, ib), u = mul2(u2, uinv);
+    const f2 t = pack(__saturatef(ia - 1.0f), __saturatef(ib - 1.0f));   // at most 1 where it is used
+    const f2 c = mul2(mul2(t, t), u);
+    const f2 q = fma2(fma2(fma2(twice(Q3), u, twice(Q2)), u, twice(Q1)), u, twice(Q0));
+    const f2 g = mul2(mul2(mul2(c, c), t), q);
+    if constexpr (OUTER) return g;
+    const f2 m = fma2(fma2(fma2(fma2(fma2(twice(I5), u, twice(I4)), u, twice(I3)), u, twice(I2)), u2, twice(I0)),
+                      mul2(u2, u), twice(1.0f));
+    const f2 gi = mul2(m, mul2(mul2(uinv, uinv), uinv));
+    float oa, ob, na, nb;
+    unpack(g, oa, ob);
+    unpack(gi, na, nb);
+    return pack(ua < 0.25f ? na : oa, ub < 0.25f ? nb : ob);
+}
+
+// Bounding box of the warp's targets and the largest squared range, kept in the
+// warp's shared memory (fewer live registers in the stream loops); returns the
+// expected candidates per pair.  Frame coordinates are not negative, so their
+// bit patterns order like the values (padding lanes repeat lane 0's target).
+__device__ __forceinline__ float warp_box(float4 *box, float mx, float my, float mz, float bcut2, float bpp2) {
+    const unsigned all = 0xffffffffu;
+    const float lx = __uint_as_float(__reduce_min_sync(all, __float_as_uint(mx)));
+    const float ly = __uint_as_float(__reduce_min_sync(all, __float_as_uint(my)));
+    const float lz = __uint_as_float(__reduce_min_sync(all, __float_as_uint(mz)));
+    const float hx = __uint_as_float(__reduce_max_sync(all, __float_as_uint(mx)));
+    const float hy = __uint_as_float(__reduce_max_sync(all, __float_as_uint(my)));
+    const float hz = __uint_as_float(__reduce_max_sync(all, __float_as_uint(mz)));
+    const float reach2 = __uint_as_float(__reduce_max_sync(all, __float_as_uint(bcut2)));
+    if ((threadIdx.x & 31) == 0) {
+        box[0] = make_float4(lx, ly, lz, reach2);
+        // beyond it every pair is in the outer half of its range and no close one
+        box[1] = make_float4(hx, hy, hz, 1.00001f * fmaxf(0.25f * reach2, bpp2));
+    }
+    __syncwarp();
+    const float ex = hx - lx, ey = hy - ly, ez = hz - lz, r = sqrtf(reach2);
+    // volume within reach of the box over that of one sphere: candidates per pair at even density
+    const float area = fmaf(ex, ey, fmaf(ey, ez, __fmul_rn(ez, ex)));
+    const float beyond = fmaf(ex * ey, ez, fmaf(2.0f * r, area, __fmul_rn(3.1416f * reach2, ex + ey + ez)));
+    return __fadd_rn(beyond / (4.1888f * reach2 * r), 1.0f);
+}
+
+// Squared distance of a source from the box [lo, hi] of the warp's targets.
+__device__ __forceinline__ float box_distance2(float4 lo, float4 hi, float4 q) {
+    const float dx = fmaxf(fmaxf(lo.x - q.x, q.x - hi.x), 0.0f);
+    const float dy = fmaxf(fmaxf(lo.y - q.y, q.y - hi.y), 0.0f);
+    const float dz = fmaxf(fmaxf(lo.z - q.z, q.z - hi.z), 0.0f);
+    return fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+}
+
+// The sources of a warp's stream, 32 positions at a time, the next ones loaded
+// while the current ones are worked on.  The segment of position b0 + lane: the
+// segments that begin inside the window [b0, b0 + 32) as one bit mask; before:
+// those begun ahead of it.
+struct PPStream {
+    int nseg, total, before, mine;   // mine: where segment `lane` begins
+    int4 g;
+    float4 raw = make_float4(0.f, 0.f, 0.f, 0.f);
+    int slot;
+    __device__ __forceinline__ void init(const PPParams &P, const PPWarpShared &W) {
+        const int lane = threadIdx.x & 31;
+        before = 0;
+        mine = lane < nseg ? W.begin[lane] : 0x7fffffff;
+        load(P, W, 0);   // the target itself is in the stream: never empty
+    }
+    __device__ __forceinline__ void load(const PPParams &P, const PPWarpShared &W, int b0) {
+        const int lane = threadIdx.x & 31;
+        unsigned d = (unsigned)(mine - b0), bit = d < 32u ? 1u << d : 0u;
+        for (int k = lane + 32; k < nseg; k += 32) {   // warps at the box's x faces only
+            d = (unsigned)(W.begin[k] - b0);
+            if (d < 32u) bit |= 1u << d;
+        }
+        const unsigned mask = __reduce_or_sync(0xffffffffu, bit);
+        g = W.seg[before + __popc(mask & (0xffffffffu >> (31 - lane))) - 1];
+        before += __popc(mask);
+        slot = b0 + lane + g.x;
+        if (b0 + lane < total) raw = __ldg(&P.pos[slot]);
+    }
+    // the source at b0 + lane in the warp's frame (of no meaning past the end)
+    __device__ __forceinline__ float4 next(const PPParams &P, const PPWarpShared &W, int b0) {
+        const float4 q = frame_position(raw, g);
+        if (b0 + 32 < total) load(P, W, b0 + 32);
+        return q;
+    }
+};
+
+// Pairs of every lane's target with n staged sources (n a multiple of 4), all
+// of them, no test.  OUTER: no pair closer than half the range.  Out-of-range
+// pairs get 0 from the clamped t; pairs closer than b_pp (the target itself
+// among them) get 0 here and their bit in close (source k of 32: bit 31 - k).
+template <bool OUTER, bool COUNT, int N>
+__device__ __forceinline__ void eval_all(const Soa<N> &S, int n, const PPLane &L, float bpp2, f2 sum[3], unsigned &pairs,
+                                         unsigned &close) {
+    const f2 nx = twice(-L.mx), ny = twice(-L.my), nz = twice(-L.mz), ib2 = twice(L.ib2);
+    f2 px = 0ull, py = 0ull, pz = 0ull;
+#pragma unroll 1
+    for (int k = 0; k < n; k += 4) {
+        const ulonglong2 X = *reinterpret_cast<const ulonglong2 *>(&S.x[k]);
+        const ulonglong2 Y = *reinterpret_cast<const ulonglong2 *>(&S.y[k]);
+        const ulonglong2 Z = *reinterpret_cast<const ulonglong2 *>(&S.z[k]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const f2 rx = add2(h ? X.y : X.x, nx), ry = add2(h ? Y.y : Y.x, ny), rz = add2(h ? Z.y : Z.x, nz);
+            const f2 r2 = fma2(rz, rz, fma2(ry, ry, mul2(rx, rx)));
+            f2 g = far_factor2<OUTER>(mul2(r2, ib2));
+            if constexpr (!OUTER || COUNT) {
+                float ra, rb;
+                unpack(r2, ra, rb);
+                if constexpr (!OUTER) {
+                    float ga, gb;
+                    unpack(g, ga, gb);
+                    const float ca = ra - bpp2, cb = rb - bpp2;
+                    g = pack(ca < 0.0f ? 0.0f : ga, cb < 0.0f ? 0.0f : gb);
+                    close = __funnelshift_l(__float_as_uint(ca), close, 1);
+                    close = __funnelshift_l(__float_as_uint(cb), close, 1);
+                }
+                if constexpr (COUNT)
+                    if (L.has) pairs += (ra > 0.0f && ra < L.bcut2) + (rb > 0.0f && rb < L.bcut2);
+            }
+            px = fma2(g, rx, px);
+            py = fma2(g, ry, py);
+            pz = fma2(g, rz, pz);
         }
     }
-    if (fill > 0) {
-        if (lane >= fill) S[lane] = make_float4(1.0e18f, 1.0e18f, 1.0e18f, 0.0f);
-        __syncwarp();
-        if (has) cands += (unsigned)fill;
-        eval32(S, mx, my, mz, bcut2, ibc, bpp2, ibp, P.coef, has, a, pairs);
-    }
-    __syncwarp();
+    sum[0] = px;
+    sum[1] = py;
+    sum[2] = pz;
 }
 
-// Warps whose targets span several rows or a wide x range (sparse regions):
+__device__ __forceinline__ void add_pairs(Sum3 &a, const PPLane &L, f2 x, f2 y, f2 z) {
+    float x0, x1, y0, y1, z0, z1;
+    unpack(x, x0, x1);
+    unpack(y, y0, y1);
+    unpack(z, z0, z1);
+    a.add_block(__fmul_rn(L.coef, x0 + x1), __fmul_rn(L.coef, y0 + y1), __fmul_rn(L.coef, z0 + z1));
+}
+
+// A warp's targets share one source stream.  Each source is staged once by one
+// lane and kept only if it lies within the warp's largest PP range of the
+// bounding box of the warp's targets (no pair of it can be in range otherwise).
+//
+// Compact warps (targets within about a cell): most kept sources are in range
+// of most targets, and evaluating every pair costs less than finding those in
+// range (20 FMA-pipe cycles a pair without a test, no idle lanes, against 6 a
+// test and about 80 a pair found).  Sources at least half a range from the box
+// are evaluated without the inner branch of the pair factor.
+template <bool COUNT>
+__device__ __forceinline__ void stream_compact(const PPParams &P, PPWarpShared &W, PPStream &T, const PPLane &L, Sum3 &a,
+                                               unsigned &pairs, unsigned &cands) {
+    const int lane = threadIdx.x & 31;
+    auto &O = W.u.d.outer;
+    auto &M = W.u.d.mixed;
+    int fo = 0, fm = 0;
+#pragma unroll 1
+    for (int b0 = 0; b0 < T.total || fo || fm; b0 += 32) {
+        if (b0 < T.total) {
+            const float4 q = T.next(P, W, b0);
+            const float4 lo = W.box[0], hi = W.box[1];
+            const float d2 = box_distance2(lo, hi, q);
+            const bool keep = b0 + lane < T.total && d2 < lo.w, far = d2 > hi.w;
+            const unsigned ko = __ballot_sync(0xffffffffu, keep && far), km = __ballot_sync(0xffffffffu, keep && !far);
+            const unsigned lt = (1u << lane) - 1u;
+            if (keep) {
+                if (far) O.put(fo + __popc(ko & lt), q);
+                else M.put(fm + __popc(km & lt), q);
+            }
+            fo += __popc(ko);
+            fm += __popc(km);
+            if (COUNT && L.has) cands += __popc(ko | km);
+        }
+        const bool last = b0 + 32 >= T.total;   // from here on only what is staged
+        f2 sum[3];
+        if (fo >= OUTER_N || (last && fo)) {
+            const int n = min(OUTER_N, (fo + 3) & ~3);
+            if (lane < n - fo) O.put(fo + lane, make_float4(PP_FAR, PP_FAR, PP_FAR, 0.f));
+            __syncwarp();
+            unsigned none = 0u;
+            eval_all<true, COUNT>(O, n, L, 0.0f, sum, pairs, none);
+            add_pairs(a, L, sum[0], sum[1], sum[2]);
+            __syncwarp();
+            fo = max(0, fo - OUTER_N);
+            if (lane < fo) O.put(lane, make_float4(O.x[OUTER_N + lane], O.y[OUTER_N + lane], O.z[OUTER_N + lane], 0.f));
+        }
+        if (fm >= MIXED_N || (last && fm)) {
+            const int n = min(MIXED_N, (fm + 3) & ~3);
+            if (lane < n - fm) M.put(fm + lane, make_float4(PP_FAR, PP_FAR, PP_FAR, 0.f));
+            __syncwarp();
+            unsigned close = 0u;
+            eval_all<false, COUNT>(M, n, L, P.bpp2, sum, pairs, close);
+            close <<= 32 - n;
+            if (__any_sync(0xffffffffu, close != 0u)) {
+                float px = 0.f, py = 0.f, pz = 0.f;
+#pragma unroll 1
+                while (close) {
+                    const int k = __clz(close);
+                    close ^= 0x80000000u >> k;
+                    const float rx = M.x[k] - L.mx, ry = M.y[k] - L.my, rz = M.z[k] - L.mz;
+                    const float r2 = fmaf(rz, rz, fmaf(ry, ry, rx * rx));
+                    if (r2 > 0.0f) {   // not the target itself, nor a coincident particle
+                        const float g = close_factor(r2 * L.ib2, P.ratio2 * L.bcut2);
+                        px = fmaf(g, rx, px);
+                        py = fmaf(g, ry, py);
+                        pz = fmaf(g, rz, pz);
+                    }
+                }
+                a.add_block(__fmul_rn(L.coef, px), __fmul_rn(L.coef, py), __fmul_rn(L.coef, pz));
+            }
+            add_pairs(a, L, sum[0], sum[1], sum[2]);
+            __syncwarp();
+            fm = max(0, fm - MIXED_N);
+            if (lane < fm) M.put(lane, make_float4(M.x[MIXED_N + lane], M.y[MIXED_N + lane], M.z[MIXED_N + lane], 0.f));
+        }
+        __syncwarp();
+    }
+}
+
+// Other warps (few of the sources are in range of any one target): every lane
+// tests all kept sources, 32 to a mask (sign of r^2 - b_cut^2 shifted in, packed
+// arithmetic: 6 FMA-pipe cycles a test), notes the sources in range in its own
+// queue, and the queues are evaluated together, two pairs at a time, once up to
+// SPARSE_N sources are through: the lanes then idle by the spread of their
+// totals, not of every mask (about 7 pair evaluations a warp instead of 12 at
+// one particle per cell).
+__device__ __forceinline__ void eval_queue(const PPParams &P, const PPWarpShared &W, int held, const PPLane &L, Sum3 &a,
+                                           unsigned &pairs) {
+    const int lane = threadIdx.x & 31;
+    const auto &S = W.u.s.src;
+    const f2 nx = twice(-L.mx), ny = twice(-L.my), nz = twice(-L.mz), ib2 = twice(L.ib2);
+    f2 px = 0ull, py = 0ull, pz = 0ull;
+#pragma unroll 1
+    for (int i = 0; i < held; i += 2) {
+        const int ka = W.u.s.queue[i][lane];
+        const int kb = i + 1 < held ? W.u.s.queue[i + 1][lane] : SPARSE_N;   // slot SPARSE_N: PP_FAR
+        const f2 rx = add2(pack(S.x[ka], S.x[kb]), nx), ry = add2(pack(S.y[ka], S.y[kb]), ny),
+                 rz = add2(pack(S.z[ka], S.z[kb]), nz);
+        const f2 r2 = fma2(rz, rz, fma2(ry, ry, mul2(rx, rx)));
+        const f2 u2 = mul2(r2, ib2);
+        f2 g = far_factor2<false>(u2);
+        float ra, rb;
+        unpack(r2, ra, rb);
+        if (__builtin_expect(fminf(ra, rb) < P.bpp2, 0)) {   // rare: a close pair; the target itself gets 0
+            float ga, gb, ua, ub;
+            unpack(g, ga, gb);
+            unpack(u2, ua, ub);
+#pragma unroll 1
+            for (int e = 0; e < 2; ++e) {
+                const float r = e ? rb : ra;
+                if (r < P.bpp2) {
+                    const float c = r > 0.0f ? close_factor(e ? ub : ua, P.ratio2 * L.bcut2) : 0.0f;
+                    pairs -= r == 0.0f;
+                    if (e) gb = c;
+                    else ga = c;
+                }
+            }
+            g = pack(ga, gb);
+        }
+        px = fma2(g, rx, px);
+        py = fma2(g, ry, py);
+        pz = fma2(g, rz, pz);
+    }
+    if (held) add_pairs(a, L, px, py, pz);
+}
+
+__device__ __forceinline__ void stream_sparse(const PPParams &P, PPWarpShared &W, PPStream &T, const PPLane &L, Sum3 &a,
+                                              unsigned &pairs, unsigned &cands) {
+    const int lane = threadIdx.x & 31;
+    auto &S = W.u.s.src;
+    int fill = 0;
+    if (lane == 0) S.put(SPARSE_N, make_float4(PP_FAR, PP_FAR, PP_FAR, 0.f));
+#pragma unroll 1
+    for (int b0 = 0; b0 < T.total; b0 += 32) {
+        const float4 q = T.next(P, W, b0);
+        const float4 lo = W.box[0], hi = W.box[1];
+        const bool keep = b0 + lane < T.total && box_distance2(lo, hi, q) < lo.w;
+        const unsigned km = __ballot_sync(0xffffffffu, keep);
+        if (keep) S.put(fill + __popc(km & ((1u << lane) - 1u)), q);
+        fill += __popc(km);
+        if (fill <= SPARSE_N - 32 && b0 + 32 < T.total) continue;
+        // pad to whole groups of 8, test, queue
+        const int n8 = (fill + 7) & ~7;
+        if (lane < n8 - fill) S.put(fill + lane, make_float4(PP_FAR, PP_FAR, PP_FAR, 0.f));
+        __syncwarp();
+        if (L.has) cands += (unsigned)fill;
+        const f2 nx = twice(-L.mx), ny = twice(-L.my), nz = twice(-L.mz), nb = twice(L.has ? -L.bcut2 : 1.0f);
+        int held = 0;
+#pragma unroll 1
+        for (int w0 = 0;; w0 += 32) {
+            unsigned m = 0u;
+            const int kn = min(32, n8 - w0);
+#pragma unroll 1
+            for (int k = 0; k < kn; k += 8) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const ulonglong2 X = *reinterpret_cast<const ulonglong2 *>(&S.x[w0 + k + 4 * h]);
+                    const ulonglong2 Y = *reinterpret_cast<const ulonglong2 *>(&S.y[w0 + k + 4 * h]);
+                    const ulonglong2 Z = *reinterpret_cast<const ulonglong2 *>(&S.z[w0 + k + 4 * h]);
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const f2 rx = add2(e ? X.y : X.x, nx), ry = add2(e ? Y.y : Y.x, ny), rz = add2(e ? Z.y : Z.x, nz);
+                        const f2 d = fma2(rx, rx, fma2(ry, ry, fma2(rz, rz, nb)));
+                        float da, db;
+                        unpack(d, da, db);
+                        m = __funnelshift_l(__float_as_uint(da), m, 1);
+                        m = __funnelshift_l(__float_as_uint(db), m, 1);
+                    }
+                }
+            }
+            const bool done = kn <= 0;   // nothing left to test: the queues' last evaluation
+            if (!done) m <<= 32 - kn;
+            const int more = __popc(m);
+            pairs += more;
+            if (done || __any_sync(0xffffffffu, held + more > QUEUE_N)) {
+                __syncwarp();
+                eval_queue(P, W, held, L, a, pairs);
+                held = 0;
+                if (done) break;
+            }
+#pragma unroll 1
+            while (m) {
+                const int k = __clz(m);
+                m ^= 0x80000000u >> k;
+                W.u.s.queue[held++][lane] = (unsigned char)(w0 + k);
+            }
+        }
+        fill = 0;
+        __syncwarp();
+    }
+}
+
+// Warps whose targets span a wide x range (nearly empty regions):
 // each lane walks its own 27 cells as 9 row ranges and evaluates the pairs in
 // range as it meets them.  Plain nested loops keep the loads pipelined.  (A
 // per-lane queue of the pairs in range, evaluated when full, measured 2x
@@ -488,13 +878,15 @@ __device__ void union_path(const PPParams &P, const WarpSegs &W, float4 *S, floa
 // region fill their queues at different steps and evaluate them one at a
 // time; skipping the rows and end cells beyond the range saved 6 % of the
 // candidates at z = 49 and cost more than that.)
-__device__ void lane_path(const PPParams &P, bool has, int c, float4 me, float bcut2, float ibc, Sum3 &a,
-                          unsigned &pairs, unsigned &cands) {
-    if (!has) return;
+__device__ void lane_path(const PPParams &P, int c, float4 me, const PPLane &L, Sum3 &a, unsigned &pairs,
+                          unsigned &cands) {
+    if (!L.has) return;
     const int n = P.n_ios;
     const int cx = c % n, cy = (c / n) % n, cz = c / (n * n);
-    const float bpp2 = P.bpp2, ibp = P.inv_bpp;
+    const float bpp2 = P.bpp2;
+#pragma unroll 1
     for (int dz = -1; dz <= 1; ++dz)
+#pragma unroll 1
         for (int dy = -1; dy <= 1; ++dy) {
             const int64_t r = ((int64_t)wrap(cz + dz, n) * n + wrap(cy + dy, n)) * n;
             const RowRanges rr(P, r, cx, n);
@@ -502,17 +894,18 @@ __device__ void lane_path(const PPParams &P, bool has, int c, float4 me, float b
             const float fdy = (float)dy, fdz = (float)dz;
             float px = 0.f, py = 0.f, pz = 0.f;
             for (int sgi = 0; sgi < rr.nseg; ++sgi) {
-#pragma unroll 4
+#pragma unroll 1
                 for (int j = rr.beg[sgi]; j < rr.end[sgi]; ++j) {
                     const float4 q = __ldg(&P.pos[j]);
                     const float fdx = (float)(rr.base[sgi] + (j >= rr.b1[sgi]) + (j >= rr.b2[sgi]));
                     const float rx = (fdx + q.x) - me.x;
                     const float ry = (fdy + q.y) - me.y;
                     const float rz = (fdz + q.z) - me.z;
-                    const float r2 = rx * rx + ry * ry + rz * rz;
-                    if (r2 < bcut2 && r2 > 0.0f) {
-                        float g = far_pair(r2, ibc, bpp2);
-                        if (__builtin_expect(r2 < bpp2, 0)) g = close_pair(r2, ibp, ibc);   // rare
+                    const float r2 = fmaf(rz, rz, fmaf(ry, ry, rx * rx));
+                    if (r2 < L.bcut2 && r2 > 0.0f) {
+                        float g, unused;
+                        if (r2 >= bpp2) unpack(far_factor2<false>(twice(r2 * L.ib2)), g, unused);
+                        else g = close_factor(r2 * L.ib2, P.ratio2 * L.bcut2);
                         px = fmaf(g, rx, px);
                         py = fmaf(g, ry, py);
                         pz = fmaf(g, rz, pz);
@@ -520,7 +913,7 @@ __device__ void lane_path(const PPParams &P, bool has, int c, float4 me, float b
                     }
                 }
             }
-            a.add_block(P.coef * px, P.coef * py, P.coef * pz);
+            a.add_block(__fmul_rn(L.coef, px), __fmul_rn(L.coef, py), __fmul_rn(L.coef, pz));
         }
 }
 
@@ -609,7 +1002,8 @@ __device__ void lane_vjp(const PPParams &P, const VjpIO &V, bool has, int c, flo
                     const float rz = (fdz + q.z) - me.z;
                     const float r2 = rx * rx + ry * ry + rz * rz;
                     if (r2 < P.bcut2 && r2 > 0.0f) {
-                        const float4 vj = make_float4(__ldg(&V.v0[j]), __ldg(&V.v1[j]), __ldg(&V.v2[j]), 0.f);
+                        const int pj = __ldg(&P.perm[j]);
+                        const float4 vj = make_float4(__ldg(&V.v0[pj]), __ldg(&V.v1[pj]), __ldg(&V.v2[pj]), 0.f);
                         jacobian_term(rx, ry, rz, r2, vj, vix, viy, viz, P, px, py, pz);
                     }
                 }
@@ -618,152 +1012,195 @@ __device__ void lane_vjp(const PPParams &P, const VjpIO &V, bool has, int c, flo
         }
 }
 
-// The particle index of stream position p (-1 past the end); s as in stage_source.
-__device__ __forceinline__ int stream_index(const WarpSegs &W, int p, int &s) {
-    if (p >= W.cum[PP_SEGS]) return -1;
-    while (p >= W.cum[s + 1]) ++s;
-    return W.beg[s] + (p - W.cum[s]);
-}
-
-__device__ void union_vjp(const PPParams &P, const VjpIO &V, const WarpSegs &W, float4 *S, float4 *SV, int64_t i,
-                          bool has, int c0, int xa, float4 me, float vix, float viy, float viz, Sum3 &a) {
-    const int lane = threadIdx.x & 31;
-    const int n = P.n_ios;
-    const int total = W.cum[PP_SEGS];
-    const int pself = has ? W.cum[8] + (int)(i - W.beg[8]) : -1000;
-    const int cx = (has ? __float_as_int(me.w) : c0) % n;
-    const float mx = (float)(cx - xa) + me.x, my = me.y + 1.0f, mz = me.z + 1.0f;
-    const float bcut2 = P.bcut2;
-    int sa = 0, sb = 0, ta = 0, tb = 0;
-    for (int b0 = 0; b0 < total; b0 += 64) {
-        S[lane] = stage_source(P, W, b0 + lane, sa);
-        S[32 + lane] = stage_source(P, W, b0 + 32 + lane, sb);
-        const int ja = stream_index(W, b0 + lane, ta), jb = stream_index(W, b0 + 32 + lane, tb);
-        SV[lane] = ja >= 0 ? make_float4(__ldg(&V.v0[ja]), __ldg(&V.v1[ja]), __ldg(&V.v2[ja]), 0.f)
-                           : make_float4(0.f, 0.f, 0.f, 0.f);
-        SV[32 + lane] = jb >= 0 ? make_float4(__ldg(&V.v0[jb]), __ldg(&V.v1[jb]), __ldg(&V.v2[jb]), 0.f)
-                                : make_float4(0.f, 0.f, 0.f, 0.f);
-        __syncwarp();
-        unsigned mh = test32(S, mx, my, mz, bcut2), ml = test32(S + 32, mx, my, mz, bcut2);
-        const int ts = pself - b0;
-        if (ts >= 0 && ts < 32) mh &= ~(0x80000000u >> ts);
-        if (ts >= 32 && ts < 64) ml &= ~(0x80000000u >> (ts - 32));
-        if (!has) mh = ml = 0u;
-        float px = 0.f, py = 0.f, pz = 0.f;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            unsigned m = h ? ml : mh;
-            const float4 *SB = S + 32 * h, *SVB = SV + 32 * h;
-            while (m) {
-                const int k = __clz(m);
-                m ^= 0x80000000u >> k;
-                const float4 q = SB[k];
-                const float rx = q.x - mx, ry = q.y - my, rz = q.z - mz;
-                const float r2 = rx * rx + ry * ry + rz * rz;
-                if (r2 > 0.0f) jacobian_term(rx, ry, rz, r2, SVB[k], vix, viy, viz, P, px, py, pz);
-            }
-        }
-        a.add_block(px, py, pz);
-        __syncwarp();
-    }
-}
-
-// the adjoint's product keeps the force's default shared-stream width
-constexpr int PP_WMAX_VJP = 16;
-
-struct PPVjpWarpShared {
-    float4 buf[64];   // staged source positions
-    float4 vbuf[64];  // and their v_j
-    WarpSegs seg;
+struct PPVjpWarpShared : PPWarpShared {
+    float4 vbuf[64];  // v_j of the staged sources
 };
 
-#ifndef PPV_MINB
-#define PPV_MINB 1
-#endif
-__global__ void __launch_bounds__(PP_CTA, PPV_MINB) pp_vjp_kernel(PPParams P, VjpIO V) {
-    __shared__ PPVjpWarpShared sh[PP_WARPS_CTA];
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int wib = threadIdx.x >> 5;
-    const bool has = i < P.N;
-    const int n = P.n_ios;
-    const float4 me = has ? P.pos[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-    int c = has ? __float_as_int(me.w) : -1;
-    const int c0 = __shfl_sync(0xffffffffu, c, 0);
-    if (!has) c = c0;
-    const int c31 = __reduce_max_sync(0xffffffffu, c);
-    const int xa = c0 % n, xb = c31 % n;
-    const bool one_row = (c0 / n) == (c31 / n) && xb - xa <= PP_WMAX_VJP && xb - xa + 3 <= n;
-    const float vix = has ? V.v0[i] : 0.f, viy = has ? V.v1[i] : 0.f, viz = has ? V.v2[i] : 0.f;
-    Sum3 a;
-    if (one_row) {
-        build_segments(P, sh[wib].seg, c0, xa, xb);
-        union_vjp(P, V, sh[wib].seg, sh[wib].buf, sh[wib].vbuf, i, has, c0, xa, me, vix, viy, viz, a);
-    } else {
-        lane_vjp(P, V, has, c, me, vix, viy, viz, a);
+// Product terms of one batch of 32 staged sources.
+__device__ __forceinline__ void vjp32(const PPParams &P, const float4 *S, const float4 *SV, float mx, float my, float mz,
+                                      float vix, float viy, float viz, bool has, Sum3 &a) {
+    unsigned m = has ? test32(S, mx, my, mz, P.bcut2) : 0u;
+    float px = 0.f, py = 0.f, pz = 0.f;
+    while (m) {
+        const int k = __clz(m);
+        m ^= 0x80000000u >> k;
+        const float4 q = S[k];
+        const float rx = q.x - mx, ry = q.y - my, rz = q.z - mz;
+        const float r2 = rx * rx + ry * ry + rz * rz;
+        if (r2 > 0.0f) jacobian_term(rx, ry, rz, r2, SV[k], vix, viy, viz, P, px, py, pz);
     }
-    if (has) {
-        V.w0[i] += V.scale * (a.x - a.cx);
-        V.w1[i] += V.scale * (a.y - a.cy);
-        V.w2[i] += V.scale * (a.z - a.cz);
+    a.add_block(px, py, pz);
+}
+
+__device__ void union_vjp(const PPParams &P, const VjpIO &V, PPVjpWarpShared &W, PPStream &T, bool has, float mx, float my,
+                          float mz, float vix, float viy, float viz, Sum3 &a) {
+    const int lane = threadIdx.x & 31;
+    float4 *S = W.u.buf, *SV = W.vbuf;
+    warp_box(W.box, mx, my, mz, P.bcut2, P.bpp2);
+    int fill = 0;
+    for (int b0 = 0; b0 < T.total; b0 += 32) {
+        const int slot = T.slot;
+        const float4 q = T.next(P, W, b0);
+        const float4 lo = W.box[0], hi = W.box[1];
+        const bool keep = b0 + lane < T.total && box_distance2(lo, hi, q) < lo.w;
+        const unsigned km = __ballot_sync(0xffffffffu, keep);
+        if (keep) {
+            const int at = fill + __popc(km & ((1u << lane) - 1u));
+            const int j = __ldg(&P.perm[slot]);
+            S[at] = q;
+            SV[at] = make_float4(__ldg(&V.v0[j]), __ldg(&V.v1[j]), __ldg(&V.v2[j]), 0.f);
+        }
+        fill += __popc(km);
+        __syncwarp();
+        if (fill >= 32) {
+            vjp32(P, S, SV, mx, my, mz, vix, viy, viz, has, a);
+            __syncwarp();
+            const float4 t = S[32 + lane], tv = SV[32 + lane];
+            if (32 + lane < fill) {
+                S[lane] = t;
+                SV[lane] = tv;
+            }
+            fill -= 32;
+            __syncwarp();
+        }
+    }
+    if (fill > 0) {
+        if (lane >= fill) S[lane] = make_float4(1.0e18f, 1.0e18f, 1.0e18f, 0.0f);
+        __syncwarp();
+        vjp32(P, S, SV, mx, my, mz, vix, viy, viz, has, a);
+    }
+    __syncwarp();
+}
+
+// The warp's target of each lane: its slot (lane 0's in padding lanes), cell
+// coordinates and the block of cells that the warp's targets span.
+struct PPTarget {
+    float4 me;
+    int slot, cx, cy, cz;
+    bool has;
+};
+
+__device__ __forceinline__ PPTarget warp_target(const PPParams &P, int j, PPBlock &B) {
+    PPTarget t;
+    t.has = j >= 0;
+    const int j0 = __shfl_sync(0xffffffffu, j, 0);   // a warp's first target is never padding
+    t.slot = t.has ? j : j0;
+    t.me = __ldg(&P.pos[t.slot]);
+    const int n = P.n_ios, c = __float_as_int(t.me.w);
+    const int row = (int)(__umulhi((unsigned)c, P.div_mul) >> P.div_shift);
+    t.cx = c - row * n;
+    t.cz = (int)(__umulhi((unsigned)row, P.div_mul) >> P.div_shift);
+    t.cy = row - t.cz * n;
+    B.xa = __reduce_min_sync(0xffffffffu, t.cx);
+    B.xb = __reduce_max_sync(0xffffffffu, t.cx);
+    B.ya = __reduce_min_sync(0xffffffffu, t.cy);
+    B.yb = __reduce_max_sync(0xffffffffu, t.cy);
+    B.za = __reduce_min_sync(0xffffffffu, t.cz);
+    B.zb = __reduce_max_sync(0xffffffffu, t.cz);
+    return t;
+}
+
+__global__ void __launch_bounds__(32) pp_vjp_kernel(PPParams P, VjpIO V) {
+    __shared__ PPVjpWarpShared sh;
+    const int64_t i = (int64_t)blockIdx.x * 32 + threadIdx.x;
+    const int j = P.tgt[i];   // with the length's load under way
+    if ((int64_t)blockIdx.x * 32 >= *P.tgt_n) return;
+    PPBlock B;
+    const PPTarget t = warp_target(P, j, B);
+    const int pi = P.perm[t.slot];
+    const float vix = V.v0[pi], viy = V.v1[pi], viz = V.v2[pi];
+    Sum3 a;
+    if (B.xb - B.xa <= P.wmax) {
+        PPStream T;
+        T.total = build_segments(P, sh.seg, sh.begin, B, T.nseg);
+        T.init(P, sh);
+        union_vjp(P, V, sh, T, t.has, (float)(t.cx - B.xa) + t.me.x, (float)(t.cy - B.ya + 1) + t.me.y,
+                  (float)(t.cz - B.za + 1) + t.me.z, vix, viy, viz, a);
+    } else {
+        lane_vjp(P, V, t.has, __float_as_int(t.me.w), t.me, vix, viy, viz, a);
+    }
+    if (t.has) {
+        V.w0[pi] += V.scale * (a.x - a.cx);
+        V.w1[pi] += V.scale * (a.y - a.cy);
+        V.w2[pi] += V.scale * (a.z - a.cz);
     }
 }
 
-// Full occupancy (16 CTAs of 4 warps, 32 registers): the per-lane walk is
-// bound by load latency, and more resident warps hide more of it than the
-// spilled registers cost (measured 14-16 % faster over the 256^3 run than
-// 3 CTAs of 8 warps at 64 registers).
-#ifndef PP_MINB
-#define PP_MINB 16
-#endif
-// The targets of one block of PP_CTA slots: [block * PP_CTA, block * PP_CTA + PP_CTA).
-// COUNT: accumulate the work counters (off unless asked for: the two counters
-// live through the whole walk and, within the 32-register budget, cost up to
-// a fifth of the sparse-region time).
+// Warps with fewer expected candidates per pair than this evaluate every pair.
+// The estimate takes the sources as evenly spread; around haloes more of them
+// are in range.  PP at z = 0 of the 256^3 run with 6 / 9 / 14 / 20: 9.8 / 9.0 /
+// 8.7 / 8.7 ms; 512^3 particles at z = 1 with 6 / 9 / 14: 25.0 / 23.4 / 22.9 ms.
+constexpr float PP_COMPACT = 14.0f;
+
+// The warp's 32 target places from i on.  COUNT: accumulate the work counters
+// (off unless asked for: they live through the whole stream).
 template <bool PM3, bool COUNT>
-__device__ __forceinline__ void pp_block(const PPParams &P, int64_t block, PPShared &sh) {
-    const int64_t i = block * PP_CTA + threadIdx.x;
-    const int wib = threadIdx.x >> 5;
-    const bool has = i < P.N;
-    const int n = P.n_ios;
-    const float4 me = has ? P.pos[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-    int c = has ? __float_as_int(me.w) : -1;
-    const int c0 = __shfl_sync(0xffffffffu, c, 0);
-    if (!has) c = c0;
-    // cells are non-decreasing along the warp (padding lanes repeat lane 0's):
-    // lane 0 and the largest cell bound its extent
-    const int c31 = __reduce_max_sync(0xffffffffu, c);
-    const int xa = c0 % n, xb = c31 % n;
-    // warps inside one row, at most wmax + 1 cells wide, share a source stream
-    const bool one_row = (c0 / n) == (c31 / n) && xb - xa <= P.wmax && xb - xa + 3 <= n;
-    if (one_row) build_segments(P, sh.w[wib].u.seg, c0, xa, xb);
+__device__ __forceinline__ void pp_warp(const PPParams &P, int64_t i, PPWarpShared &W) {
+    const int j = P.tgt[i];   // with the length's load under way
+    if ((i & ~(int64_t)31) >= *P.tgt_n) return;   // whole warps: places past the last pencil's end
+    PPBlock B;
+    const PPTarget t = warp_target(P, j, B);
+    const bool stream = B.xb - B.xa <= P.wmax;
+    // the sums' destinations on their way while the pairs are worked on (perm
+    // stays inside the cell; both prefetches: 1.38 -> 1.35 ms at z = 49)
+    if (P.accumulate) {
+        prefetch_l1(&P.acc0[t.slot]);
+        prefetch_l1(&P.acc1[t.slot]);
+        prefetch_l1(&P.acc2[t.slot]);
+    }
+    if (P.kick != 0.0f) {
+        prefetch_l1(&P.vel0[t.slot]);
+        prefetch_l1(&P.vel1[t.slot]);
+        prefetch_l1(&P.vel2[t.slot]);
+    }
+    PPLane L;
+    L.has = t.has;
     // PP range of this target: b_3 inside a refined subtile of the third level
-    float bcut2 = P.bcut2, ibc = P.inv_bcut;
-    if (PM3 && has) {
+    float ibc = P.inv_bcut;
+    L.bcut2 = P.bcut2;
+    if (PM3) {
         const int T = P.pm3_T;
-        const int s = ((c / (n * n)) / T * P.pm3_ns + ((c / n) % n) / T) * P.pm3_ns + (c % n) / T;
+        const int s = (t.cz / T * P.pm3_ns + t.cy / T) * P.pm3_ns + t.cx / T;
         if (__ldg(&P.pm3_slot[s]) >= 0) {
-            bcut2 = P.bcut2_3;
+            L.bcut2 = P.bcut2_3;
             ibc = P.inv_bcut_3;
         }
     }
+    L.ib2 = ibc * ibc;
+    L.coef = P.coef * (L.ib2 * ibc);
+    L.mx = (float)(t.cx - B.xa) + t.me.x;
+    L.my = (float)(t.cy - B.ya + 1) + t.me.y;
+    L.mz = (float)(t.cz - B.za + 1) + t.me.z;
     Sum3 a;
     unsigned pairs = 0, cands = 0;
-    if (one_row)
-        union_path(P, sh.w[wib].u.seg, sh.w[wib].u.buf, sh.w[wib].u.box, i, has, c0, xa, me, bcut2, ibc, a, pairs,
-                   cands);
-    else
-        lane_path(P, has, c, me, bcut2, ibc, a, pairs, cands);
-    if (has) finish(P, P.perm[i], a.x - a.cx, a.y - a.cy, a.z - a.cz);
+    if (stream) {
+        PPStream T;
+        T.total = build_segments(P, W.seg, W.begin, B, T.nseg);
+        T.init(P, W);
+        if (warp_box(W.box, L.mx, L.my, L.mz, L.bcut2, P.bpp2) < PP_COMPACT)
+            stream_compact<COUNT>(P, W, T, L, a, pairs, cands);
+        else
+            stream_sparse(P, W, T, L, a, pairs, cands);
+    } else {
+        lane_path(P, __float_as_int(t.me.w), t.me, L, a, pairs, cands);
+    }
+    if (t.has) finish(P, P.perm[t.slot], a.x - a.cx, a.y - a.cy, a.z - a.cz);
     if constexpr (COUNT) {
         add_stats(P.stats, pairs, cands);
-        if (!one_row) add_stats(P.stats + 2, pairs, cands);   // warp-uniform
+        if (!stream) add_stats(P.stats + 2, pairs, cands);   // warp-uniform
     }
 }
 
+// 64 registers, 32 warps per SM: the stream loops' packed constants and sums fit;
+// more warps with 48 registers or fewer with 80 measured slower (z = 49 / z = 0:
+// 1.56 / 9.4 and 1.59 / 9.0 ms against 1.38 / 8.7), and so did a kernel of its own
+// for the compact warps (1.40 / 9.3).  Two warps per CTA: one is 2 % faster late
+// (long warps hold no place of a finished one) and 6 % slower early.
+constexpr int PP_WARPS = 2;
 template <bool PM3, bool COUNT>
-__global__ void __launch_bounds__(PP_CTA, PP_MINB) pp_kernel(PPParams P) {
-    __shared__ PPShared sh;
-    pp_block<PM3, COUNT>(P, blockIdx.x, sh);
+__global__ void __launch_bounds__(PP_WARPS * 32, 32 / PP_WARPS) pp_kernel(PPParams P) {
+    __shared__ PPWarpShared sh[PP_WARPS];
+    pp_warp<PM3, COUNT>(P, (int64_t)blockIdx.x * (PP_WARPS * 32) + threadIdx.x, sh[threadIdx.x >> 5]);
 }
 
 // ------------------------------------------------- ensemble: one persistent PP
@@ -797,10 +1234,13 @@ __global__ void __launch_bounds__(256) pp_item_cost_kernel(const PPParams *__res
     if (k >= n_items) return;
     const int b = item_box[k];
     const PPParams &P = boxes[b];
-    const int64_t i0 = (int64_t)(k - base[b]) * PP_CTA;
-    const int64_t i1 = min(i0 + PP_CTA, P.N);
+    const int64_t i0 = (int64_t)(k - base[b]) * PP_ITEM;
+    const int64_t i1 = min(i0 + PP_ITEM, (int64_t)*P.tgt_n);
     unsigned s = 0;
-    for (int64_t i = i0; i < i1; ++i) s += (unsigned)__ldg(&P.count[__float_as_int(__ldg(&P.pos[i]).w)]);
+    for (int64_t i = i0; i < i1; ++i) {
+        const int j = P.tgt[i];
+        if (j >= 0) s += (unsigned)__ldg(&P.count[__float_as_int(__ldg(&P.pos[j]).w)]);
+    }
     cost[k] = s;
 }
 
@@ -826,13 +1266,13 @@ __global__ void __launch_bounds__(1024) pp_item_order_kernel(const unsigned *__r
     for (int k = threadIdx.x; k < n_items; k += blockDim.x) order[atomicAdd(&offs[32 - __clz(cost[k] + 1u)], 1)] = k;
 }
 
-__global__ void __launch_bounds__(PP_CTA, PP_MINB) pp_persistent_kernel(const PPParams *__restrict__ boxes,
+__global__ void __launch_bounds__(PP_ITEM, 8) pp_persistent_kernel(const PPParams *__restrict__ boxes,
                                                                        const int32_t *__restrict__ item_box,
                                                                        const int32_t *__restrict__ base,
                                                                        const int32_t *__restrict__ order,
                                                                        PPQueueDev *q, int epoch,
                                                                        unsigned long long timeout_ns) {
-    __shared__ PPShared sh;
+    __shared__ PPWarpShared sh[PP_ITEM / 32];
     __shared__ int s_item, s_ok;
     if (threadIdx.x == 0) {
         int ok = 1;
@@ -858,13 +1298,50 @@ __global__ void __launch_bounds__(PP_CTA, PP_MINB) pp_persistent_kernel(const PP
         if (item >= count) break;
         const int k = order[item];
         const int b = item_box[k];
-        pp_block<false, false>(boxes[b], (int64_t)(k - base[b]), sh);
+        pp_warp<false, false>(boxes[b], (int64_t)(k - base[b]) * PP_ITEM + threadIdx.x, sh[threadIdx.x >> 5]);
     }
 }
 
 }  // namespace
 
+// Target places, a whole number of items: every pencil's tail padded to a whole
+// warp (a pencil with targets is at most 31 places longer than they are).
+int64_t pp_target_items(int64_t N, int n_ios) {
+    const int64_t pencils = (int64_t)pencils_y(n_ios) * pencils_z(n_ios);
+    return (N + 31 * (pencils < N ? pencils : N) + PP_ITEM - 1) / PP_ITEM;
+}
+
+int64_t pp_target_slots(int64_t N, int n_ios) { return pp_target_items(N, n_ios) * PP_ITEM; }
+
+// Cells that can hold PP_SORT_MIN particles.
+int64_t pp_dense_cells(int64_t N) { return N / PP_SORT_MIN; }
+
 static PPParams pp_params(cube2_ctx *ctx, const cube2_particles *p, int accumulate, float kick);
+
+// PP inputs: target order, float positions, dense cells sorted by sub-cell.
+static void launch_pp_inputs(cube2_ctx *ctx, const cube2_particles *p) {
+    const int n = ctx->n_ios;
+    int *list_n = ctx->big_n;
+    unsigned *tgt_n = reinterpret_cast<unsigned *>(ctx->big_n + 1);
+    {
+        ProfScope prof(ctx, P_PP_ORDER, 0);
+        cudaMemsetAsync(ctx->big_n, 0, 2 * sizeof(int), ctx->stream);
+        pp_pencil_kernel<<<(unsigned)(pencils_y(n) * pencils_z(n)), PREP_CTA, 0, ctx->stream>>>(
+            p->count, p->start, n, PP_SORT_MIN, ctx->pp_tgt, tgt_n, ctx->pp_dense, list_n);
+    }
+    {
+        ProfScope prof(ctx, P_PREP, 0);
+        prep_positions_kernel<<<(unsigned)((ctx->N + PREP_CTA - 1) / PREP_CTA), PREP_CTA, 0, ctx->stream>>>(
+            p->off[0], p->off[1], p->off[2], ctx->cellid, ctx->pos4, ctx->pp_perm, ctx->N);
+    }
+    {
+        ProfScope prof(ctx, P_PP_ORDER, 0);
+        pp_dense_sort_kernel<<<(unsigned)(ctx->num_sms * 8), 256, 0, ctx->stream>>>(
+            p->off[0], p->off[1], p->off[2], p->count, p->start, ctx->pp_dense, list_n, ctx->pos4, ctx->pp_perm,
+            ctx->pp_tgt);
+    }
+    ctx->launches += 3;
+}
 
 cudaError_t launch_pp_vjp(cube2_ctx *ctx, const cube2_particles *p, const float *const v[3], float *const w[3]) {
     if (ctx->N == 0) return cudaSuccess;
@@ -873,12 +1350,10 @@ cudaError_t launch_pp_vjp(cube2_ctx *ctx, const cube2_particles *p, const float 
     V.v0 = v[0]; V.v1 = v[1]; V.v2 = v[2];
     V.w0 = w[0]; V.w1 = w[1]; V.w2 = w[2];
     V.scale = (float)((double)P.coef / ctx->s_ios);
+    launch_pp_inputs(ctx, p);
     ProfScope prof(ctx, P_PP_VJP, 0);
-    const int nblocks = (int)((ctx->N + PP_CTA - 1) / PP_CTA);
-    prep_positions_kernel<<<(unsigned)nblocks, PP_CTA, 0, ctx->stream>>>(p->off[0], p->off[1], p->off[2], ctx->cellid,
-                                                                       ctx->pos4, nullptr, ctx->N);
-    pp_vjp_kernel<<<(unsigned)nblocks, PP_CTA, 0, ctx->stream>>>(P, V);
-    ctx->launches += 2;
+    pp_vjp_kernel<<<(unsigned)(pp_target_slots(ctx->N, ctx->n_ios) / 32), 32, 0, ctx->stream>>>(P, V);
+    ctx->launches += 1;
     return cudaGetLastError();
 }
 
@@ -886,6 +1361,8 @@ static PPParams pp_params(cube2_ctx *ctx, const cube2_particles *p, int accumula
     PPParams P{};
     P.pos = ctx->pos4;
     P.perm = ctx->pp_perm;
+    P.tgt = ctx->pp_tgt;
+    P.tgt_n = reinterpret_cast<unsigned *>(ctx->big_n + 1);
     P.count = p->count; P.start = p->start;
     P.acc0 = p->acc[0]; P.acc1 = p->acc[1]; P.acc2 = p->acc[2];
     if (ctx->vel32) {   // FP16 storage: the second kick updates the step's FP32 working copy
@@ -896,12 +1373,19 @@ static PPParams pp_params(cube2_ctx *ctx, const cube2_particles *p, int accumula
     P.stats = ctx->pp_stats;
     P.N = ctx->N;
     P.n_ios = ctx->n_ios;
+    {   // ceil(2^(31 + l) / n) with 2^(l-1) < n <= 2^l: exact quotients below 2^31
+        int l = 1;
+        while ((1 << l) < ctx->n_ios) ++l;
+        P.div_mul = (unsigned)(((1ull << (31 + l)) + (unsigned)ctx->n_ios - 1) / (unsigned)ctx->n_ios);
+        P.div_shift = l - 1;
+    }
     P.accumulate = accumulate;
     const double s = ctx->s_ios;
     P.inv_bpp = (float)(s / ctx->cfg.b_pp);
     P.inv_bcut = (float)(s / ctx->b_range);
     P.bcut2 = (float)((ctx->b_range / s) * (ctx->b_range / s));
     P.bpp2 = (float)((ctx->cfg.b_pp / s) * (ctx->cfg.b_pp / s));
+    P.ratio2 = (float)((s / ctx->cfg.b_pp) * (s / ctx->cfg.b_pp));
     const double vp = ctx->cfg.box * ctx->cfg.box * ctx->cfg.box / (double)ctx->N;
     P.coef = (float)(vp / (4.0 * 3.14159265358979323846) / (s * s));
     P.kick = kick;
@@ -920,36 +1404,23 @@ static PPParams pp_params(cube2_ctx *ctx, const cube2_particles *p, int accumula
 cudaError_t launch_pp(cube2_ctx *ctx, const cube2_particles *p, int accumulate, float kick) {
     PPParams P = pp_params(ctx, p, accumulate, kick);
     if (ctx->N == 0) return cudaSuccess;
-    const int nblocks = (int)((ctx->N + PP_CTA - 1) / PP_CTA);
-    {
-        ProfScope prof(ctx, P_PREP, 0);
-        prep_positions_kernel<<<(unsigned)nblocks, PP_CTA, 0, ctx->stream>>>(p->off[0], p->off[1], p->off[2],
-                                                                           ctx->cellid, ctx->pos4, ctx->pp_perm, ctx->N);
-    }
-    {
-        ProfScope prof(ctx, P_PP_ORDER, 0);
-        cudaMemsetAsync(ctx->big_n, 0, sizeof(int), ctx->stream);
-        pp_dense_list_kernel<<<(unsigned)((ctx->n_cells + 255) / 256), 256, 0, ctx->stream>>>(p->count, ctx->n_cells,
-                                                                                          ctx->big, ctx->big_n);
-        pp_dense_sort_kernel<<<(unsigned)(ctx->num_sms * 8), 256, 0, ctx->stream>>>(
-            p->off[0], p->off[1], p->off[2], p->count, p->start, ctx->big, ctx->big_n, ctx->pos4, ctx->pp_perm);
-    }
+    const unsigned ctas = (unsigned)(pp_target_slots(ctx->N, ctx->n_ios) / (PP_WARPS * 32));
+    launch_pp_inputs(ctx, p);
     if (ctx->defer_pp) {   // an ensemble's persistent kernel runs this box's PP later
         static_assert(sizeof(PPParams) <= sizeof(ctx->pp_deferred), "deferred PP parameters");
         memcpy(ctx->pp_deferred, &P, sizeof P);
-        ctx->launches += 3;
         return cudaGetLastError();
     }
     {
         ProfScope prof(ctx, P_PP, 0);
         if (P.pm3_slot)
-            (ctx->pp_count ? pp_kernel<true, true> : pp_kernel<true, false>)<<<(unsigned)nblocks, PP_CTA, 0,
+            (ctx->pp_count ? pp_kernel<true, true> : pp_kernel<true, false>)<<<ctas, PP_WARPS * 32, 0,
                                                                               ctx->stream>>>(P);
         else
-            (ctx->pp_count ? pp_kernel<false, true> : pp_kernel<false, false>)<<<(unsigned)nblocks, PP_CTA, 0,
+            (ctx->pp_count ? pp_kernel<false, true> : pp_kernel<false, false>)<<<ctas, PP_WARPS * 32, 0,
                                                                                 ctx->stream>>>(P);
     }
-    ctx->launches += 4;
+    ctx->launches += 1;
     return cudaGetLastError();
 }
 
@@ -965,7 +1436,7 @@ cudaError_t launch_pp_persistent_step(cudaStream_t st, const void *boxes, const 
     // the host's publication of this step's work count
     cudaError_t e = cudaMemcpyAsync(&q->ready, publish_host, sizeof(int), cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return e;
-    pp_persistent_kernel<<<(unsigned)grid, PP_CTA, 0, st>>>(B, item_box, base, order, q, epoch, timeout_ns);
+    pp_persistent_kernel<<<(unsigned)grid, PP_ITEM, 0, st>>>(B, item_box, base, order, q, epoch, timeout_ns);
     return cudaGetLastError();
 }
 
