@@ -15,6 +15,7 @@
 
 namespace cube2 {
 bool fft_size_supported(int n);
+int64_t fft_twiddle_entries(int n);
 
 int set_error(cube2_ctx *ctx, int code, const std::string &msg) {
     if (ctx) ctx->err = msg;
@@ -320,7 +321,7 @@ int cube2_init_mesh(cube2_ctx **out, const cube2_config *cfg, void *stream) {
             const size_t h = (size_t)(L.n / 2 + 1);
             alloc((void **)&L.green2, h * h * (size_t)L.kxp * sizeof(float));
         }
-        alloc((void **)&L.tw, (size_t)L.n * sizeof(float2));
+        alloc((void **)&L.tw, (size_t)fft_twiddle_entries(L.n) * sizeof(float2));
         if (e == cudaSuccess) e = cudaMemsetAsync(L.spec, 0, nh * sizeof(float2), c->stream);
     }
     const size_t N = (size_t)c->N;
@@ -351,7 +352,7 @@ int cube2_init_mesh(cube2_ctx **out, const cube2_config *cfg, void *stream) {
         alloc((void **)&L.spec, (size_t)M.max_tiles * nh * sizeof(float2));
         L.green_len = green_table_len(L.n);
         alloc((void **)&L.green, (size_t)L.green_len * sizeof(float));
-        alloc((void **)&L.tw, (size_t)L.n * sizeof(float2));
+        alloc((void **)&L.tw, (size_t)fft_twiddle_entries(L.n) * sizeof(float2));
         alloc((void **)&M.rho_max, (size_t)M.n_sub * 4);
         alloc((void **)&M.slot, (size_t)M.n_sub * 4);
         alloc((void **)&M.list, (size_t)M.max_tiles * 4);

@@ -51,7 +51,7 @@ struct Level {
     // (zero past kx = n/2): read by the z pass with plain indices (n <= 1024)
     float *green2 = nullptr;
     int64_t green_len = 0;   // entries of the reduced table
-    float2 *tw = nullptr;    // [n] twiddles exp(-2 pi i k / n)
+    float2 *tw = nullptr;    // twiddle rows of every stage, both directions (fft.cu)
     uint64_t mean_int = 0;   // M = floor(N 2^48 / n^3)
     float dens_scale = 0;    // RN32(n^3/N 2^-48)
     bool has_green = false, has_density = false, has_potential = false;

@@ -6,21 +6,29 @@
 // (multiple of 16, so every row starts on a 128-byte boundary).
 //
 // Passes (each one read + one write of the grid, in place where possible):
-//   X  r2c : 2L real rows per CTA packed as L complex lines a + ib, one complex
-//            FFT per line, split into the two half spectra.
+//   X  r2c : two real rows packed as one complex line a + ib, one complex FFT per
+//            line, split into the two half spectra.
 //   Y      : L consecutive kx columns x n rows of one kz plane per CTA.
 //   Z+G    : L consecutive kx columns x n planes of one ky row per CTA: forward
 //            FFT along z, multiply by G(k) (1/n^3 folded in), inverse FFT along z.
 //   Y^-1, X^-1 c2r : mirror images of Y and X.
-// Within a CTA the L lines live in shared memory as S[pos * (L+1) + line]; the
-// odd line stride keeps both line-parallel and position-parallel accesses free
-// of bank conflicts.  Each line is transformed by a Stockham autosort sequence of
-// radix-8/4/3/2 stages (natural order in and out): a stage reads R values with
-// stride n/R, applies the twiddles exp(-2 pi i r (j mod Ns) / (Ns R)), does an
-// R-point DFT in registers and writes them with stride Ns to position
-// (j / Ns) Ns R + (j mod Ns).  Every thread holds its values in registers
-// across a barrier, so stages run in place.  Twiddles are an FP32 table
-// exp(-2 pi i k/n) built from FP64 sincospi.
+// A line is transformed by a Stockham autosort sequence of radix-16/8/4/3/2 stages
+// (natural order in and out): a stage takes R values with stride n/R, applies
+// the twiddles exp(-2 pi i r (j mod Ns) / (Ns R)), does an R-point DFT in
+// registers and puts them with stride Ns to position (j / Ns) Ns R + (j mod Ns).
+// The first stage takes its values straight from global memory and the last one
+// writes them there, so a line of three stages crosses shared memory twice; the
+// passes are bound by that crossing, not by DRAM.  In the z pass the forward
+// transform's last stage leaves each thread the values that the inverse's first
+// stage wants (the inverse runs the radices in reverse), with G applied between
+// them in registers.  In the x passes the threads of a line take the last
+// (first) stage's butterflies in pairs j, n/R - j, which hold both members of
+// every conjugate pair k, n - k: the two half spectra are split (joined) in
+// registers.  512^3: x 0.35 -> 0.18 ms each (0.165 at the copy rate), z + G 0.41 -> 0.38, y
+// 0.23 -> 0.24 (the rate of its strided rows); all five 1.58 -> 1.23 ms, at 1024^3
+// 15.5 -> 10.3 ms, at 128^3 59 -> 44 us, against every stage through shared memory.
+// Twiddles are FP32 tables built from FP64 sincospi, one row of n/R entries per
+// stage and factor r, so that a stage's reads are consecutive.
 #include "common.cuh"
 
 #include <algorithm>
@@ -89,6 +97,39 @@ struct Dft<8, INV> {
 };
 
 template <bool INV>
+struct Dft<16, INV> {   // 4 x 4
+    __device__ __forceinline__ static void run(float2 *v) {
+        constexpr float c1 = 0.92387953251128675613f, s1 = 0.38268343236508977173f, h = 0.70710678118654752440f;
+        // w16^m, m = n2 k1 (forward: exp(-i pi m / 8))
+        constexpr float C[10] = {1.0f, c1, h, s1, 0.0f, 0.0f, -h, 0.0f, 0.0f, -c1};
+        constexpr float D[10] = {0.0f, s1, h, c1, 1.0f, 0.0f, h, 0.0f, 0.0f, -s1};
+        float2 a[4][4];
+#pragma unroll
+        for (int n2 = 0; n2 < 4; ++n2) {
+#pragma unroll
+            for (int n1 = 0; n1 < 4; ++n1) a[n2][n1] = v[4 * n1 + n2];
+            Dft<4, INV>::run(a[n2]);
+        }
+#pragma unroll
+        for (int n2 = 1; n2 < 4; ++n2)
+#pragma unroll
+            for (int k1 = 1; k1 < 4; ++k1) {
+                const int m = n2 * k1;
+                const float2 b = a[n2][k1];
+                if (m == 4) a[n2][k1] = rot90<INV>(b);
+                else a[n2][k1] = cmul(b, make_float2(C[m], INV ? D[m] : -D[m]));
+            }
+#pragma unroll
+        for (int k1 = 0; k1 < 4; ++k1) {
+            float2 b[4] = {a[0][k1], a[1][k1], a[2][k1], a[3][k1]};
+            Dft<4, INV>::run(b);
+#pragma unroll
+            for (int k2 = 0; k2 < 4; ++k2) v[k1 + 4 * k2] = b[k2];
+        }
+    }
+};
+
+template <bool INV>
 struct Dft<3, INV> {
     __device__ __forceinline__ static void run(float2 *v) {
         const float c = -0.5f;
@@ -103,195 +144,367 @@ struct Dft<3, INV> {
     }
 };
 
-__host__ __device__ constexpr int pick_radix(int rem) {
-    return rem % 3 == 0 ? 3 : (rem == 2 || rem == 4) ? rem : rem == 16 ? 4 : rem % 8 == 0 ? 8 : rem % 4 == 0 ? 4 : 2;
+// Radix of stage s of an n-point line (0 past the last): as few stages as radices
+// up to 16 allow with the values per thread below (fewer exchanges, fewer
+// rounded twiddles), a 3 last, which leaves the last stage an even number of
+// butterflies.  The x passes (xp) hold two butterflies of the last radix at once
+// and take 128 as 16 8.  (256 as 16 16 is no faster and its low modes come out
+// less exact: relative error of the potential 9.4e-7 against 5.8e-7.)
+__host__ __device__ constexpr int radix_at(int n, int s, bool xp) {
+    constexpr int P[17][6] = {{8, 4, 2}, {12, 4, 3}, {16, 4, 4}, {24, 8, 3}, {32, 8, 4}, {48, 4, 4, 3}, {64, 8, 8},
+                              {96, 8, 4, 3}, {128, 8, 16}, {192, 8, 8, 3}, {256, 8, 8, 4}, {384, 8, 4, 4, 3}, {512, 8, 8, 8},
+                              {768, 8, 8, 4, 3}, {1024, 16, 8, 8}, {1536, 8, 8, 8, 3}, {2048, 16, 16, 8}};
+    if (xp && n == 128) return s == 0 ? 16 : s == 1 ? 8 : 0;
+    for (int i = 0; i < 17; ++i)
+        if (P[i][0] == n) return s < 5 ? P[i][s + 1] : 0;
+    return 0;
+}
+__host__ __device__ constexpr int stages_of(int n, bool xp) {
+    int s = 0;
+    while (radix_at(n, s, xp) != 0) ++s;
+    return s;
+}
+// Twiddle rows: for the tile passes and the x passes, forward and inverse (which
+// runs the radices in reverse), stage by stage from the second on, entry
+// (r - 1) n/R + j of a stage is exp(-+ 2 pi i r (j mod Ns) / (Ns R)).
+__host__ __device__ constexpr int twiddle_row(int n, bool xp, bool inv, int stage) {
+    int v = 0;
+    for (int k = 0; k < 4; ++k) {
+        const bool kx = k >= 2, ki = k % 2 == 1;
+        const int S = stages_of(n, kx);
+        for (int i = 1; i < S; ++i) {
+            if (kx == xp && ki == inv && i == stage) return v;
+            const int R = radix_at(n, ki ? S - 1 - i : i, kx);
+            v += (R - 1) * (n / R);
+        }
+        if (kx == xp && ki == inv) return v;   // stage past the last: the end of these rows
+    }
+    return v;
+}
+__host__ __device__ constexpr int twiddle_entries(int n) { return twiddle_row(n, true, true, 99); }
+
+template <int N, bool INV, bool XP>
+struct Plan {
+    static constexpr int S = stages_of(N, XP);
+    __host__ __device__ static constexpr int radix(int s) { return radix_at(N, INV ? S - 1 - s : s, XP); }
+    __host__ __device__ static constexpr int span(int s) {   // Ns: product of the earlier radices
+        int v = 1;
+        for (int i = 0; i < s; ++i) v *= radix(i);
+        return v;
+    }
+};
+
+__global__ void twiddle_rows_kernel(float2 *tw, int n) {
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    for (int k = 0; k < 4; ++k) {
+        const bool xp = k >= 2, inv = k % 2 == 1;
+        const int S = stages_of(n, xp);
+        int span = radix_at(n, inv ? S - 1 : 0, xp);
+        for (int s = 1; s < S; ++s) {
+            const int R = radix_at(n, inv ? S - 1 - s : s, xp), nb = n / R, at = twiddle_row(n, xp, inv, s);
+            if (idx >= at && idx < at + (R - 1) * nb) {
+                const int r = (idx - at) / nb + 1, j = (idx - at) % nb;
+                double si, co;
+                sincospi((inv ? 2.0 : -2.0) * (double)(r * (j % span)) / (double)(span * R), &si, &co);
+                tw[idx] = make_float2((float)co, (float)si);
+                return;
+            }
+            span *= R;
+        }
+    }
 }
 
-template <int N, int L, int LP, int T, int R, int NS, bool INV>
-__device__ __forceinline__ void stockham_stage(float2 *S, const float2 *__restrict__ tw) {
-    constexpr int NB = N / R;
-    constexpr int TOT = NB * L;
-    constexpr int PER = (TOT + T - 1) / T;
+// Values of stage s's butterflies j twiddled and transformed; nothing to twiddle in stage 0.
+template <int N, bool INV, bool XP, int s, int R>
+__device__ __forceinline__ void butterfly(float2 (&v)[R], int j, const float2 *__restrict__ tw) {
+    if constexpr (s > 0) {
+        constexpr int row = twiddle_row(N, XP, INV, s);
+#pragma unroll
+        for (int r = 1; r < R; ++r) v[r] = cmul(v[r], __ldg(&tw[row + (r - 1) * (N / R) + j]));
+    }
+    Dft<R, INV>::run(v);
+}
+
+// ------------------------------------------------------- tiles of y and z
+// L lines (columns) per tile, position-major in shared memory: a row of a tile
+// is 16 consecutive complex values (128 bytes) in shared memory as in global.
+// Thread b takes butterflies b, b + T, ... of every stage: line b % L, j = b / L.
+// About 16 values (24 with a radix 3) per thread: at 512 two CTAs of 512 threads
+// per SM with 64 registers.  A 1024-point tile of 16 lines leaves one CTA per SM:
+// its y passes take 8 lines (2.34 -> 1.83 ms), the z pass, with the strides of
+// whole planes, stays at 16 (3.85 against 4.26 ms).  Up to 128 points the grids
+// are small and registers are left to the compiler (z at 64: 8.9 -> 6.7 us).
+template <int N, bool Z>
+struct Tile {
+    static constexpr int L = N >= 2048 || (N == 1024 && !Z) ? 8 : FFT_LINES;
+    static constexpr int V = (N % 3 == 0 ? 3 : 2) * (N <= 96 ? 4 : 8);
+    static constexpr int T0 = N * L / V;
+    static constexpr int T = T0 < 32 ? 32 : (T0 > 1024 ? 1024 : T0);
+    static constexpr size_t SMEM = (size_t)N * L * sizeof(float2);
+    static constexpr int MINB = (N > 128 && T <= 512 && 2 * SMEM <= 200 * 1024) ? (N % 3 == 0 ? 768 : 1024) / T : 1;
+    template <int R>
+    static constexpr int per() { return (N / R * L + T - 1) / T; }
+};
+
+// Tiles are read and written once a pass: streaming loads and stores (512^3: z
+// 0.41 -> 0.38 ms); past 512 the plain L2 ones (z at 1024: 3.85 against 4.00 ms).
+template <int N>
+__device__ __forceinline__ float2 tile_load(const float2 *p) {
+    if constexpr (N <= 512) return __ldcs(p);
+    return __ldcg(p);
+}
+template <int N>
+__device__ __forceinline__ void tile_store(float2 *p, float2 v) {
+    if constexpr (N <= 512) __stcs(p, v);
+    else __stcg(p, v);
+}
+
+// Stages s .. of the tile's lines.  In stage 0 the values come from load(pos,
+// line); the last stage hands its values to store(pos, line, v) or, with KEEP,
+// leaves them in out.
+template <int N, bool Z, bool INV, int s, class Load, class Store>
+__device__ __forceinline__ void tile_stages(float2 *S, const float2 *__restrict__ tw, Load load, Store store) {
+    using TL = Tile<N, Z>;
+    constexpr int R = Plan<N, INV, false>::radix(s), NB = N / R, NS = Plan<N, INV, false>::span(s), L = TL::L, T = TL::T;
+    constexpr int PER = TL::template per<R>();
+    constexpr bool LAST = s + 1 == Plan<N, INV, false>::S;
     float2 v[PER][R];
 #pragma unroll
     for (int p = 0; p < PER; ++p) {
         const int b = threadIdx.x + p * T;
-        if (TOT % T == 0 || b < TOT) {
+        if (NB * L % T == 0 || b < NB * L) {
             const int line = b % L, j = b / L;
 #pragma unroll
-            for (int r = 0; r < R; ++r) v[p][r] = S[(j + r * NB) * LP + line];
-            if (NS > 1) {
-                const int k = j % NS;
-#pragma unroll
-                for (int r = 1; r < R; ++r) {
-                    float2 w = __ldg(&tw[r * k * (N / (NS * R))]);
-                    if (INV) w.y = -w.y;
-                    v[p][r] = cmul(v[p][r], w);
-                }
-            }
-            Dft<R, INV>::run(v[p]);
+            for (int r = 0; r < R; ++r) v[p][r] = s == 0 ? load(j + r * NB, line, p, r) : S[(j + r * NB) * L + line];
         }
     }
-    __syncthreads();
 #pragma unroll
     for (int p = 0; p < PER; ++p) {
         const int b = threadIdx.x + p * T;
-        if (TOT % T == 0 || b < TOT) {
-            const int line = b % L, j = b / L;
-            const int k = j % NS;
-            const int base = (j / NS) * NS * R + k;
+        if (NB * L % T == 0 || b < NB * L) butterfly<N, INV, false, s>(v[p], b / L, tw);
+    }
+    if constexpr (!LAST) {
+        if (s > 0) __syncthreads();   // all have read what is overwritten now
 #pragma unroll
-            for (int r = 0; r < R; ++r) S[(base + r * NS) * LP + line] = v[p][r];
+        for (int p = 0; p < PER; ++p) {
+            const int b = threadIdx.x + p * T;
+            if (NB * L % T == 0 || b < NB * L) {
+                const int line = b % L, j = b / L, base = (j / NS) * NS * R + j % NS;
+#pragma unroll
+                for (int r = 0; r < R; ++r) S[(base + r * NS) * L + line] = v[p][r];
+            }
+        }
+        __syncthreads();
+        tile_stages<N, Z, INV, s + 1>(S, tw, load, store);
+    } else {
+#pragma unroll
+        for (int p = 0; p < PER; ++p) {
+            const int b = threadIdx.x + p * T;
+            if (NB * L % T == 0 || b < NB * L) {
+                const int line = b % L, j = b / L;
+#pragma unroll
+                for (int r = 0; r < R; ++r) store(j + r * NS, line, p, r, v[p][r]);   // NS = NB: base is j
+            }
         }
     }
-    __syncthreads();
 }
-
-template <int N, int L, int LP, int T, int NS, bool INV>
-__device__ __forceinline__ void fft_lines(float2 *S, const float2 *__restrict__ tw) {
-    if constexpr (NS < N) {
-        constexpr int R = pick_radix(N / NS);
-        stockham_stage<N, L, LP, T, R, NS, INV>(S, tw);
-        fft_lines<N, L, LP, T, NS * R, INV>(S, tw);
-    }
-}
-
-// L lines per tile; x passes pad the line stride to L + 1 (their load and store
-// phases are position-parallel), y/z passes keep it at L so every tile row is a
-// 16-byte-aligned 128-byte line filled with asynchronous 16-byte copies.
-template <int N>
-struct Tile {
-    static constexpr int L = N >= 2048 ? 8 : FFT_LINES;
-    static constexpr int LP = L + 1;
-    static constexpr int LPY = L;
-    static constexpr int T0 = N * L / 16;
-    static constexpr int T = T0 < 64 ? 64 : (T0 > 1024 ? 1024 : T0);
-    static constexpr size_t SMEM = (size_t)N * LP * sizeof(float2);
-    static constexpr size_t SMEMY = (size_t)N * LPY * sizeof(float2);
-    // resident CTAs the z pass asks registers for: two for 512-thread tiles
-    // that fit twice in shared memory (64 registers, no spills); one otherwise
-    // (larger tiles do not fit twice, and smaller bounds only cost registers).
-    // Three 512-thread CTAs per SM (40 registers, spills) measured slower for
-    // the y and z passes (0.37 and 0.66 ms against 0.23 and 0.44 at 512^3) and
-    // equal for the x passes.
-    static constexpr int ZMINB = (T == 512 && 2 * SMEMY <= 200 * 1024) ? 2 : 1;
-};
-
-__device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc) {
-    const unsigned dst = (unsigned)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 // ---------------------------------------------------------------- X passes
 // Each pass is a per-block body with two entry kernels: one block per tile for
 // a single mesh (BATCH = false), or, for the batched meshes of the adaptive
 // third level (BATCH = true), a resident-sized grid whose blocks loop over the
 // tiles of the meshes in use (*active, on the device).
+//
+// TL threads per line (a warp or a part of one up to 1024 / 3 * 2 points: the
+// stages then meet at warp barriers only; beyond that 64 or 128 threads at a
+// named barrier), lanes along the line: global rows are read and written in
+// full sectors.  In shared memory position p of a line lies at p + p / 8.
 template <int N>
-__device__ __forceinline__ void x_r2c_block(float2 *S, const float *__restrict__ in, float2 *__restrict__ out,
-                                            int64_t nrows, int kxp, const float2 *__restrict__ tw, int64_t vb) {
-    constexpr int L = Tile<N>::L, LP = Tile<N>::LP, T = Tile<N>::T;
-    const int64_t row0 = vb * 2 * L;
-    if constexpr (N % 4 == 0) {
-        // four x of the two rows of a line per thread (16-byte loads, 8-byte
-        // shared stores), lanes over the lines: 8 % faster than one element per
-        // thread at 512^3 (the inverse pass's matching 16-byte stores, 16 rows
-        // per warp instruction, measured 1.6x slower)
-        constexpr int Q = N / 4;
-        for (int i = threadIdx.x; i < L * Q; i += T) {
-            const int l = i % L, x = 4 * (i / L);
-            const int64_t ra = row0 + 2 * l;
-            const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-            const float4 a = ra < nrows ? __ldg(reinterpret_cast<const float4 *>(in + ra * N + x)) : z4;
-            const float4 b = ra + 1 < nrows ? __ldg(reinterpret_cast<const float4 *>(in + (ra + 1) * N + x)) : z4;
-            S[(x + 0) * LP + l] = make_float2(a.x, b.x);
-            S[(x + 1) * LP + l] = make_float2(a.y, b.y);
-            S[(x + 2) * LP + l] = make_float2(a.z, b.z);
-            S[(x + 3) * LP + l] = make_float2(a.w, b.w);
-        }
-    } else {
-        for (int i = threadIdx.x; i < 2 * L * N; i += T) {
-            const int r = i / N, x = i % N;
-            const int64_t row = row0 + r;
-            const float v = row < nrows ? __ldg(&in[row * N + x]) : 0.0f;
-            reinterpret_cast<float *>(&S[x * LP + (r >> 1)])[r & 1] = v;
+struct XLine {
+    static constexpr int V = N % 3 == 0 ? (N == 48 || N == 12 ? 12 : 24) : (N == 32 || N == 16 ? 8 : N == 8 ? 4 : 16);
+    static constexpr int TL0 = N / V;
+    static constexpr int TL = N == 12 ? 2 : N == 24 ? 4 : TL0;
+    static constexpr int CTA = 256;
+    static constexpr int MINB = N % 3 == 0 ? 3 : 4;   // 64 registers; 80 with a radix 3
+    static constexpr int LINES = CTA / TL;
+    static constexpr int PITCH = N + N / 8;
+    static constexpr size_t SMEM = (size_t)LINES * PITCH * sizeof(float2);
+    static constexpr int R1 = radix_at(N, stages_of(N, true) - 1, true);   // radix of the paired stage
+    static constexpr int NB1 = N / R1, PAIRS = NB1 / 2 / TL;
+    static_assert(NB1 % 2 == 0 && NB1 / 2 % TL == 0, "paired butterflies deal out evenly");
+    __device__ __forceinline__ static void sync(int line) {
+        if constexpr (TL <= 32) __syncwarp();
+        else asm volatile("bar.sync %0, %1;" ::"r"(line + 1), "r"(TL) : "memory");
+    }
+};
+
+__device__ __forceinline__ int pad8(int p) { return p + (p >> 3); }
+
+// One plain stage (not the paired one) of a line: values from load or shared
+// memory, to shared memory or store.
+template <int N, bool INV, int s, class Load, class Store>
+__device__ __forceinline__ void line_stage(float2 *S, int t, int line, const float2 *__restrict__ tw, Load load,
+                                           Store store) {
+    using X = XLine<N>;
+    constexpr int R = Plan<N, INV, true>::radix(s), NB = N / R, NS = Plan<N, INV, true>::span(s), TL = X::TL;
+    constexpr int PER = (NB + TL - 1) / TL;
+    constexpr bool LAST = s + 1 == Plan<N, INV, true>::S;
+    float2 v[PER][R];
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+        const int j = t + p * TL;
+        if (NB % TL == 0 || j < NB) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[p][r] = s == 0 ? load(j + r * NB) : S[pad8(j + r * NB)];
         }
     }
-    __syncthreads();
-    fft_lines<N, L, LP, T, 1, false>(S, tw);
-    constexpr int NH = N / 2 + 1;
-    for (int i = threadIdx.x; i < L * NH; i += T) {
-        const int l = i / NH, k = i % NH;
-        const float2 z = S[k * LP + l];
-        const float2 zc = S[((N - k) % N) * LP + l];
-        const float2 A = make_float2(0.5f * (z.x + zc.x), 0.5f * (z.y - zc.y));
-        const float2 B = make_float2(0.5f * (z.y + zc.y), -0.5f * (z.x - zc.x));
-        const int64_t ra = row0 + 2 * l;
-        if (ra < nrows) out[ra * kxp + k] = A;
-        if (ra + 1 < nrows) out[(ra + 1) * kxp + k] = B;
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+        const int j = t + p * TL;
+        if (NB % TL == 0 || j < NB) butterfly<N, INV, true, s>(v[p], j, tw);
+    }
+    if (!LAST && s > 0) X::sync(line);
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+        const int j = t + p * TL;
+        if (NB % TL == 0 || j < NB) {
+            const int base = (j / NS) * NS * R + j % NS;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if constexpr (LAST) store(base + r * NS, v[p][r]);
+                else S[pad8(base + r * NS)] = v[p][r];
+            }
+        }
+    }
+    if (!LAST) X::sync(line);
+}
+
+template <int N, bool INV, int s, int END, class Load, class Store>
+__device__ __forceinline__ void line_stages(float2 *S, int t, int line, const float2 *__restrict__ tw, Load load,
+                                            Store store) {
+    if constexpr (s < END) {
+        line_stage<N, INV, s>(S, t, line, tw, load, store);
+        line_stages<N, INV, s + 1, END>(S, t, line, tw, load, store);
+    }
+}
+
+template <int N>
+__device__ __forceinline__ void x_r2c_block(float2 *smem, const float *__restrict__ in, float2 *__restrict__ out,
+                                            int64_t nlines, int kxp, const float2 *__restrict__ tw, int64_t vb) {
+    using X = XLine<N>;
+    constexpr int R = X::R1, NB = X::NB1, TL = X::TL, LAST = Plan<N, false, true>::S - 1;
+    const int line = threadIdx.x / TL, t = threadIdx.x % TL;
+    const int64_t want = vb * X::LINES + line, l = want < nlines ? want : nlines - 1;   // spare threads repeat the last
+    const float *a = in + 2 * l * N, *b = a + N;
+    float2 *S = smem + line * X::PITCH;
+    line_stages<N, false, 0, LAST>(S, t, line, tw, [&](int x) { return make_float2(__ldg(&a[x]), __ldg(&b[x])); },
+                                   [](int, float2) {});
+    float2 *A = out + 2 * l * kxp, *B = A + kxp;
+#pragma unroll
+    for (int i = 0; i < X::PAIRS; ++i) {
+        // butterflies q and NB - q (0 and NB / 2): outputs k = q + r NB and their conjugates' n - k
+        const int q = t + i * TL, jb = q ? NB - q : NB / 2;
+        float2 va[R], vb2[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            va[r] = S[pad8(q + r * NB)];
+            vb2[r] = S[pad8(jb + r * NB)];
+        }
+        butterfly<N, false, true, LAST>(va, q, tw);
+        butterfly<N, false, true, LAST>(vb2, jb, tw);
+        auto split = [&](int k, float2 z, float2 zc) {
+            A[k] = make_float2(0.5f * (z.x + zc.x), 0.5f * (z.y - zc.y));
+            B[k] = make_float2(0.5f * (z.y + zc.y), -0.5f * (z.x - zc.x));
+        };
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float2 ca = q ? vb2[R - 1 - r] : va[(R - r) % R], cb = q ? va[R - 1 - r] : vb2[R - 1 - r];
+            if (q + r * NB <= N / 2) split(q + r * NB, va[r], ca);
+            if (jb + r * NB <= N / 2) split(jb + r * NB, vb2[r], cb);
+        }
+    }
+}
+
+template <int N>
+__device__ __forceinline__ void x_c2r_block(float2 *smem, const float2 *__restrict__ in, float *__restrict__ out,
+                                            int64_t nlines, int kxp, const float2 *__restrict__ tw, int64_t vb) {
+    using X = XLine<N>;
+    constexpr int R = X::R1, NB = X::NB1, TL = X::TL;
+    const int line = threadIdx.x / TL, t = threadIdx.x % TL;
+    const int64_t want = vb * X::LINES + line, l = want < nlines ? want : nlines - 1;
+    const float2 *A = in + 2 * l * kxp, *B = A + kxp;
+    float2 *S = smem + line * X::PITCH;
+#pragma unroll
+    for (int i = 0; i < X::PAIRS; ++i) {
+        const int q = t + i * TL, jb = q ? NB - q : NB / 2;
+        float2 va[R], vb2[R];
+        // Z[k] = A + iB and Z[n - k] = conj(A) + i conj(B) of every k <= n/2 that q or NB - q holds
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int ka = q + r * NB, kb = jb + r * NB;
+            if (ka <= N / 2) {
+                float2 x = A[ka], y = B[ka];
+                if (ka == 0 || ka == N / 2) x.y = y.y = 0.0f;
+                const float2 z = make_float2(x.x - y.y, x.y + y.x), zc = make_float2(x.x + y.y, y.x - x.y);
+                va[r] = z;
+                if (q) vb2[R - 1 - r] = zc;
+                else if (ka != 0 && ka != N / 2) va[(R - r) % R] = zc;
+            }
+            if (kb <= N / 2) {
+                float2 x = A[kb], y = B[kb];
+                if (kb == N / 2) x.y = y.y = 0.0f;
+                const float2 z = make_float2(x.x - y.y, x.y + y.x), zc = make_float2(x.x + y.y, y.x - x.y);
+                vb2[r] = z;
+                if (q) va[R - 1 - r] = zc;
+                else if (kb != N / 2) vb2[R - 1 - r] = zc;
+            }
+        }
+        Dft<R, true>::run(va);
+        Dft<R, true>::run(vb2);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {   // the first stage of the inverse: span 1
+            S[pad8(q * R + r)] = va[r];
+            S[pad8(jb * R + r)] = vb2[r];
+        }
+    }
+    X::sync(line);
+    float *a = out + 2 * l * N, *b = a + N;
+    line_stages<N, true, 1, Plan<N, true, true>::S>(S, t, line, tw, [](int) { return make_float2(0.f, 0.f); },
+                                              [&](int x, float2 v) {
+                                                  a[x] = v.x;
+                                                  b[x] = v.y;
+                                              });
+}
+
+template <int N, bool BATCH>
+__global__ void __launch_bounds__(XLine<N>::CTA, XLine<N>::MINB) fft_x_r2c(const float *__restrict__ in, float2 *__restrict__ out,
+                                                              int64_t nlines, int kxp, const float2 *__restrict__ tw,
+                                                              const int *__restrict__ active) {
+    extern __shared__ __align__(16) float2 S[];
+    if constexpr (BATCH) {
+        nlines = (int64_t)*active * N * N / 2;
+        for (int64_t vb = blockIdx.x; vb * XLine<N>::LINES < nlines; vb += gridDim.x) {
+            x_r2c_block<N>(S, in, out, nlines, kxp, tw, vb);
+            __syncthreads();
+        }
+    } else {
+        x_r2c_block<N>(S, in, out, nlines, kxp, tw, blockIdx.x);
     }
 }
 
 template <int N, bool BATCH>
-__global__ void __launch_bounds__(Tile<N>::T) fft_x_r2c(const float *__restrict__ in, float2 *__restrict__ out,
-                                                       int64_t nrows, int kxp, const float2 *__restrict__ tw,
-                                                       const int *__restrict__ active) {
-    extern __shared__ float2 S[];
+__global__ void __launch_bounds__(XLine<N>::CTA, XLine<N>::MINB) fft_x_c2r(const float2 *__restrict__ in, float *__restrict__ out,
+                                                              int64_t nlines, int kxp, const float2 *__restrict__ tw,
+                                                              const int *__restrict__ active) {
+    extern __shared__ __align__(16) float2 S[];
     if constexpr (BATCH) {
-        constexpr int L = Tile<N>::L;
-        const int64_t nvb = ((int64_t)*active * N * N + 2 * L - 1) / (2 * L);
-        for (int64_t vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
-            x_r2c_block<N>(S, in, out, nrows, kxp, tw, vb);
+        nlines = (int64_t)*active * N * N / 2;
+        for (int64_t vb = blockIdx.x; vb * XLine<N>::LINES < nlines; vb += gridDim.x) {
+            x_c2r_block<N>(S, in, out, nlines, kxp, tw, vb);
             __syncthreads();
         }
     } else {
-        x_r2c_block<N>(S, in, out, nrows, kxp, tw, blockIdx.x);
-    }
-}
-
-template <int N>
-__device__ __forceinline__ void x_c2r_block(float2 *S, const float2 *__restrict__ in, float *__restrict__ out,
-                                            int64_t nrows, int kxp, const float2 *__restrict__ tw, int64_t vb) {
-    constexpr int L = Tile<N>::L, LP = Tile<N>::LP, T = Tile<N>::T;
-    const int64_t row0 = vb * 2 * L;
-    constexpr int NH = N / 2 + 1;
-    for (int i = threadIdx.x; i < L * NH; i += T) {
-        const int l = i / NH, k = i % NH;
-        const int64_t ra = row0 + 2 * l;
-        float2 A = ra < nrows ? in[ra * kxp + k] : make_float2(0.f, 0.f);
-        float2 B = ra + 1 < nrows ? in[(ra + 1) * kxp + k] : make_float2(0.f, 0.f);
-        if (k == 0 || k == N / 2) { A.y = 0.f; B.y = 0.f; }
-        S[k * LP + l] = make_float2(A.x - B.y, A.y + B.x);                    // A + iB
-        if (k > 0 && k < N / 2) S[(N - k) * LP + l] = make_float2(A.x + B.y, B.x - A.y);  // conj(A) + i conj(B)
-    }
-    __syncthreads();
-    fft_lines<N, L, LP, T, 1, true>(S, tw);
-    // one x of a line per thread: its two rows from one 8-byte shared load,
-    // written by two coalesced 4-byte stores
-    for (int i = threadIdx.x; i < L * N; i += T) {
-        const int l = i / N, x = i % N;
-        const int64_t ra = row0 + 2 * l;
-        const float2 v = S[x * LP + l];
-        if (ra < nrows) out[ra * N + x] = v.x;
-        if (ra + 1 < nrows) out[(ra + 1) * N + x] = v.y;
-    }
-}
-
-template <int N, bool BATCH>
-__global__ void __launch_bounds__(Tile<N>::T) fft_x_c2r(const float2 *__restrict__ in, float *__restrict__ out,
-                                                       int64_t nrows, int kxp, const float2 *__restrict__ tw,
-                                                       const int *__restrict__ active) {
-    extern __shared__ float2 S[];
-    if constexpr (BATCH) {
-        constexpr int L = Tile<N>::L;
-        const int64_t nvb = ((int64_t)*active * N * N + 2 * L - 1) / (2 * L);
-        for (int64_t vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
-            x_c2r_block<N>(S, in, out, nrows, kxp, tw, vb);
-            __syncthreads();
-        }
-    } else {
-        x_c2r_block<N>(S, in, out, nrows, kxp, tw, blockIdx.x);
+        x_c2r_block<N>(S, in, out, nlines, kxp, tw, blockIdx.x);
     }
 }
 
@@ -299,30 +512,23 @@ __global__ void __launch_bounds__(Tile<N>::T) fft_x_c2r(const float2 *__restrict
 template <int N, bool INV>
 __device__ __forceinline__ void y_block(float2 *S, float2 *__restrict__ data, int kxp, const float2 *__restrict__ tw,
                                         int64_t vb) {
-    constexpr int L = Tile<N>::L, LP = Tile<N>::LPY, T = Tile<N>::T;
-    const int tiles_x = kxp / L;
+    using TL = Tile<N, false>;
+    const int tiles_x = kxp / TL::L;
     const int tx = (int)(vb % tiles_x);
     const int64_t z = vb / tiles_x;                    // plane over all batched meshes
-    float2 *base = data + z * N * kxp + tx * L;
-    for (int i = threadIdx.x; i < N * L / 2; i += T) {
-        const int y = i / (L / 2), l2 = 2 * (i % (L / 2));
-        cp_async16(&S[y * LP + l2], &base[(int64_t)y * kxp + l2]);
-    }
-    cp_async_wait_all();
-    __syncthreads();
-    fft_lines<N, L, LP, T, 1, INV>(S, tw);
-    for (int i = threadIdx.x; i < N * L / 2; i += T) {
-        const int y = i / (L / 2), l2 = 2 * (i % (L / 2));
-        *reinterpret_cast<float4 *>(&base[(int64_t)y * kxp + l2]) = *reinterpret_cast<const float4 *>(&S[y * LP + l2]);
-    }
+    float2 *base = data + z * N * kxp + tx * TL::L;
+    tile_stages<N, false, INV, 0>(
+        S, tw, [&](int y, int line, int, int) { return tile_load<N>(&base[(int64_t)y * kxp + line]); },
+        [&](int y, int line, int, int, float2 v) { tile_store<N>(&base[(int64_t)y * kxp + line], v); });
 }
 
 template <int N, bool INV, bool BATCH>
-__global__ void __launch_bounds__(Tile<N>::T) fft_y(float2 *__restrict__ data, int kxp, const float2 *__restrict__ tw,
-                                                   const int *__restrict__ active) {
+__global__ void __launch_bounds__(Tile<N, false>::T, Tile<N, false>::MINB) fft_y(float2 *__restrict__ data, int kxp,
+                                                                   const float2 *__restrict__ tw,
+                                                                   const int *__restrict__ active) {
     extern __shared__ __align__(16) float2 S[];
     if constexpr (BATCH) {
-        const int64_t nvb = (int64_t)*active * N * (kxp / Tile<N>::L);
+        const int64_t nvb = (int64_t)*active * N * (kxp / Tile<N, false>::L);
         for (int64_t vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
             y_block<N, INV>(S, data, kxp, tw, vb);
             __syncthreads();
@@ -339,59 +545,49 @@ __global__ void __launch_bounds__(Tile<N>::T) fft_y(float2 *__restrict__ data, i
 template <int N, int GMODE>
 __device__ __forceinline__ void z_block(float2 *S, float2 *__restrict__ data, const float *__restrict__ green,
                                         int kxp, const float2 *__restrict__ tw, int64_t vb) {
-    constexpr int L = Tile<N>::L, LP = Tile<N>::LPY, T = Tile<N>::T;
+    using TL = Tile<N, true>;
+    constexpr int L = TL::L;
     const int tiles_x = kxp / L;
     const int tx = (int)(vb % tiles_x);
     const int64_t row = vb / tiles_x;                     // (mesh, ky) over all batched meshes
     const int64_t mesh = row / N;
-    const int64_t ky = row - mesh * N;
+    const int ky = (int)(row - mesh * N);
     const int64_t zstride = (int64_t)N * kxp;
-    float2 *base = data + mesh * N * zstride + ky * kxp + tx * L;
-    for (int i = threadIdx.x; i < N * L / 2; i += T) {
-        const int z = i / (L / 2), l2 = 2 * (i % (L / 2));
-        cp_async16(&S[z * LP + l2], &base[z * zstride + l2]);
-    }
-    cp_async_wait_all();
-    __syncthreads();
-    fft_lines<N, L, LP, T, 1, false>(S, tw);
-    if (GMODE != 0) {
-        const float *g = green + ky * kxp + tx * L;
-        for (int i = threadIdx.x; i < N * L / 2; i += T) {
-            const int z = i / (L / 2), l2 = 2 * (i % (L / 2));
-            float2 gv;
+    float2 *base = data + mesh * N * zstride + (int64_t)ky * kxp + tx * L;
+    auto load = [&](int z, int line, int, int) { return tile_load<N>(&base[z * zstride + line]); };
+    auto store = [&](int z, int line, int, int, float2 v) { tile_store<N>(&base[z * zstride + line], v); };
+    if constexpr (GMODE == 0) {
+        tile_stages<N, true, false, 0>(S, tw, load, store);
+    } else {
+        // the forward's last stage and the inverse's first have the same radix
+        // and positions: the values stay with their thread
+        constexpr int R = Plan<N, false, false>::radix(Plan<N, false, false>::S - 1);
+        static_assert(R == Plan<N, true, false>::radix(0), "radices reversed");
+        float2 keep[TL::template per<R>()][R];
+        tile_stages<N, true, false, 0>(S, tw, load, [&](int z, int line, int p, int r, float2 v) {
+            const int kx = tx * L + line;
+            float g;
             if (GMODE == 1) {
-                gv = __ldg(reinterpret_cast<const float2 *>(&g[z * zstride + l2]));
+                g = __ldg(&green[(int64_t)z * zstride + (int64_t)ky * kxp + kx]);
             } else if (GMODE == 3) {
-                const int zf = z <= N / 2 ? z : N - z, kyf = ky <= N / 2 ? (int)ky : N - (int)ky;
-                gv = __ldg(reinterpret_cast<const float2 *>(
-                    &green[((int64_t)zf * (N / 2 + 1) + kyf) * kxp + tx * L + l2]));
-            } else {
-                const int kx = tx * L + l2;   // padding columns (kx > N/2) hold zeros
-                gv.x = kx <= N / 2 ? __ldg(&green[green_index(kx, (int)ky, z, N)]) : 0.0f;
-                gv.y = kx + 1 <= N / 2 ? __ldg(&green[green_index(kx + 1, (int)ky, z, N)]) : 0.0f;
+                const int zf = z <= N / 2 ? z : N - z, kyf = ky <= N / 2 ? ky : N - ky;
+                g = __ldg(&green[((int64_t)zf * (N / 2 + 1) + kyf) * kxp + kx]);
+            } else {   // padding columns (kx > N/2) hold zeros
+                g = kx <= N / 2 ? __ldg(&green[green_index(kx, ky, z, N)]) : 0.0f;
             }
-            float4 v = *reinterpret_cast<const float4 *>(&S[z * LP + l2]);
-            v.x *= gv.x;
-            v.y *= gv.x;
-            v.z *= gv.y;
-            v.w *= gv.y;
-            *reinterpret_cast<float4 *>(&S[z * LP + l2]) = v;
-        }
-        __syncthreads();
-        fft_lines<N, L, LP, T, 1, true>(S, tw);
-    }
-    for (int i = threadIdx.x; i < N * L / 2; i += T) {
-        const int z = i / (L / 2), l2 = 2 * (i % (L / 2));
-        *reinterpret_cast<float4 *>(&base[z * zstride + l2]) = *reinterpret_cast<const float4 *>(&S[z * LP + l2]);
+            keep[p][r] = make_float2(v.x * g, v.y * g);
+        });
+        __syncthreads();   // the inverse's first exchange overwrites what the forward's last stage has read
+        tile_stages<N, true, true, 0>(S, tw, [&](int, int, int p, int r) { return keep[p][r]; }, store);
     }
 }
 
 template <int N, int GMODE, bool BATCH>
-__global__ void __launch_bounds__(Tile<N>::T, Tile<N>::ZMINB) fft_z(float2 *__restrict__ data, const float *__restrict__ green,
+__global__ void __launch_bounds__(Tile<N, true>::T, Tile<N, true>::MINB) fft_z(float2 *__restrict__ data, const float *__restrict__ green,
                                                    int kxp, const float2 *__restrict__ tw, const int *__restrict__ active) {
     extern __shared__ __align__(16) float2 S[];
     if constexpr (BATCH) {
-        const int64_t nvb = (int64_t)*active * N * (kxp / Tile<N>::L);
+        const int64_t nvb = (int64_t)*active * N * (kxp / Tile<N, true>::L);
         for (int64_t vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
             z_block<N, GMODE>(S, data, green, kxp, tw, vb);
             __syncthreads();
@@ -414,47 +610,47 @@ template <int N>
 struct Launcher {
     template <bool B>
     static cudaError_t forward_v(cube2_ctx *ctx, Level &Lv) {
-        const int64_t nrows = (int64_t)Lv.batch * N * N;
-        const unsigned bx = pass_grid(ctx, Lv, (nrows + 2 * Tile<N>::L - 1) / (2 * Tile<N>::L));
+        const int64_t nlines = (int64_t)Lv.batch * N * N / 2;
+        const unsigned bx = pass_grid(ctx, Lv, (nlines + XLine<N>::LINES - 1) / XLine<N>::LINES);
         {
             ProfScope prof(ctx, B ? -1 : P_FFT_X_FWD, Lv.index);   // batched meshes: profiled as one group by the caller
-            fft_x_r2c<N, B><<<bx, Tile<N>::T, Tile<N>::SMEM, ctx->stream>>>(Lv.real, Lv.spec, nrows, Lv.kxp, Lv.tw,
+            fft_x_r2c<N, B><<<bx, XLine<N>::CTA, XLine<N>::SMEM, ctx->stream>>>(Lv.real, Lv.spec, nlines, Lv.kxp, Lv.tw,
                                                                             Lv.active);
         }
-        const unsigned by = pass_grid(ctx, Lv, (int64_t)Lv.batch * N * (Lv.kxp / Tile<N>::L));
+        const unsigned by = pass_grid(ctx, Lv, (int64_t)Lv.batch * N * (Lv.kxp / Tile<N, false>::L));
         {
             ProfScope prof(ctx, B ? -1 : P_FFT_Y_FWD, Lv.index);
-            fft_y<N, false, B><<<by, Tile<N>::T, Tile<N>::SMEMY, ctx->stream>>>(Lv.spec, Lv.kxp, Lv.tw, Lv.active);
+            fft_y<N, false, B><<<by, Tile<N, false>::T, Tile<N, false>::SMEM, ctx->stream>>>(Lv.spec, Lv.kxp, Lv.tw, Lv.active);
         }
         ctx->launches += 2;
         return cudaGetLastError();
     }
     template <bool B>
     static cudaError_t z_pass_v(cube2_ctx *ctx, Level &Lv, bool green) {
-        const unsigned bz = pass_grid(ctx, Lv, (int64_t)Lv.batch * N * (Lv.kxp / Tile<N>::L));
+        const unsigned bz = pass_grid(ctx, Lv, (int64_t)Lv.batch * N * (Lv.kxp / Tile<N, true>::L));
         ProfScope prof(ctx, B ? -1 : P_FFT_Z_GREEN, Lv.index);
         if (green && !B && Lv.green2)
-            fft_z<N, 3, false><<<bz, Tile<N>::T, Tile<N>::SMEMY, ctx->stream>>>(Lv.spec, Lv.green2, Lv.kxp, Lv.tw,
+            fft_z<N, 3, false><<<bz, Tile<N, true>::T, Tile<N, true>::SMEM, ctx->stream>>>(Lv.spec, Lv.green2, Lv.kxp, Lv.tw,
                                                                               Lv.active);
         else if (green)
-            fft_z<N, 2, B><<<bz, Tile<N>::T, Tile<N>::SMEMY, ctx->stream>>>(Lv.spec, Lv.green, Lv.kxp, Lv.tw, Lv.active);
+            fft_z<N, 2, B><<<bz, Tile<N, true>::T, Tile<N, true>::SMEM, ctx->stream>>>(Lv.spec, Lv.green, Lv.kxp, Lv.tw, Lv.active);
         else
-            fft_z<N, 0, B><<<bz, Tile<N>::T, Tile<N>::SMEMY, ctx->stream>>>(Lv.spec, nullptr, Lv.kxp, Lv.tw, Lv.active);
+            fft_z<N, 0, B><<<bz, Tile<N, true>::T, Tile<N, true>::SMEM, ctx->stream>>>(Lv.spec, nullptr, Lv.kxp, Lv.tw, Lv.active);
         ctx->launches += 1;
         return cudaGetLastError();
     }
     template <bool B>
     static cudaError_t inverse_v(cube2_ctx *ctx, Level &Lv) {
-        const unsigned by = pass_grid(ctx, Lv, (int64_t)Lv.batch * N * (Lv.kxp / Tile<N>::L));
+        const unsigned by = pass_grid(ctx, Lv, (int64_t)Lv.batch * N * (Lv.kxp / Tile<N, false>::L));
         {
             ProfScope prof(ctx, B ? -1 : P_FFT_Y_INV, Lv.index);
-            fft_y<N, true, B><<<by, Tile<N>::T, Tile<N>::SMEMY, ctx->stream>>>(Lv.spec, Lv.kxp, Lv.tw, Lv.active);
+            fft_y<N, true, B><<<by, Tile<N, false>::T, Tile<N, false>::SMEM, ctx->stream>>>(Lv.spec, Lv.kxp, Lv.tw, Lv.active);
         }
-        const int64_t nrows = (int64_t)Lv.batch * N * N;
-        const unsigned bx = pass_grid(ctx, Lv, (nrows + 2 * Tile<N>::L - 1) / (2 * Tile<N>::L));
+        const int64_t nlines = (int64_t)Lv.batch * N * N / 2;
+        const unsigned bx = pass_grid(ctx, Lv, (nlines + XLine<N>::LINES - 1) / XLine<N>::LINES);
         {
             ProfScope prof(ctx, B ? -1 : P_FFT_X_INV, Lv.index);
-            fft_x_c2r<N, B><<<bx, Tile<N>::T, Tile<N>::SMEM, ctx->stream>>>(Lv.spec, Lv.real, nrows, Lv.kxp, Lv.tw,
+            fft_x_c2r<N, B><<<bx, XLine<N>::CTA, XLine<N>::SMEM, ctx->stream>>>(Lv.spec, Lv.real, nlines, Lv.kxp, Lv.tw,
                                                                             Lv.active);
         }
         ctx->launches += 2;
@@ -483,9 +679,9 @@ struct Launcher {
     }
     template <bool B>
     static void setup_v() {
-        const int smem = (int)Tile<N>::SMEM;
-        cudaFuncSetAttribute(fft_x_r2c<N, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaFuncSetAttribute(fft_x_c2r<N, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        const int smem = (int)std::max(Tile<N, false>::SMEM, Tile<N, true>::SMEM), xmem = (int)XLine<N>::SMEM;
+        cudaFuncSetAttribute(fft_x_r2c<N, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, xmem);
+        cudaFuncSetAttribute(fft_x_c2r<N, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, xmem);
         cudaFuncSetAttribute(fft_y<N, false, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         cudaFuncSetAttribute(fft_y<N, true, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         cudaFuncSetAttribute(fft_z<N, 0, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -495,8 +691,8 @@ struct Launcher {
         static bool done = false;
         if (done) return;
         setup_v<false>();
-        cudaFuncSetAttribute(fft_z<N, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Tile<N>::SMEM);
-        cudaFuncSetAttribute(fft_z<N, 3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Tile<N>::SMEM);
+        cudaFuncSetAttribute(fft_z<N, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Tile<N, true>::SMEM);
+        cudaFuncSetAttribute(fft_z<N, 3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Tile<N, true>::SMEM);
         if constexpr (N <= BATCH_MAX_N) setup_v<true>();
         done = true;
     }
@@ -539,6 +735,14 @@ cudaError_t dispatch(cube2_ctx *ctx, Level &Lv, Op op) {
 }
 
 }  // namespace
+
+int64_t fft_twiddle_entries(int n) { return twiddle_entries(n); }
+
+cudaError_t launch_init_twiddles(cube2_ctx *ctx, Level &L) {
+    twiddle_rows_kernel<<<(twiddle_entries(L.n) + 255) / 256, 256, 0, ctx->stream>>>(L.tw, L.n);
+    ctx->launches++;
+    return cudaGetLastError();
+}
 
 bool fft_size_supported(int n) {
     switch (n) {
@@ -583,7 +787,7 @@ constexpr int NOALLOC_KXP = ((NOALLOC_MAX_N / 2 + 1) + 15) / 16 * 16;
 constexpr size_t NOALLOC_HALF = (size_t)NOALLOC_MAX_N * NOALLOC_MAX_N * NOALLOC_KXP;
 constexpr size_t NOALLOC_SPEC_BYTES = NOALLOC_HALF * sizeof(float2);
 constexpr size_t NOALLOC_GREEN_BYTES = NOALLOC_HALF * sizeof(float);
-constexpr size_t NOALLOC_BYTES = NOALLOC_SPEC_BYTES + NOALLOC_GREEN_BYTES + NOALLOC_MAX_N * sizeof(float2);
+constexpr size_t NOALLOC_BYTES = NOALLOC_SPEC_BYTES + NOALLOC_GREEN_BYTES + twiddle_entries(NOALLOC_MAX_N) * sizeof(float2);
 
 // Working memory of every cube2_solve_pm_noalloc call on a device (15.7 MB).
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_BYTES];
@@ -592,27 +796,20 @@ constexpr int NOALLOC_MAX_DEVICES = 64;
 std::mutex g_noalloc_mutex;
 void *g_noalloc_ptr[NOALLOC_MAX_DEVICES] = {};
 
-__global__ void noalloc_twiddle_kernel(float2 *tw, int n) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    double s, c;
-    sincospi(-2.0 * (double)k / (double)n, &s, &c);
-    tw[k] = make_float2((float)c, (float)s);
-}
-
 template <int N>
 cudaError_t noalloc_passes(const float *rho, float2 *spec, const float *gpad, float *phi, const float2 *tw, int kxp,
                            cudaStream_t st) {
     Launcher<N>::setup();
-    constexpr int L = Tile<N>::L;
-    const int64_t nrows = (int64_t)N * N;
-    const unsigned bx = (unsigned)((nrows + 2 * L - 1) / (2 * L));
+    constexpr int L = Tile<N, true>::L;
+    static_assert(L == Tile<N, false>::L, "one grid for y and z");
+    const int64_t nlines = (int64_t)N * N / 2;
+    const unsigned bx = (unsigned)((nlines + XLine<N>::LINES - 1) / XLine<N>::LINES);
     const unsigned by = (unsigned)((int64_t)N * (kxp / L));
-    fft_x_r2c<N, false><<<bx, Tile<N>::T, Tile<N>::SMEM, st>>>(rho, spec, nrows, kxp, tw, nullptr);
-    fft_y<N, false, false><<<by, Tile<N>::T, Tile<N>::SMEMY, st>>>(spec, kxp, tw, nullptr);
-    fft_z<N, 1, false><<<by, Tile<N>::T, Tile<N>::SMEMY, st>>>(spec, gpad, kxp, tw, nullptr);
-    fft_y<N, true, false><<<by, Tile<N>::T, Tile<N>::SMEMY, st>>>(spec, kxp, tw, nullptr);
-    fft_x_c2r<N, false><<<bx, Tile<N>::T, Tile<N>::SMEM, st>>>(spec, phi, nrows, kxp, tw, nullptr);
+    fft_x_r2c<N, false><<<bx, XLine<N>::CTA, XLine<N>::SMEM, st>>>(rho, spec, nlines, kxp, tw, nullptr);
+    fft_y<N, false, false><<<by, Tile<N, false>::T, Tile<N, false>::SMEM, st>>>(spec, kxp, tw, nullptr);
+    fft_z<N, 1, false><<<by, Tile<N, true>::T, Tile<N, true>::SMEM, st>>>(spec, gpad, kxp, tw, nullptr);
+    fft_y<N, true, false><<<by, Tile<N, false>::T, Tile<N, false>::SMEM, st>>>(spec, kxp, tw, nullptr);
+    fft_x_c2r<N, false><<<bx, XLine<N>::CTA, XLine<N>::SMEM, st>>>(spec, phi, nlines, kxp, tw, nullptr);
     return cudaGetLastError();
 }
 
@@ -674,7 +871,7 @@ extern "C" int cube2_solve_pm_noalloc(const float *rho, const float *green, floa
     if (e == cudaSuccess && (size_t)kxp > nh)
         e = cudaMemset2DAsync(gpad + nh, kxp * sizeof(float), 0, (kxp - nh) * sizeof(float), (size_t)n * n, st);
     if (e == cudaSuccess) {
-        noalloc_twiddle_kernel<<<(n + 127) / 128, 128, 0, st>>>(tw, n);
+        twiddle_rows_kernel<<<(twiddle_entries(n) + 127) / 128, 128, 0, st>>>(tw, n);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) {

@@ -1,5 +1,5 @@
-// Optimised Green's function of one PM level, Eq. (Gk) of the paper (Sec. 2.1.2),
-// and the FFT twiddle tables.  FP64 arithmetic on the GPU, FP32 result.
+// Optimised Green's function of one PM level, Eq. (Gk) of the paper (Sec. 2.1.2).
+// FP64 arithmetic on the GPU, FP32 result.
 //
 // For a mode k = 2 pi m / n (m_d in (-n/2, n/2]) the kernel forms
 //   d_d   = 4/3 sin k_d - 1/6 sin 2k_d                     (Eq. diff, D = i d)
@@ -143,21 +143,7 @@ __global__ void green_fold_kernel(const float *__restrict__ G, float *__restrict
     out[idx] = kx <= n / 2 ? G[green_index(kx, ky, kz, n)] : 0.0f;
 }
 
-__global__ void twiddle_kernel(float2 *tw, int n) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    double s, c;
-    sincospi(-2.0 * (double)k / (double)n, &s, &c);
-    tw[k] = make_float2((float)c, (float)s);
-}
-
 }  // namespace
-
-cudaError_t launch_init_twiddles(cube2_ctx *ctx, Level &L) {
-    twiddle_kernel<<<(L.n + 255) / 256, 256, 0, ctx->stream>>>(L.tw, L.n);
-    ctx->launches++;
-    return cudaGetLastError();
-}
 
 cudaError_t launch_green_expand(cube2_ctx *ctx, const Level &L, float *out) {
     const int64_t total = (int64_t)L.n * L.n * (L.n / 2 + 1);
