@@ -9,12 +9,15 @@
 //                   (atomic: a provisional, order-dependent rank in the cell)
 //   2. scan       : nstart = exclusive prefix sum of ncount (multi-level)
 //   3. scatter    : perm[nstart[cell] + slot] = old index
-//   4. sort       : every cell's perm segment sorted by old index, which makes
-//                   the result stable and independent of the atomics' order:
-//                   cells of <= 32 particles by one thread (insertion sort),
-//                   larger ones by a CTA (bitonic in shared memory up to 8192,
-//                   beyond that sorted 8192-runs merged through global scratch)
-//   5. gather     : off, vel, cellid of new index i from old index perm[i]
+//   4. sort       : cells of more than RANK_MAX particles get their perm segment
+//                   sorted by old index: up to 1024 by a warp, larger ones by a
+//                   CTA (bitonic in shared memory up to 8192, beyond that sorted
+//                   8192-runs merged through global scratch)
+//   5. gather     : off, vel, cellid and the map of each new index from its old
+//                   one.  In a cell of up to RANK_MAX particles the new index is
+//                   the start plus the number of smaller old indices in the
+//                   segment, which makes the result stable and independent of
+//                   the atomics' order without sorting it first.
 //   6. ncount/nstart copied into the caller's count/start
 #include "common.cuh"
 
@@ -22,6 +25,23 @@
 
 namespace cube2 {
 namespace {
+
+// A place in each lane's cell.  Particles come in cell order and most stay in
+// their cell or move with their neighbours: one atomic per run of lanes with the
+// same cell (256^3 run's kick and drift at z = 0 / 1 / 49: 0.31 / 0.27 / 0.19 -> 0.23 / 0.22
+// / 0.20 ms; one per distinct cell by __match_any_sync: 0.21 / 0.23 / 0.35).  mask: the
+// warp's lanes with a particle, from lane 0 on.
+__device__ __forceinline__ int take_slot(int32_t *count, int cell, unsigned mask) {
+    const int lane = threadIdx.x & 31;
+    const int before = __shfl_up_sync(mask, cell, 1);
+    const unsigned heads = __ballot_sync(mask, lane == 0 || before != cell);
+    const int head = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+    const unsigned later = heads & ~(0xffffffffu >> (31 - head));   // heads after this run's
+    const int end = later ? __ffs(later) - 1 : __popc(mask);
+    int base = 0;
+    if (lane == head) base = atomicAdd(&count[cell], end - head);
+    return __shfl_sync(mask, base, head) + lane - head;
+}
 
 constexpr int SCAN_THREADS = 512;
 constexpr int SCAN_ITEMS = 8;
@@ -57,6 +77,7 @@ struct DriftParams {
 
 __global__ void __launch_bounds__(256) kick_drift_kernel(DriftParams P) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned mask = __ballot_sync(0xffffffffu, i < P.N);
     if (i >= P.N) return;
     const int n = P.n_ios;
     const int c = P.cellid[i];
@@ -90,7 +111,7 @@ __global__ void __launch_bounds__(256) kick_drift_kernel(DriftParams P) {
     }
     if (bad) set_status(P.status, isfinite(v[0] + v[1] + v[2]) ? ST_DISPLACEMENT : ST_NONFINITE);
     const int cell = (nc[2] * n + nc[1]) * n + nc[0];
-    const int slot = atomicAdd(&P.count[cell], 1);
+    const int slot = take_slot(P.count, cell, mask);
     P.toff[i] = no[0];
     P.toff[P.N + i] = no[1];
     P.toff[2 * P.N + i] = no[2];
@@ -216,38 +237,32 @@ __global__ void scatter_kernel(const int32_t *tcell, const int32_t *tslot, const
     perm[start[tcell[i]] + tslot[i]] = (int32_t)i;
 }
 
-// Sort each cell's segment of perm ascending (old index = stable order).  One
-// thread per cell sorts segments of up to 32 by insertion; cells of up to
-// WARP_SORT are listed from the front of `big` for sort_mid_kernel (one warp
-// per cell), larger ones from the back for sort_big_kernel (one CTA per cell).
-constexpr int SMALL_SORT = 32;
-constexpr int WARP_SORT = 1024;
-constexpr int MID_WARPS = 8;
+// Cells of more than RANK_MAX particles, whose segments are sorted ascending
+// (old index = stable order): up to WARP_SORT from the front of `big` (one warp
+// per cell), larger ones from the back (one CTA per cell: a warp takes 80 us for a
+// cell of 1000, which the whole step of a small box waits for).  Ranking in the
+// gather costs reads of cached slots and scales with a cell's square; at 160 the
+// 256^3 run at z = 0 takes 0.34 ms there and 0.124 here, at 96 0.33 and 0.153, at
+// 48 0.33 and 0.195.  512 threads: one cell of some thousands costs a 64^3 box
+// 0.033 ms (256: 0.052, 1024: 0.025), the many of the 256^3 run 0.124 (0.128, 0.197).
+constexpr int RANK_MAX = 160;
+constexpr int WARP_SORT = 256;
+constexpr int SORT_THREADS = 512, SORT_WARPS = SORT_THREADS / 32;
 constexpr int BIG_SORT_SMEM = 8192;
-constexpr int BIG_SORT_THREADS = 512;
 
-__global__ void sort_small_kernel(const int32_t *count, const int32_t *start, int32_t *perm, int64_t n_cells,
-                                  int32_t *big, int *big_n) {
-    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n_cells) return;
-    const int cnt = count[c];
-    if (cnt < 2) return;
-    if (cnt > SMALL_SORT) {
-        if (cnt <= WARP_SORT)
-            big[atomicAdd(&big_n[0], 1)] = (int32_t)c;
-        else
-            big[n_cells - 1 - atomicAdd(&big_n[1], 1)] = (int32_t)c;
-        return;
-    }
-    int32_t *seg = perm + start[c];
-    for (int a = 1; a < cnt; ++a) {
-        const int32_t key = seg[a];
-        int b = a - 1;
-        while (b >= 0 && seg[b] > key) {
-            seg[b + 1] = seg[b];
-            --b;
-        }
-        seg[b + 1] = key;
+__global__ void __launch_bounds__(256) sort_list_kernel(const int32_t *__restrict__ count, int64_t n_cells, int32_t *big,
+                                                        int *big_n) {
+    const int64_t c0 = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+    int4 v = make_int4(0, 0, 0, 0);
+    if (c0 + 3 < n_cells) v = __ldg(reinterpret_cast<const int4 *>(count + c0));
+    else
+        for (int k = 0; c0 + k < n_cells && k < 4; ++k) (&v.x)[k] = count[c0 + k];
+    if (max(max(v.x, v.y), max(v.z, v.w)) <= RANK_MAX) return;
+    for (int k = 0; k < 4; ++k) {
+        const int cnt = (&v.x)[k];
+        if (cnt <= RANK_MAX) continue;
+        if (cnt <= WARP_SORT) big[atomicAdd(&big_n[0], 1)] = (int32_t)(c0 + k);
+        else big[n_cells - 1 - atomicAdd(&big_n[1], 1)] = (int32_t)(c0 + k);
     }
 }
 
@@ -296,50 +311,40 @@ __device__ void merge_runs(const int32_t *a, int la, const int32_t *b, int lb, i
     }
 }
 
-// Cells of 33 .. WARP_SORT particles: one warp per cell, a bitonic sort of the
-// segment (padded to a power of two) in the warp's own shared buffer, every
-// lane exchanging pairs at each stage, with warp barriers only.
-__global__ void __launch_bounds__(MID_WARPS * 32) sort_mid_kernel(const int32_t *count, const int32_t *start,
-                                                                 int32_t *perm, const int32_t *big,
-                                                                 const int *big_n) {
-    __shared__ int32_t buf[MID_WARPS][WARP_SORT];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int32_t *s = buf[w];
-    const int total = big_n[0];
-    for (int item = blockIdx.x * MID_WARPS + w; item < total; item += gridDim.x * MID_WARPS) {
-        const int64_t c = big[item];
-        const int n = count[c];
-        int32_t *seg = perm + start[c];
-        int np2 = 64;
-        while (np2 < n) np2 <<= 1;
-        for (int i = lane; i < np2; i += 32) s[i] = i < n ? seg[i] : 0x7fffffff;
-        __syncwarp();
-        for (int k = 2; k <= np2; k <<= 1)
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                for (int q = lane; q < (np2 >> 1); q += 32) {
-                    const int i = ((q & ~(j - 1)) << 1) | (q & (j - 1));   // lower index of pair q
-                    const int ixj = i | j;
-                    const bool up = (i & k) == 0;
-                    const int32_t a = s[i], b = s[ixj];
-                    if ((a > b) == up) {
-                        s[i] = b;
-                        s[ixj] = a;
-                    }
+// One cell of up to WARP_SORT particles by a warp: a bitonic sort of the segment
+// (padded to a power of two) in the warp's own shared buffer, every lane
+// exchanging pairs at each stage, with warp barriers only.
+__device__ void sort_warp(int32_t *seg, int n, int32_t *s) {
+    const int lane = threadIdx.x & 31;
+    int np2 = 64;
+    while (np2 < n) np2 <<= 1;
+    for (int i = lane; i < np2; i += 32) s[i] = i < n ? seg[i] : 0x7fffffff;
+    __syncwarp();
+    for (int k = 2; k <= np2; k <<= 1)
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            for (int q = lane; q < (np2 >> 1); q += 32) {
+                const int i = ((q & ~(j - 1)) << 1) | (q & (j - 1));   // lower index of pair q
+                const int ixj = i | j;
+                const bool up = (i & k) == 0;
+                const int32_t a = s[i], b = s[ixj];
+                if ((a > b) == up) {
+                    s[i] = b;
+                    s[ixj] = a;
                 }
-                __syncwarp();
             }
-        for (int i = lane; i < n; i += 32) seg[i] = s[i];
-        __syncwarp();
-    }
+            __syncwarp();
+        }
+    for (int i = lane; i < n; i += 32) seg[i] = s[i];
+    __syncwarp();
 }
 
-__global__ void __launch_bounds__(BIG_SORT_THREADS) sort_big_kernel(const int32_t *count, const int32_t *start,
-                                                                    int32_t *perm, int32_t *perm2,
-                                                                    const int32_t *big, const int *big_n,
-                                                                    int64_t n_cells) {
+__global__ void __launch_bounds__(SORT_THREADS) sort_cells_kernel(const int32_t *count, const int32_t *start,
+                                                                  int32_t *perm, int32_t *scratch, const int32_t *big,
+                                                                  const int *big_n, int64_t n_cells) {
     __shared__ int32_t s[BIG_SORT_SMEM];
-    const int total = big_n[1];
-    for (int item = blockIdx.x; item < total; item += gridDim.x) {
+    static_assert(SORT_WARPS * WARP_SORT <= BIG_SORT_SMEM, "a buffer per warp");
+    const int n_cta = big_n[1];
+    for (int item = blockIdx.x; item < n_cta; item += gridDim.x) {
         const int64_t c = big[n_cells - 1 - item];
         const int n = count[c];
         int32_t *seg = perm + start[c];
@@ -348,7 +353,7 @@ __global__ void __launch_bounds__(BIG_SORT_THREADS) sort_big_kernel(const int32_
             continue;
         }
         for (int r = 0; r < n; r += BIG_SORT_SMEM) sort_run_smem(seg + r, min(BIG_SORT_SMEM, n - r), s);
-        int32_t *src = seg, *dst = perm2 + start[c];
+        int32_t *src = seg, *dst = scratch + start[c];
         for (int w = BIG_SORT_SMEM; w < n; w <<= 1) {
             for (int lo = 0; lo < n; lo += 2 * w) {
                 const int la = min(w, n - lo), lb = max(0, min(w, n - lo - w));
@@ -361,10 +366,17 @@ __global__ void __launch_bounds__(BIG_SORT_THREADS) sort_big_kernel(const int32_
             for (int i = threadIdx.x; i < n; i += blockDim.x) seg[i] = src[i];
         __syncthreads();
     }
+    const int w = threadIdx.x >> 5, n_warp = big_n[0];
+    for (int item = blockIdx.x * SORT_WARPS + w; item < n_warp; item += gridDim.x * SORT_WARPS) {
+        const int64_t c = big[item];
+        sort_warp(perm + start[c], count[c], s + w * WARP_SORT);
+    }
 }
 
 struct GatherParams {
-    const int32_t *perm, *tcell;
+    const int32_t *slots;          // old index by provisional slot (scatter_kernel)
+    int32_t *perm;                 // old index by new index
+    const int32_t *tcell, *count, *start;
     const uint16_t *toff;
     const float *tvel;
     uint16_t *off0, *off1, *off2;
@@ -373,17 +385,31 @@ struct GatherParams {
     int64_t N;
 };
 
-__global__ void gather_kernel(GatherParams P) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= P.N) return;
-    const int64_t j = P.perm[i];
+// One thread per provisional slot: its place is its rank in the cell.  Bound by
+// the scattered reads of a particle's 24 bytes.  A pass of its own that sorted the
+// small segments, a thread per cell, took 0.28 ms and the gather 0.25 on the 256^3
+// run at z = 0 (512^3 at z = 1: 1.91 and 2.01); together they take 0.34 (2.63).
+__global__ void __launch_bounds__(256) gather_kernel(GatherParams P) {
+    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= P.N) return;
+    const int j = P.slots[s];
+    const int c = P.tcell[j];
+    const int cnt = __ldg(&P.count[c]);
+    int64_t i = s;
+    if (cnt > 1 && cnt <= RANK_MAX) {
+        const int st = __ldg(&P.start[c]);
+        int rank = 0;
+        for (int k = 0; k < cnt; ++k) rank += __ldg(&P.slots[st + k]) < j;
+        i = st + rank;
+    }
+    P.perm[i] = j;
     P.off0[i] = P.toff[j];
     P.off1[i] = P.toff[P.N + j];
     P.off2[i] = P.toff[2 * P.N + j];
     P.vel0[i] = P.tvel[j];
     P.vel1[i] = P.tvel[P.N + j];
     P.vel2[i] = P.tvel[2 * P.N + j];
-    P.cellid[i] = P.tcell[j];
+    P.cellid[i] = c;
 }
 
 // FP16 velocity codec: per IOS cell the FP32 scale max_p,d |v_d| (an atomic
@@ -554,26 +580,26 @@ cudaError_t launch_rebin(cube2_ctx *ctx, const cube2_particles *p) {
     if (pb > 0) {
         {
             ProfScope prof(ctx, P_SCATTER, 0);
-            scatter_kernel<<<(unsigned)pb, 256, 0, ctx->stream>>>(ctx->tcell, ctx->tslot, ctx->nstart, ctx->perm,
+            scatter_kernel<<<(unsigned)pb, 256, 0, ctx->stream>>>(ctx->tcell, ctx->tslot, ctx->nstart, ctx->perm2,
                                                                   ctx->N);
         }
         e = cudaMemsetAsync(ctx->big_n, 0, 2 * sizeof(int), ctx->stream);
         if (e != cudaSuccess) return e;
         {
             ProfScope prof(ctx, P_SORT, 0);
-            sort_small_kernel<<<(unsigned)cb, 256, 0, ctx->stream>>>(ctx->ncount, ctx->nstart, ctx->perm,
-                                                                     ctx->n_cells, ctx->big, ctx->big_n);
+            sort_list_kernel<<<(unsigned)((cb + 3) / 4), 256, 0, ctx->stream>>>(ctx->ncount, ctx->n_cells, ctx->big,
+                                                                               ctx->big_n);
         }
         {
             ProfScope prof(ctx, P_SORT_BIG, 0);
-            sort_mid_kernel<<<(unsigned)(ctx->num_sms * 6), MID_WARPS * 32, 0, ctx->stream>>>(
-                ctx->ncount, ctx->nstart, ctx->perm, ctx->big, ctx->big_n);
-            sort_big_kernel<<<(unsigned)(ctx->num_sms * 2), BIG_SORT_THREADS, 0, ctx->stream>>>(
-                ctx->ncount, ctx->nstart, ctx->perm, ctx->perm2, ctx->big, ctx->big_n, ctx->n_cells);
+            sort_cells_kernel<<<(unsigned)(ctx->num_sms * (1536 / SORT_THREADS)), SORT_THREADS, 0, ctx->stream>>>(
+                ctx->ncount, ctx->nstart, ctx->perm2, ctx->perm, ctx->big, ctx->big_n, ctx->n_cells);
         }
-        ctx->launches++;
         GatherParams G{};
+        G.slots = ctx->perm2;
         G.perm = ctx->perm;
+        G.count = ctx->ncount;
+        G.start = ctx->nstart;
         G.tcell = ctx->tcell;
         G.toff = ctx->toff;
         G.tvel = ctx->tvel;
