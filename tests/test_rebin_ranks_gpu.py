@@ -57,3 +57,33 @@ def test_order_is_the_stable_one(sizes, rest, fp16):
     assert torch.equal(p.off, before)
     ctx.check()
     ctx.close()
+
+
+@pytest.mark.parametrize("box", [6.0, 7.3, 6.0e-7, 6.0e31])
+def test_positions_round_as_fp64_division_does(box):
+    # the placement's integer quotient: halves and their neighbours, whole values,
+    # other periods and signs, zeros, the smallest values and those past 2^31
+    n = 6
+    s_ios = box / n
+    rng = np.random.default_rng(11)
+    u = np.concatenate([rng.integers(-2 ** 30, 2 ** 30, 4000) + 0.5, rng.integers(0, n * 65536, 4000) + 0.5,
+                        rng.integers(-10 ** 6, 10 ** 6, 4000), rng.uniform(-2e6, 2e6, 20000), rng.uniform(-2e12, 2e12, 4000),
+                        rng.choice([-1.0, 1.0], 4000) * 10.0 ** rng.uniform(-300, 9, 4000), np.arange(-8, 8) * 0.25])
+    x = u * (s_ios / 65536.0)
+    x = np.concatenate([x, np.nextafter(x, np.inf), np.nextafter(x, -np.inf), x + 2.0 ** -21 * s_ios, [0.0, -0.0, 5e-324]])
+    x = x[:3 * (x.size // 3)].reshape(3, -1)
+    X = np.rint(x / s_ios * 65536.0).astype(np.int64) % (n * 65536)
+    cells = (X >> 16)[0] + n * ((X >> 16)[1] + n * (X >> 16)[2])
+    order = np.argsort(cells, kind="stable")
+    w = C1.with_(name="round", n_ios=n, box=box, levels=(Level(2 * n, 0.8),), b_pp=0.05 * s_ios)
+    ctx = cube2.init_mesh(cube2.make_config(w, n_particles=x.shape[1]))
+    p, perm = cube2.ios_from_positions(ctx, torch.tensor(x, device="cuda"))
+    assert np.array_equal(perm.cpu().numpy(), order)
+    assert np.array_equal(p.off.cpu().numpy().view(np.uint16).astype(int), (X & 0xffff)[:, order])
+    ctx.check()
+    bad = torch.tensor(x, device="cuda")
+    bad[1, 7] = float("inf")
+    cube2.ios_from_positions(ctx, bad)
+    with pytest.raises(cube2.Cube2Error):
+        ctx.check()
+    ctx.close()
