@@ -120,14 +120,11 @@ void free_ctx(cube2_ctx *c) {
         cudaFree(c->lev[l].tw);
     }
     cudaFree(c->cellid);
-    cudaFree(c->toff);
-    cudaFree(c->tvel);
-    cudaFree(c->tcell);
+    cudaFree(c->moved16);
+    cudaFree(c->moved8);
     cudaFree(c->tslot);
     cudaFree(c->perm);
     cudaFree(c->scan_tmp);
-    cudaFree(c->ncount);
-    cudaFree(c->nstart);
     cudaFree(c->perm2);
     cudaFree(c->big);
     cudaFree(c->big_n);
@@ -326,13 +323,10 @@ int cube2_init_mesh(cube2_ctx **out, const cube2_config *cfg, void *stream) {
     }
     const size_t N = (size_t)c->N;
     alloc((void **)&c->cellid, N * 4);
-    alloc((void **)&c->toff, N * 3 * 2);
-    alloc((void **)&c->tvel, N * 3 * 4);
-    alloc((void **)&c->tcell, N * 4);
+    alloc((void **)&c->moved16, N * 16);
+    alloc((void **)&c->moved8, N * 8);
     alloc((void **)&c->tslot, N * 4);
     alloc((void **)&c->perm, N * 4);
-    alloc((void **)&c->ncount, (size_t)c->n_cells * 4);
-    alloc((void **)&c->nstart, (size_t)c->n_cells * 4);
     alloc((void **)&c->perm2, N * 4);
     alloc((void **)&c->big, (size_t)c->n_cells * 4);
     alloc((void **)&c->big_n, 2 * sizeof(int));
@@ -592,7 +586,7 @@ int cube2_ios_from_positions(cube2_ctx *ctx, const double *const pos[3], const f
         return set_error(ctx, CUBE2_ERR_BAD_ARG, "null position arrays");
     if (ctx->N > 0 && mom && (!mom[0] || !mom[1] || !mom[2]))
         return set_error(ctx, CUBE2_ERR_BAD_ARG, "momenta must be three arrays or null");
-    cudaError_t e = launch_place(ctx, pos, mom);
+    cudaError_t e = launch_place(ctx, pos, mom, p);
     if (e == cudaSuccess) e = launch_rebin(ctx, p);
     if (e == cudaSuccess && perm && ctx->N > 0)
         e = cudaMemcpyAsync(perm, ctx->perm, sizeof(int32_t) * (size_t)ctx->N, cudaMemcpyDeviceToDevice, ctx->stream);

@@ -101,13 +101,10 @@ struct cube2_ctx {
     double b_range = 0;      // PP range [Mpc/h] (softening of the finest level)
     // particle scratch (all [N] unless noted)
     int32_t *cellid = nullptr;
-    uint16_t *toff = nullptr;      // [3][N]
-    float *tvel = nullptr;         // [3][N]
-    int32_t *tcell = nullptr;
+    void *moved16 = nullptr;       // [N] records of the particles on the move (kdk.cu)
+    void *moved8 = nullptr;
     int32_t *tslot = nullptr;
     int32_t *perm = nullptr;
-    int32_t *ncount = nullptr;     // [n_cells] histogram of the new cells
-    int32_t *nstart = nullptr;     // [n_cells] its exclusive scan
     int32_t *perm2 = nullptr;      // [N] merge scratch of the segmented sort
     int32_t *big = nullptr;        // [n_cells] cells too large for the per-thread sort
     int *big_n = nullptr;          // [2] their numbers (up to 1024 particles, more); in PP: dense cells, target
@@ -211,7 +208,7 @@ cudaError_t launch_kick(cube2_ctx *ctx, const cube2_particles *p, float kick);
 cudaError_t launch_kick_drift(cube2_ctx *ctx, const cube2_particles *p, float kick, float drift_fix);
 cudaError_t launch_scan(cube2_ctx *ctx, const int32_t *in, int32_t *out, int64_t n);
 cudaError_t launch_rebin(cube2_ctx *ctx, const cube2_particles *p);
-cudaError_t launch_place(cube2_ctx *ctx, const double *const pos[3], const float *const mom[3]);
+cudaError_t launch_place(cube2_ctx *ctx, const double *const pos[3], const float *const mom[3], const cube2_particles *p);
 int64_t scan_scratch_len(int64_t n);
 // force vector-Jacobian product
 cudaError_t launch_vjp_gather_e(cube2_ctx *ctx, Level &L, const cube2_particles *p, const float *const v[3],

@@ -298,20 +298,57 @@ __global__ void __launch_bounds__(INTERP_THREADS) interp_kernel(InterpParams P) 
     }
 }
 
-__global__ void cellid_kernel(const int32_t *__restrict__ count, const int32_t *__restrict__ start,
-                              int32_t *__restrict__ cellid, int64_t n_cells) {
-    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n_cells) return;
-    const int s = start[c], e = s + count[c];
-    for (int p = s; p < e; ++p) cellid[p] = (int32_t)c;
+// The cell of every particle, a warp per one or four groups of 32 cells.  A group's
+// particles lie in a row: each lane takes one and finds its cell among the 32
+// starts, so that the writes are whole lines; four groups keep enough loads in
+// flight (256^3 run at z = 49 / 0: a thread per cell, writing its own particles,
+// took 0.083 / 0.116 ms, one group a warp 0.070 / 0.085, now 0.042 / 0.056).  Below
+// a warp for every slot of the chip one group each is better (64^3: 0.0104 against
+// 0.0135 ms).  More than 256 particles are written cell by cell, without the search.
+template <int CELLID_GROUPS>
+__global__ void __launch_bounds__(256) cellid_kernel(const int32_t *__restrict__ count, const int32_t *__restrict__ start,
+                                                     int32_t *__restrict__ cellid, int64_t n_cells) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warp0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - lane) * CELLID_GROUPS;
+    int cnt[CELLID_GROUPS], s[CELLID_GROUPS];
+#pragma unroll
+    for (int g = 0; g < CELLID_GROUPS; ++g) {
+        const int64_t c = warp0 + g * 32 + lane;
+        cnt[g] = c < n_cells ? count[c] : 0;
+        s[g] = c < n_cells ? start[c] : 0x7fffffff;
+    }
+#pragma unroll
+    for (int g = 0; g < CELLID_GROUPS; ++g) {
+        const int first = (int)(warp0 + g * 32);
+        const int b = __shfl_sync(0xffffffffu, s[g], 0);
+        const int total = __reduce_add_sync(0xffffffffu, cnt[g]);
+        if (total <= 256) {
+            for (int k = lane; k - lane < total; k += 32) {
+                const int i = b + k;
+                int at = 0;   // the last start that is not above i
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1)
+                    if (__shfl_sync(0xffffffffu, s[g], at + o) <= i) at += o;
+                if (k < total) cellid[i] = first + at;
+            }
+            continue;
+        }
+        for (int k = 0; k < 32; ++k) {
+            const int n = __shfl_sync(0xffffffffu, cnt[g], k), from = __shfl_sync(0xffffffffu, s[g], k);
+            for (int i = lane; i < n; i += 32) cellid[from + i] = first + k;
+        }
+    }
 }
 
 }  // namespace
 
 cudaError_t launch_cellid(cube2_ctx *ctx, const cube2_particles *p) {
-    const int64_t blocks = (ctx->n_cells + 255) / 256;
     ProfScope prof(ctx, P_CELLID, 0);
-    cellid_kernel<<<(unsigned)blocks, 256, 0, ctx->stream>>>(p->count, p->start, ctx->cellid, ctx->n_cells);
+    const bool many = ctx->n_cells >= (int64_t)ctx->num_sms * 64 * 32 * 4;
+    const int64_t per = many ? 1024 : 256;
+    const unsigned blocks = (unsigned)((ctx->n_cells + per - 1) / per);
+    if (many) cellid_kernel<4><<<blocks, 256, 0, ctx->stream>>>(p->count, p->start, ctx->cellid, ctx->n_cells);
+    else cellid_kernel<1><<<blocks, 256, 0, ctx->stream>>>(p->count, p->start, ctx->cellid, ctx->n_cells);
     ctx->launches++;
     return cudaGetLastError();
 }

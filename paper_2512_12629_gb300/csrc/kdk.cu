@@ -5,20 +5,21 @@
 // even), X_d = c_d 2^16 + off_d.  Re-bin: a stable counting sort by the new
 // cell id (ties keep the previous order) rebuilds count/start and permutes the
 // offsets and momenta, so the IOS order stays the cell list.
-//   1. kick_drift : new coordinates into scratch; slot = ncount[new cell]++
+//   1. kick_drift : new coordinates into scratch records; slot = count[new cell]++
 //                   (atomic: a provisional, order-dependent rank in the cell)
-//   2. scan       : nstart = exclusive prefix sum of ncount (multi-level)
-//   3. scatter    : perm[nstart[cell] + slot] = old index
-//   4. sort       : cells of more than RANK_MAX particles get their perm segment
-//                   sorted by old index: up to 1024 by a warp, larger ones by a
-//                   CTA (bitonic in shared memory up to 8192, beyond that sorted
-//                   8192-runs merged through global scratch)
+//   2. scan       : start = exclusive prefix sum of count (multi-level)
+//   3. scatter    : slots[start[cell] + slot] = old index
+//   4. sort       : cells of more than RANK_MAX particles get their segment of
+//                   slots sorted by old index: up to WARP_SORT by a warp, larger
+//                   ones by a CTA (bitonic in shared memory up to 8192, beyond that
+//                   sorted 8192-runs merged through global scratch)
 //   5. gather     : off, vel, cellid and the map of each new index from its old
 //                   one.  In a cell of up to RANK_MAX particles the new index is
 //                   the start plus the number of smaller old indices in the
 //                   segment, which makes the result stable and independent of
 //                   the atomics' order without sorting it first.
-//   6. ncount/nstart copied into the caller's count/start
+// The histogram and its scan are made in the caller's count and start, which the
+// step no longer reads once cellid is known.
 #include "common.cuh"
 
 #include <cuda_fp16.h>
@@ -58,6 +59,21 @@ __global__ void kick_kernel(float *v0, float *v1, float *v2, const float *a0, co
     if (!isfinite(x) || !isfinite(y) || !isfinite(z)) set_status(status, ST_NONFINITE);
 }
 
+// A particle between its old place and its new one, by old index: two records, so
+// that the gather's scattered reads touch two or three sectors and not seven (256^3
+// run at z = 49 / 0: gather 0.29 / 0.34 -> 0.18 / 0.23 ms; 512^3 2.63 -> 1.67).
+struct Moved {
+    float4 *vel_off;   // three velocities, the first two offsets in 16 bits each
+    int2 *cell_off;    // new cell, third offset
+    int32_t *slot;     // provisional slot within the cell
+
+    __device__ __forceinline__ void put(int64_t i, float vx, float vy, float vz, const uint16_t off[3], int cell, int s) const {
+        vel_off[i] = make_float4(vx, vy, vz, __uint_as_float((unsigned)off[0] | (unsigned)off[1] << 16));
+        cell_off[i] = make_int2(cell, off[2]);
+        slot[i] = s;
+    }
+};
+
 struct DriftParams {
     const uint16_t *off0, *off1, *off2;
     const float *vel0, *vel1, *vel2;
@@ -66,9 +82,7 @@ struct DriftParams {
     const float *acc0, *acc1, *acc2;
     const int32_t *cellid;
     int32_t *count;           // zeroed before the launch, receives the new histogram
-    uint16_t *toff;           // [3][N]
-    float *tvel;              // [3][N]
-    int32_t *tcell, *tslot;
+    Moved to;
     int64_t N;
     int n_ios;
     float kick, drift_fix;    // drift_fix = Dr 2^16 / s_ios
@@ -112,14 +126,7 @@ __global__ void __launch_bounds__(256) kick_drift_kernel(DriftParams P) {
     if (bad) set_status(P.status, isfinite(v[0] + v[1] + v[2]) ? ST_DISPLACEMENT : ST_NONFINITE);
     const int cell = (nc[2] * n + nc[1]) * n + nc[0];
     const int slot = take_slot(P.count, cell, mask);
-    P.toff[i] = no[0];
-    P.toff[P.N + i] = no[1];
-    P.toff[2 * P.N + i] = no[2];
-    P.tvel[i] = v[0];
-    P.tvel[P.N + i] = v[1];
-    P.tvel[2 * P.N + i] = v[2];
-    P.tcell[i] = cell;
-    P.tslot[i] = slot;
+    P.to.put(i, v[0], v[1], v[2], no, cell, slot);
 }
 
 // Placement of arbitrary positions into IOS (the entry of a differentiable
@@ -137,9 +144,7 @@ struct PlaceParams {
     const double *pos0, *pos1, *pos2;
     const float *mom0, *mom1, *mom2;   // may be null: zero momenta
     int32_t *count;
-    uint16_t *toff;
-    float *tvel;
-    int32_t *tcell, *tslot;
+    Moved to;
     int64_t N;
     int n_ios;
     double s_ios;
@@ -200,14 +205,7 @@ __global__ void __launch_bounds__(256) place_kernel(PlaceParams P) {
     if (bad) set_status(P.status, ST_NONFINITE);
     const int cell = (nc[2] * n + nc[1]) * n + nc[0];
     const int slot = atomicAdd(&P.count[cell], 1);
-    P.toff[i] = no[0];
-    P.toff[P.N + i] = no[1];
-    P.toff[2 * P.N + i] = no[2];
-    P.tvel[i] = P.mom0 ? P.mom0[i] : 0.0f;
-    P.tvel[P.N + i] = P.mom1 ? P.mom1[i] : 0.0f;
-    P.tvel[2 * P.N + i] = P.mom2 ? P.mom2[i] : 0.0f;
-    P.tcell[i] = cell;
-    P.tslot[i] = slot;
+    P.to.put(i, P.mom0 ? P.mom0[i] : 0.0f, P.mom1 ? P.mom1[i] : 0.0f, P.mom2 ? P.mom2[i] : 0.0f, no, cell, slot);
 }
 
 // -------------------------------------------------------------- scan
@@ -238,12 +236,28 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *warp_sums, int &
     return out;
 }
 
-__global__ void __launch_bounds__(SCAN_THREADS) scan_reduce_kernel(const int32_t *in, int32_t *sums, int64_t n) {
+// A thread's SCAN_ITEMS elements; wide: both arrays on 16-byte boundaries (256^3
+// cells: 0.095 -> 0.049 ms against single words, 512^3 0.65 -> 0.28)
+__device__ __forceinline__ void scan_load(const int32_t *in, int64_t base, int64_t n, bool wide, int v[SCAN_ITEMS]) {
+    if (wide && base + SCAN_ITEMS <= n) {
+#pragma unroll
+        for (int k = 0; k < SCAN_ITEMS; k += 4) {
+            const int4 q = *reinterpret_cast<const int4 *>(in + base + k);
+            v[k] = q.x; v[k + 1] = q.y; v[k + 2] = q.z; v[k + 3] = q.w;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < SCAN_ITEMS; ++k) v[k] = base + k < n ? in[base + k] : 0;
+    }
+}
+
+__global__ void __launch_bounds__(SCAN_THREADS) scan_reduce_kernel(const int32_t *in, int32_t *sums, int64_t n, bool wide) {
     __shared__ int ws[33];
     const int64_t base = (int64_t)blockIdx.x * SCAN_CHUNK + (int64_t)threadIdx.x * SCAN_ITEMS;
-    int s = 0;
+    int v[SCAN_ITEMS], s = 0;
+    scan_load(in, base, n, wide, v);
 #pragma unroll
-    for (int k = 0; k < SCAN_ITEMS; ++k) s += (base + k < n) ? in[base + k] : 0;
+    for (int k = 0; k < SCAN_ITEMS; ++k) s += v[k];
     int total;
     block_exclusive_scan(s, ws, total);
     if (threadIdx.x == 0) sums[blockIdx.x] = total;
@@ -251,31 +265,38 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_reduce_kernel(const int32_t
 
 // exclusive scan of in[0, n) into out, adding offsets[blockIdx] (if non-null)
 __global__ void __launch_bounds__(SCAN_THREADS) scan_apply_kernel(const int32_t *in, int32_t *out, int64_t n,
-                                                                  const int32_t *offsets) {
+                                                                  const int32_t *offsets, bool wide) {
     __shared__ int ws[33];
     const int64_t base = (int64_t)blockIdx.x * SCAN_CHUNK + (int64_t)threadIdx.x * SCAN_ITEMS;
-    int v[SCAN_ITEMS];
-    int s = 0;
+    int v[SCAN_ITEMS], s = 0;
+    scan_load(in, base, n, wide, v);
 #pragma unroll
-    for (int k = 0; k < SCAN_ITEMS; ++k) {
-        v[k] = (base + k < n) ? in[base + k] : 0;
-        s += v[k];
-    }
+    for (int k = 0; k < SCAN_ITEMS; ++k) s += v[k];
     int total;
     int run = block_exclusive_scan(s, ws, total) + (offsets ? offsets[blockIdx.x] : 0);
 #pragma unroll
     for (int k = 0; k < SCAN_ITEMS; ++k) {
-        if (base + k < n) out[base + k] = run;
-        run += v[k];
+        const int t = v[k];
+        v[k] = run;
+        run += t;
+    }
+    if (wide && base + SCAN_ITEMS <= n) {
+#pragma unroll
+        for (int k = 0; k < SCAN_ITEMS; k += 4)
+            *reinterpret_cast<int4 *>(out + base + k) = make_int4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < SCAN_ITEMS; ++k)
+            if (base + k < n) out[base + k] = v[k];
     }
 }
 
 // ------------------------------------------------------------- rebin
-__global__ void scatter_kernel(const int32_t *tcell, const int32_t *tslot, const int32_t *start,
-                               int32_t *perm, int64_t n) {
+__global__ void __launch_bounds__(256) scatter_kernel(Moved from, const int32_t *__restrict__ start, int32_t *perm,
+                                                      int64_t n) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    perm[start[tcell[i]] + tslot[i]] = (int32_t)i;
+    perm[__ldg(&start[from.cell_off[i].x]) + from.slot[i]] = (int32_t)i;
 }
 
 // Cells of more than RANK_MAX particles, whose segments are sorted ascending
@@ -292,10 +313,10 @@ constexpr int SORT_THREADS = 512, SORT_WARPS = SORT_THREADS / 32;
 constexpr int BIG_SORT_SMEM = 8192;
 
 __global__ void __launch_bounds__(256) sort_list_kernel(const int32_t *__restrict__ count, int64_t n_cells, int32_t *big,
-                                                        int *big_n) {
+                                                        int *big_n, bool wide) {
     const int64_t c0 = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
     int4 v = make_int4(0, 0, 0, 0);
-    if (c0 + 3 < n_cells) v = __ldg(reinterpret_cast<const int4 *>(count + c0));
+    if (wide && c0 + 3 < n_cells) v = __ldg(reinterpret_cast<const int4 *>(count + c0));
     else
         for (int k = 0; c0 + k < n_cells && k < 4; ++k) (&v.x)[k] = count[c0 + k];
     if (max(max(v.x, v.y), max(v.z, v.w)) <= RANK_MAX) return;
@@ -417,9 +438,8 @@ __global__ void __launch_bounds__(SORT_THREADS) sort_cells_kernel(const int32_t 
 struct GatherParams {
     const int32_t *slots;          // old index by provisional slot (scatter_kernel)
     int32_t *perm;                 // old index by new index
-    const int32_t *tcell, *count, *start;
-    const uint16_t *toff;
-    const float *tvel;
+    const int32_t *count, *start;
+    Moved from;
     uint16_t *off0, *off1, *off2;
     float *vel0, *vel1, *vel2;
     int32_t *cellid;
@@ -429,12 +449,15 @@ struct GatherParams {
 // One thread per provisional slot: its place is its rank in the cell.  Bound by
 // the scattered reads of a particle's 24 bytes.  A pass of its own that sorted the
 // small segments, a thread per cell, took 0.28 ms and the gather 0.25 on the 256^3
-// run at z = 0 (512^3 at z = 1: 1.91 and 2.01); together they take 0.34 (2.63).
+// run at z = 0 (512^3 at z = 1: 1.91 and 2.01); together they took 0.34
+// (2.63), with the packed records 0.23 (1.67).
 __global__ void __launch_bounds__(256) gather_kernel(GatherParams P) {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= P.N) return;
     const int j = P.slots[s];
-    const int c = P.tcell[j];
+    const int2 co = __ldg(&P.from.cell_off[j]);
+    const float4 vo = __ldg(&P.from.vel_off[j]);
+    const int c = co.x;
     const int cnt = __ldg(&P.count[c]);
     int64_t i = s;
     if (cnt > 1 && cnt <= RANK_MAX) {
@@ -443,41 +466,92 @@ __global__ void __launch_bounds__(256) gather_kernel(GatherParams P) {
         for (int k = 0; k < cnt; ++k) rank += __ldg(&P.slots[st + k]) < j;
         i = st + rank;
     }
+    const unsigned off01 = __float_as_uint(vo.w);
     P.perm[i] = j;
-    P.off0[i] = P.toff[j];
-    P.off1[i] = P.toff[P.N + j];
-    P.off2[i] = P.toff[2 * P.N + j];
-    P.vel0[i] = P.tvel[j];
-    P.vel1[i] = P.tvel[P.N + j];
-    P.vel2[i] = P.tvel[2 * P.N + j];
+    P.off0[i] = (uint16_t)off01;
+    P.off1[i] = (uint16_t)(off01 >> 16);
+    P.off2[i] = (uint16_t)co.y;
+    P.vel0[i] = vo.x;
+    P.vel1[i] = vo.y;
+    P.vel2[i] = vo.z;
     P.cellid[i] = c;
 }
 
 // FP16 velocity codec: per IOS cell the FP32 scale max_p,d |v_d| (an atomic
 // max on the bit patterns, which order like the values for v >= 0, so the
 // result does not depend on order), then code = RN_half(RN32(v / scale)).
-__global__ void vel_scale_kernel(const float *__restrict__ v0, const float *__restrict__ v1,
-                                 const float *__restrict__ v2, const int32_t *__restrict__ cellid,
-                                 float *__restrict__ vscale, int64_t N) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const float m = fmaxf(fabsf(v0[i]), fmaxf(fabsf(v1[i]), fabsf(v2[i])));
-    atomicMax(reinterpret_cast<int *>(&vscale[cellid[i]]), __float_as_int(m));
+//
+// One pass, a CTA per 1024 cells: their particles lie in a row, the maxima stay in
+// shared memory, the first ENCODE_HELD rounds of velocities in registers (more, in a
+// dense state, are read again from the caches).  As two kernels with the maxima in
+// global memory it took 1.81 ms for 512^3 particles, now 0.86 (256 cells
+// and one round, waiting for its loads: 1.73; 512 cells: 1.07).
+constexpr int ENCODE_CELLS = 1024, ENCODE_HELD = 4, ENCODE_THREADS = 256;
+
+__device__ __forceinline__ uint16_t velocity_code(float v, float s) {
+    return s > 0.0f ? __half_as_ushort(__float2half_rn(__fdiv_rn(v, s))) : (uint16_t)0;
 }
 
-__global__ void vel_encode_kernel(const float *__restrict__ v0, const float *__restrict__ v1,
-                                  const float *__restrict__ v2, const int32_t *__restrict__ cellid,
-                                  const float *__restrict__ vscale, uint16_t *__restrict__ c0,
-                                  uint16_t *__restrict__ c1, uint16_t *__restrict__ c2, int64_t N) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const float s = vscale[cellid[i]];
-    if (s > 0.0f) {
-        c0[i] = __half_as_ushort(__float2half_rn(__fdiv_rn(v0[i], s)));
-        c1[i] = __half_as_ushort(__float2half_rn(__fdiv_rn(v1[i], s)));
-        c2[i] = __half_as_ushort(__float2half_rn(__fdiv_rn(v2[i], s)));
-    } else {
-        c0[i] = c1[i] = c2[i] = 0;
+__global__ void __launch_bounds__(ENCODE_THREADS)
+vel_encode_kernel(const float *__restrict__ v0, const float *__restrict__ v1, const float *__restrict__ v2,
+                  const int32_t *__restrict__ cellid, const int32_t *__restrict__ count,
+                  const int32_t *__restrict__ start, float *__restrict__ vscale, uint16_t *__restrict__ c0,
+                  uint16_t *__restrict__ c1, uint16_t *__restrict__ c2, int64_t n_cells) {
+    __shared__ int top[ENCODE_CELLS];
+    const int64_t first = (int64_t)blockIdx.x * ENCODE_CELLS;
+    const int cells = (int)min((int64_t)ENCODE_CELLS, n_cells - first);
+    const int lane = threadIdx.x & 31;
+    const int64_t b = start[first], e = (int64_t)start[first + cells - 1] + count[first + cells - 1];
+    for (int k = threadIdx.x; k < ENCODE_CELLS; k += ENCODE_THREADS) top[k] = 0;
+    auto largest = [&](int c, float x, float y, float z) {
+        int m = c >= 0 ? __float_as_int(fmaxf(fabsf(x), fmaxf(fabsf(y), fabsf(z)))) : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {   // a run of lanes in one cell: its maximum, at its last lane
+            const int cu = __shfl_up_sync(0xffffffffu, c, o), mu = __shfl_up_sync(0xffffffffu, m, o);
+            if (lane >= o && cu == c) m = max(m, mu);
+        }
+        const int next = __shfl_down_sync(0xffffffffu, c, 1);
+        if (c >= 0 && (lane == 31 || next != c)) atomicMax(&top[c], m);
+    };
+    int c[ENCODE_HELD];
+    float x[ENCODE_HELD], y[ENCODE_HELD], z[ENCODE_HELD];
+#pragma unroll
+    for (int k = 0; k < ENCODE_HELD; ++k) {
+        const int64_t i = b + k * ENCODE_THREADS + threadIdx.x;
+        c[k] = -1;
+        x[k] = y[k] = z[k] = 0.0f;
+        if (i < e) {
+            c[k] = cellid[i] - (int)first;
+            x[k] = v0[i]; y[k] = v1[i]; z[k] = v2[i];
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < ENCODE_HELD; ++k)
+        if (b + k * ENCODE_THREADS < e) largest(c[k], x[k], y[k], z[k]);
+    const int64_t rest = b + ENCODE_HELD * ENCODE_THREADS;
+    for (int64_t w = rest + (threadIdx.x & ~31); w < e; w += ENCODE_THREADS) {   // a warp at a time
+        const int64_t i = w + lane;
+        const bool in = i < e;
+        largest(in ? cellid[i] - (int)first : -1, in ? v0[i] : 0.0f, in ? v1[i] : 0.0f, in ? v2[i] : 0.0f);
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < cells; k += ENCODE_THREADS) vscale[first + k] = __int_as_float(top[k]);
+#pragma unroll
+    for (int k = 0; k < ENCODE_HELD; ++k) {
+        const int64_t i = b + k * ENCODE_THREADS + threadIdx.x;
+        if (i < e) {
+            const float s = __int_as_float(top[c[k]]);
+            c0[i] = velocity_code(x[k], s);
+            c1[i] = velocity_code(y[k], s);
+            c2[i] = velocity_code(z[k], s);
+        }
+    }
+    for (int64_t i = rest + threadIdx.x; i < e; i += ENCODE_THREADS) {
+        const float s = __int_as_float(top[cellid[i] - (int)first]);
+        c0[i] = velocity_code(v0[i], s);
+        c1[i] = velocity_code(v1[i], s);
+        c2[i] = velocity_code(v2[i], s);
     }
 }
 
@@ -497,14 +571,12 @@ __global__ void vel_decode_kernel(const uint16_t *__restrict__ c0, const uint16_
 
 // p->vel16 / p->vscale from FP32 momenta v (ctx->cellid must hold p's cells).
 cudaError_t launch_vel_encode(cube2_ctx *ctx, const cube2_particles *p, const float *const v[3]) {
-    cudaError_t e = cudaMemsetAsync(p->vscale, 0, sizeof(float) * ctx->n_cells, ctx->stream);
-    const int64_t blocks = (ctx->N + 255) / 256;
-    if (e != cudaSuccess || blocks == 0) return e;
+    if (ctx->N == 0) return cudaMemsetAsync(p->vscale, 0, sizeof(float) * ctx->n_cells, ctx->stream);
     ProfScope prof(ctx, P_KICK, 0);
-    vel_scale_kernel<<<(unsigned)blocks, 256, 0, ctx->stream>>>(v[0], v[1], v[2], ctx->cellid, p->vscale, ctx->N);
-    vel_encode_kernel<<<(unsigned)blocks, 256, 0, ctx->stream>>>(v[0], v[1], v[2], ctx->cellid, p->vscale, p->vel16[0],
-                                                                p->vel16[1], p->vel16[2], ctx->N);
-    ctx->launches += 2;
+    vel_encode_kernel<<<(unsigned)((ctx->n_cells + ENCODE_CELLS - 1) / ENCODE_CELLS), ENCODE_THREADS, 0, ctx->stream>>>(
+        v[0], v[1], v[2], ctx->cellid, p->count, p->start, p->vscale, p->vel16[0], p->vel16[1], p->vel16[2],
+        ctx->n_cells);
+    ctx->launches++;
     return cudaGetLastError();
 }
 
@@ -527,8 +599,10 @@ int64_t scan_scratch_len(int64_t n) {
 }
 
 cudaError_t launch_scan(cube2_ctx *ctx, const int32_t *in, int32_t *out, int64_t n) {
+    // the callers' arrays may lie anywhere (4-byte words): wide loads only where both allow them
+    const bool wide = ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
     if (n <= SCAN_CHUNK) {
-        scan_apply_kernel<<<1, SCAN_THREADS, 0, ctx->stream>>>(in, out, n, nullptr);
+        scan_apply_kernel<<<1, SCAN_THREADS, 0, ctx->stream>>>(in, out, n, nullptr, wide);
         ctx->launches++;
         return cudaGetLastError();
     }
@@ -536,14 +610,14 @@ cudaError_t launch_scan(cube2_ctx *ctx, const int32_t *in, int32_t *out, int64_t
     const int64_t nb = (n + SCAN_CHUNK - 1) / SCAN_CHUNK;
     int32_t *sums = ctx->scan_tmp;
     // reserve this level's sums, recurse on the remainder of the scratch
-    scan_reduce_kernel<<<(unsigned)nb, SCAN_THREADS, 0, ctx->stream>>>(in, sums, n);
+    scan_reduce_kernel<<<(unsigned)nb, SCAN_THREADS, 0, ctx->stream>>>(in, sums, n, wide);
     ctx->launches++;
     int32_t *saved = ctx->scan_tmp;
     ctx->scan_tmp = saved + nb;
     cudaError_t e = launch_scan(ctx, sums, sums, nb);
     ctx->scan_tmp = saved;
     if (e != cudaSuccess) return e;
-    scan_apply_kernel<<<(unsigned)nb, SCAN_THREADS, 0, ctx->stream>>>(in, out, n, sums);
+    scan_apply_kernel<<<(unsigned)nb, SCAN_THREADS, 0, ctx->stream>>>(in, out, n, sums, wide);
     ctx->launches++;
     return cudaGetLastError();
 }
@@ -558,6 +632,10 @@ cudaError_t launch_kick(cube2_ctx *ctx, const cube2_particles *p, float kick) {
     return cudaGetLastError();
 }
 
+static Moved moved(const cube2_ctx *ctx) {
+    return {reinterpret_cast<float4 *>(ctx->moved16), reinterpret_cast<int2 *>(ctx->moved8), ctx->tslot};
+}
+
 cudaError_t launch_kick_drift(cube2_ctx *ctx, const cube2_particles *p, float kick, float drift_fix) {
     DriftParams P{};
     P.off0 = p->off[0]; P.off1 = p->off[1]; P.off2 = p->off[2];
@@ -568,18 +646,15 @@ cudaError_t launch_kick_drift(cube2_ctx *ctx, const cube2_particles *p, float ki
     }
     P.acc0 = p->acc[0]; P.acc1 = p->acc[1]; P.acc2 = p->acc[2];
     P.cellid = ctx->cellid;
-    P.count = ctx->ncount;
-    P.toff = ctx->toff;
-    P.tvel = ctx->tvel;
-    P.tcell = ctx->tcell;
-    P.tslot = ctx->tslot;
+    P.count = p->count;
+    P.to = moved(ctx);
     P.N = ctx->N;
     P.n_ios = ctx->n_ios;
     P.kick = kick;
     P.drift_fix = drift_fix;
     P.status = ctx->dev_status;
     ProfScope prof(ctx, P_KICK_DRIFT, 0);
-    cudaError_t e = cudaMemsetAsync(ctx->ncount, 0, sizeof(int32_t) * ctx->n_cells, ctx->stream);
+    cudaError_t e = cudaMemsetAsync(p->count, 0, sizeof(int32_t) * ctx->n_cells, ctx->stream);
     if (e != cudaSuccess) return e;
     const int64_t blocks = (ctx->N + 255) / 256;
     if (blocks == 0) return cudaSuccess;
@@ -588,21 +663,19 @@ cudaError_t launch_kick_drift(cube2_ctx *ctx, const cube2_particles *p, float ki
     return cudaGetLastError();
 }
 
-cudaError_t launch_place(cube2_ctx *ctx, const double *const pos[3], const float *const mom[3]) {
+cudaError_t launch_place(cube2_ctx *ctx, const double *const pos[3], const float *const mom[3],
+                         const cube2_particles *p) {
     PlaceParams P{};
     P.pos0 = pos[0]; P.pos1 = pos[1]; P.pos2 = pos[2];
     if (mom) { P.mom0 = mom[0]; P.mom1 = mom[1]; P.mom2 = mom[2]; }
-    P.count = ctx->ncount;
-    P.toff = ctx->toff;
-    P.tvel = ctx->tvel;
-    P.tcell = ctx->tcell;
-    P.tslot = ctx->tslot;
+    P.count = p->count;
+    P.to = moved(ctx);
     P.N = ctx->N;
     P.n_ios = ctx->n_ios;
     P.s_ios = ctx->s_ios;
     reciprocal(ctx->s_ios, P.recip, P.recip_shift);
     P.status = ctx->dev_status;
-    cudaError_t e = cudaMemsetAsync(ctx->ncount, 0, sizeof(int32_t) * ctx->n_cells, ctx->stream);
+    cudaError_t e = cudaMemsetAsync(p->count, 0, sizeof(int32_t) * ctx->n_cells, ctx->stream);
     if (e != cudaSuccess) return e;
     const int64_t blocks = (ctx->N + 255) / 256;
     if (blocks == 0) return cudaSuccess;
@@ -615,36 +688,33 @@ cudaError_t launch_rebin(cube2_ctx *ctx, const cube2_particles *p) {
     cudaError_t e;
     {
         ProfScope prof(ctx, P_SCAN, 0);
-        e = launch_scan(ctx, ctx->ncount, ctx->nstart, ctx->n_cells);
+        e = launch_scan(ctx, p->count, p->start, ctx->n_cells);
     }
     if (e != cudaSuccess) return e;
     const int64_t pb = (ctx->N + 255) / 256, cb = (ctx->n_cells + 255) / 256;
     if (pb > 0) {
         {
             ProfScope prof(ctx, P_SCATTER, 0);
-            scatter_kernel<<<(unsigned)pb, 256, 0, ctx->stream>>>(ctx->tcell, ctx->tslot, ctx->nstart, ctx->perm2,
-                                                                  ctx->N);
+            scatter_kernel<<<(unsigned)pb, 256, 0, ctx->stream>>>(moved(ctx), p->start, ctx->perm2, ctx->N);
         }
         e = cudaMemsetAsync(ctx->big_n, 0, 2 * sizeof(int), ctx->stream);
         if (e != cudaSuccess) return e;
         {
             ProfScope prof(ctx, P_SORT, 0);
-            sort_list_kernel<<<(unsigned)((cb + 3) / 4), 256, 0, ctx->stream>>>(ctx->ncount, ctx->n_cells, ctx->big,
-                                                                               ctx->big_n);
+            sort_list_kernel<<<(unsigned)((cb + 3) / 4), 256, 0, ctx->stream>>>(
+                p->count, ctx->n_cells, ctx->big, ctx->big_n, (reinterpret_cast<uintptr_t>(p->count) & 15) == 0);
         }
         {
             ProfScope prof(ctx, P_SORT_BIG, 0);
             sort_cells_kernel<<<(unsigned)(ctx->num_sms * (1536 / SORT_THREADS)), SORT_THREADS, 0, ctx->stream>>>(
-                ctx->ncount, ctx->nstart, ctx->perm2, ctx->perm, ctx->big, ctx->big_n, ctx->n_cells);
+                p->count, p->start, ctx->perm2, ctx->perm, ctx->big, ctx->big_n, ctx->n_cells);
         }
         GatherParams G{};
         G.slots = ctx->perm2;
         G.perm = ctx->perm;
-        G.count = ctx->ncount;
-        G.start = ctx->nstart;
-        G.tcell = ctx->tcell;
-        G.toff = ctx->toff;
-        G.tvel = ctx->tvel;
+        G.count = p->count;
+        G.start = p->start;
+        G.from = moved(ctx);
         G.off0 = p->off[0]; G.off1 = p->off[1]; G.off2 = p->off[2];
         if (ctx->vel32) {   // FP16 storage: the step's FP32 working copy
             G.vel0 = ctx->vel32; G.vel1 = ctx->vel32 + ctx->N; G.vel2 = ctx->vel32 + 2 * ctx->N;
@@ -659,10 +729,6 @@ cudaError_t launch_rebin(cube2_ctx *ctx, const cube2_particles *p) {
         }
         ctx->launches += 4;
     }
-    e = cudaMemcpyAsync(p->count, ctx->ncount, sizeof(int32_t) * ctx->n_cells, cudaMemcpyDeviceToDevice, ctx->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(p->start, ctx->nstart, sizeof(int32_t) * ctx->n_cells, cudaMemcpyDeviceToDevice, ctx->stream);
-    if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
