@@ -375,8 +375,8 @@ void cube2_destroy(cube2_ctx *ctx);
  * the CIC deposit of v_d (G even, D_d odd); for PP,
  * sum_j (g I + g'/r d d^T)(v_j - v_i), g = V_p R_PP(r)/(4 pi r). */
 
-/* Allocate the adjoint's scratch (three FP32 meshes of the largest level,
- * 15 FP32 values per particle).  The one allocating call after
+/* Allocate the adjoint's scratch (four FP32 values per cell of the largest
+ * level, 9 per particle).  The one allocating call after
  * cube2_init_mesh; idempotent. */
 int cube2_adjoint_init(cube2_ctx *ctx);
 

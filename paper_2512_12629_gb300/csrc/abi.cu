@@ -602,9 +602,9 @@ int cube2_adjoint_init(cube2_ctx *ctx) {
     int64_t m = 0;
     for (int l = 0; l < ctx->nl; ++l) m = std::max(m, (int64_t)ctx->lev[l].n * ctx->lev[l].n * ctx->lev[l].n);
     const size_t N = (size_t)std::max<int64_t>(ctx->N, 1);
-    cudaError_t e = cudaMalloc((void **)&ctx->vjp_mu, sizeof(float) * 3 * (size_t)m);
+    cudaError_t e = cudaMalloc((void **)&ctx->vjp_mu, sizeof(float) * 4 * (size_t)m);
     if (e == cudaSuccess) e = cudaMalloc((void **)&ctx->vjp_t, sizeof(float) * 3 * N);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&ctx->vjp_u, sizeof(float) * 12 * N);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&ctx->vjp_u, sizeof(float) * 6 * N);
     if (e == cudaSuccess) e = cudaMalloc((void **)&ctx->vjp_sq, sizeof(double));
     if (e != cudaSuccess) {
         cudaFree(ctx->vjp_mu);

@@ -15,7 +15,7 @@
 // forward's exact integer CIC weights at the stored positions.
 //
 // Kernels: vjp_gather (mode E: the first sum with E from phi by the 4-point
-// difference; mode PSI: the second sum), mu_deposit (three FP32 fields, float
+// difference; mode PSI: the second sum), mu_deposit (FP32 field of vectors, float
 // atomics, so the sum order and the last bits vary between runs) and
 // div_stencil (s, written into the level's real grid for the Poisson solve).
 #include "common.cuh"
@@ -46,10 +46,6 @@ __device__ __forceinline__ CicPoint cic_point(const uint16_t *off0, const uint16
 
 __device__ __forceinline__ int wrapn(int j, int n) { return j < 0 ? j + n : (j >= n ? j - n : j); }
 
-__device__ __forceinline__ float at(const float *g, int n, int x, int y, int z) {
-    return __ldg(&g[((int64_t)wrapn(z, n) * n + wrapn(y, n)) * n + wrapn(x, n)]);
-}
-
 struct VjpParams {
     const uint16_t *off0, *off1, *off2;
     const int32_t *cellid;
@@ -61,11 +57,22 @@ struct VjpParams {
     int n_ios, n, shift;
 };
 
+// The six mesh coordinates i0 - 2 .. i0 + 3 of one axis, wrapped, times the axis'
+// stride: all that a particle's corners and their 4-point differences touch.
+struct Reach {
+    int64_t o[6];
+    __device__ __forceinline__ Reach(int i0, int n, int64_t stride) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) o[k] = wrapn(i0 - 2 + k, n) * stride;
+    }
+};
+
+// Mode E reads the 56 values around a particle that the 4-point differences of its
+// eight corners share, with their offsets wrapped once: 96 reads with an address each
+// took 0.55 ms in the four gathers (two of each mode) of a gradient of 128^3
+// particles, now 0.33.
 template <bool MODE_E>
-#ifndef VJP_MINB
-#define VJP_MINB 1
-#endif
-__global__ void __launch_bounds__(256, VJP_MINB) vjp_gather_kernel(VjpParams P) {
+__global__ void __launch_bounds__(256) vjp_gather_kernel(VjpParams P) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= P.N) return;
     const CicPoint C = cic_point(P.off0, P.off1, P.off2, i, P.cellid[i], P.n_ios, P.shift);
@@ -76,47 +83,55 @@ __global__ void __launch_bounds__(256, VJP_MINB) vjp_gather_kernel(VjpParams P) 
         v[2] = P.v2[i];
     }
     const int n = P.n;
+    const Reach X(C.i0[0], n, 1), Y(C.i0[1], n, n), Z(C.i0[2], n, (int64_t)n * n);
+    const float *f = P.grid;
     float g[3] = {0.f, 0.f, 0.f};
 #pragma unroll
     for (int cz = 0; cz < 2; ++cz)
 #pragma unroll
-        for (int cy = 0; cy < 2; ++cy)
+        for (int cy = 0; cy < 2; ++cy) {
+            const float *row = f + Z.o[2 + cz] + Y.o[2 + cy];
+            float r[6] = {};
+#pragma unroll
+            for (int k = MODE_E ? 0 : 2; k < (MODE_E ? 6 : 4); ++k) r[k] = __ldg(row + X.o[k]);
 #pragma unroll
             for (int cx = 0; cx < 2; ++cx) {
-                const int x = C.i0[0] + cx, y = C.i0[1] + cy, z = C.i0[2] + cz;
                 const float wx = cx ? C.w1[0] : 1.0f - C.w1[0];
                 const float wy = cy ? C.w1[1] : 1.0f - C.w1[1];
                 const float wz = cz ? C.w1[2] : 1.0f - C.w1[2];
                 const float sx = cx ? 1.0f : -1.0f, sy = cy ? 1.0f : -1.0f, sz = cz ? 1.0f : -1.0f;
                 float val;
                 if (MODE_E) {
-                    const float *f = P.grid;
-                    const float ex = (2.0f / 3.0f) * (at(f, n, x + 1, y, z) - at(f, n, x - 1, y, z)) -
-                                     (1.0f / 12.0f) * (at(f, n, x + 2, y, z) - at(f, n, x - 2, y, z));
-                    const float ey = (2.0f / 3.0f) * (at(f, n, x, y + 1, z) - at(f, n, x, y - 1, z)) -
-                                     (1.0f / 12.0f) * (at(f, n, x, y + 2, z) - at(f, n, x, y - 2, z));
-                    const float ez = (2.0f / 3.0f) * (at(f, n, x, y, z + 1) - at(f, n, x, y, z - 1)) -
-                                     (1.0f / 12.0f) * (at(f, n, x, y, z + 2) - at(f, n, x, y, z - 2));
+                    // the neighbours' values of the other corners are among the row's own
+                    const float *fy = f + Z.o[2 + cz] + X.o[2 + cx], *fz = f + Y.o[2 + cy] + X.o[2 + cx];
+                    const float ex = (2.0f / 3.0f) * (r[3 + cx] - r[1 + cx]) - (1.0f / 12.0f) * (r[4 + cx] - r[cx]);
+                    const float ey = (2.0f / 3.0f) * (__ldg(fy + Y.o[3 + cy]) - __ldg(fy + Y.o[1 + cy])) -
+                                     (1.0f / 12.0f) * (__ldg(fy + Y.o[4 + cy]) - __ldg(fy + Y.o[cy]));
+                    const float ez = (2.0f / 3.0f) * (__ldg(fz + Z.o[3 + cz]) - __ldg(fz + Z.o[1 + cz])) -
+                                     (1.0f / 12.0f) * (__ldg(fz + Z.o[4 + cz]) - __ldg(fz + Z.o[cz]));
                     val = -(ex * v[0] + ey * v[1] + ez * v[2]);
                 } else {
-                    val = at(P.grid, n, x, y, z);
+                    val = r[2 + cx];
                 }
                 g[0] += sx * wy * wz * val;
                 g[1] += wx * sy * wz * val;
                 g[2] += wx * wy * sz * val;
             }
+        }
     P.w0[i] += P.scale * g[0];
     P.w1[i] += P.scale * g[1];
     P.w2[i] += P.scale * g[2];
 }
 
-__global__ void __launch_bounds__(256) mu_deposit_kernel(VjpParams P, float *mu) {
+// The three components lie together, so that a corner is one 16-byte reduction:
+// bound by the reductions at L2, 24 single ones a particle made the two sources of a
+// gradient of 128^3 particles take 0.88 ms, eight wide ones 0.69.
+__global__ void __launch_bounds__(256) mu_deposit_kernel(VjpParams P, float4 *mu) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= P.N) return;
     const CicPoint C = cic_point(P.off0, P.off1, P.off2, i, P.cellid[i], P.n_ios, P.shift);
     const float v[3] = {P.v0[i], P.v1[i], P.v2[i]};
     const int n = P.n;
-    const int64_t n3 = (int64_t)n * n * n;
 #pragma unroll
     for (int cz = 0; cz < 2; ++cz)
 #pragma unroll
@@ -127,24 +142,27 @@ __global__ void __launch_bounds__(256) mu_deposit_kernel(VjpParams P, float *mu)
                                 (cz ? C.w1[2] : 1.0f - C.w1[2]);
                 const int64_t c = ((int64_t)wrapn(C.i0[2] + cz, n) * n + wrapn(C.i0[1] + cy, n)) * n +
                                   wrapn(C.i0[0] + cx, n);
-                atomicAdd(&mu[c], W * v[0]);
-                atomicAdd(&mu[n3 + c], W * v[1]);
-                atomicAdd(&mu[2 * n3 + c], W * v[2]);
+                asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(
+                                 __cvta_generic_to_global(mu + c)),
+                             "f"(W * v[0]), "f"(W * v[1]), "f"(W * v[2]), "f"(0.0f)
+                             : "memory");
             }
 }
 
-__global__ void __launch_bounds__(256) div_stencil_kernel(const float *mu, float *s, int n, float scale) {
+__global__ void __launch_bounds__(256) div_stencil_kernel(const float4 *__restrict__ mu, float *__restrict__ s, int n,
+                                                          float scale) {
     const int64_t n3 = (int64_t)n * n * n;
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= n3) return;
     const int x = (int)(c % n), y = (int)((c / n) % n), z = (int)(c / ((int64_t)n * n));
-    const float *mx = mu, *my = mu + n3, *mz = mu + 2 * n3;
-    const float dx = (2.0f / 3.0f) * (at(mx, n, x + 1, y, z) - at(mx, n, x - 1, y, z)) -
-                     (1.0f / 12.0f) * (at(mx, n, x + 2, y, z) - at(mx, n, x - 2, y, z));
-    const float dy = (2.0f / 3.0f) * (at(my, n, x, y + 1, z) - at(my, n, x, y - 1, z)) -
-                     (1.0f / 12.0f) * (at(my, n, x, y + 2, z) - at(my, n, x, y - 2, z));
-    const float dz = (2.0f / 3.0f) * (at(mz, n, x, y, z + 1) - at(mz, n, x, y, z - 1)) -
-                     (1.0f / 12.0f) * (at(mz, n, x, y, z + 2) - at(mz, n, x, y, z - 2));
+    const Reach X(x, n, 1), Y(y, n, n), Z(z, n, (int64_t)n * n);
+    const float4 *mx = mu + Z.o[2] + Y.o[2], *my = mu + Z.o[2] + x, *mz = mu + Y.o[2] + x;
+    const float dx = (2.0f / 3.0f) * (__ldg(&mx[X.o[3]].x) - __ldg(&mx[X.o[1]].x)) -
+                     (1.0f / 12.0f) * (__ldg(&mx[X.o[4]].x) - __ldg(&mx[X.o[0]].x));
+    const float dy = (2.0f / 3.0f) * (__ldg(&my[Y.o[3]].y) - __ldg(&my[Y.o[1]].y)) -
+                     (1.0f / 12.0f) * (__ldg(&my[Y.o[4]].y) - __ldg(&my[Y.o[0]].y));
+    const float dz = (2.0f / 3.0f) * (__ldg(&mz[Z.o[3]].z) - __ldg(&mz[Z.o[1]].z)) -
+                     (1.0f / 12.0f) * (__ldg(&mz[Z.o[4]].z) - __ldg(&mz[Z.o[0]].z));
     s[c] = scale * (dx + dy + dz);
 }
 
@@ -165,39 +183,49 @@ VjpParams make_params(cube2_ctx *ctx, const Level &L, const cube2_particles *p, 
 }
 
 // g(c) = 2 (delta(c) - target(c)) / n^3 in place of delta; sum of squares into *sq.
-__global__ void __launch_bounds__(256) mse_residual_kernel(float *grid, const float *target, int64_t n3, double *sq) {
-    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// A CTA adds one term to the sum: one FP64 atomic per warp of 32 cells, all on one
+// address, took 1.3 ms of a 7.9 ms gradient of 128^3 particles.
+constexpr int MSE_THREADS = 256;
+
+__global__ void __launch_bounds__(MSE_THREADS) mse_residual_kernel(float *__restrict__ grid, const float *__restrict__ target,
+                                                                   int64_t n3, double *sq) {
+    const float scale = (float)(2.0 / (double)n3);
     double r2 = 0.0;
-    if (c < n3) {
+    for (int64_t c = (int64_t)blockIdx.x * MSE_THREADS + threadIdx.x; c < n3; c += (int64_t)gridDim.x * MSE_THREADS) {
         const float r = grid[c] - target[c];
-        r2 = (double)r * (double)r;
-        grid[c] = r * (float)(2.0 / (double)n3);
+        r2 += (double)r * (double)r;
+        grid[c] = r * scale;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) r2 += __shfl_xor_sync(0xffffffffu, r2, o);
-    if ((threadIdx.x & 31) == 0 && r2 != 0.0) atomicAdd(sq, r2);
+    __shared__ double part[MSE_THREADS / 32];
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = r2;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < MSE_THREADS / 32; ++w) r2 += part[w];
+        if (r2 != 0.0) atomicAdd(sq, r2);
+    }
 }
 
 // Reverse of one KDK step, part 1 (post-step order n -> pre-step order perm[n]):
 // xs[perm[n]] = xbar[n] + k2 t[n],  ps[perm[n]] = pbar[n].
-__global__ void __launch_bounds__(256) kdk_adjoint_scatter_kernel(const int32_t *perm, const float *xbar,
-                                                                  const float *pbar, const float *t, float *xs,
-                                                                  float *ps, int64_t N, float k2) {
+struct Ptr3 {
+    float *p[3];
+};
+
+__global__ void __launch_bounds__(256) kdk_adjoint_scatter_kernel(const int32_t *perm, Ptr3 xbar, Ptr3 pbar, const float *t,
+                                                                  float *xs, float *ps, int64_t N, float k2) {
     const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= N) return;
     const int64_t o = perm[n];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        xs[d * N + o] = xbar[d * N + n] + k2 * t[d * N + n];
-        ps[d * N + o] = pbar[d * N + n];
+        xs[d * N + o] = xbar.p[d][n] + k2 * t[d * N + n];
+        ps[d * N + o] = pbar.p[d][n];
     }
 }
 
 // Part 2 (pre-step order): xbar = xs, pbar = ps + drift * xs; part 3: xbar += k1 t.
-struct Ptr3 {
-    float *p[3];
-};
-
 __global__ void __launch_bounds__(256) kdk_adjoint_drift3_kernel(const float *xs, const float *ps, Ptr3 xbar, Ptr3 pbar,
                                                                  int64_t N, float drift) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -224,7 +252,9 @@ __global__ void __launch_bounds__(256) axpy3p_kernel(Ptr3 y, const float *t, int
 cudaError_t launch_density_mse_vjp(cube2_ctx *ctx, Level &L, const cube2_particles *p, const float *target,
                                    float *const w[3], double *sq) {
     const int64_t n3 = (int64_t)L.n * L.n * L.n;
-    mse_residual_kernel<<<(unsigned)((n3 + 255) / 256), 256, 0, ctx->stream>>>(L.real, target, n3, sq);
+    const int64_t tiles = (n3 + MSE_THREADS - 1) / MSE_THREADS;
+    mse_residual_kernel<<<(unsigned)std::min<int64_t>(tiles, ctx->num_sms * 8), MSE_THREADS, 0, ctx->stream>>>(
+        L.real, target, n3, sq);
     ctx->launches++;
     if (ctx->N == 0) return cudaGetLastError();
     const float *const nv[3] = {nullptr, nullptr, nullptr};
@@ -251,20 +281,12 @@ cudaError_t launch_density_vjp(cube2_ctx *ctx, Level &L, const cube2_particles *
 
 cudaError_t launch_kdk_adjoint_scatter(cube2_ctx *ctx, const int32_t *perm, float *const xbar[3],
                                        float *const pbar[3], const float *t, float k2) {
-    // xbar/pbar are three separate arrays: gather them through the scratch rows
     const int64_t N = ctx->N;
     if (N == 0) return cudaSuccess;
     ProfScope prof(ctx, P_ADJ_KDK, 0);
-    float *xs = ctx->vjp_u, *ps = ctx->vjp_u + 3 * N, *xc = ctx->vjp_u + 6 * N;
-    cudaError_t e = cudaSuccess;
-    for (int d = 0; d < 3 && e == cudaSuccess; ++d) {
-        e = cudaMemcpyAsync(xc + d * N, xbar[d], sizeof(float) * N, cudaMemcpyDeviceToDevice, ctx->stream);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(xc + (3 + d) * N, pbar[d], sizeof(float) * N, cudaMemcpyDeviceToDevice, ctx->stream);
-    }
-    if (e != cudaSuccess) return e;
-    kdk_adjoint_scatter_kernel<<<(unsigned)((N + 255) / 256), 256, 0, ctx->stream>>>(perm, xc, xc + 3 * N, t, xs, ps,
-                                                                                   N, k2);
+    Ptr3 X{{xbar[0], xbar[1], xbar[2]}}, Pb{{pbar[0], pbar[1], pbar[2]}};
+    kdk_adjoint_scatter_kernel<<<(unsigned)((N + 255) / 256), 256, 0, ctx->stream>>>(perm, X, Pb, t, ctx->vjp_u,
+                                                                                   ctx->vjp_u + 3 * N, N, k2);
     ctx->launches++;
     return cudaGetLastError();
 }
@@ -315,16 +337,17 @@ cudaError_t launch_vjp_gather_psi(cube2_ctx *ctx, Level &L, const cube2_particle
 cudaError_t launch_vjp_source(cube2_ctx *ctx, Level &L, const cube2_particles *p, const float *const v[3]) {
     const int64_t n3 = (int64_t)L.n * L.n * L.n;
     ProfScope prof(ctx, P_VJP_SOURCE, L.index);
-    cudaError_t e = cudaMemsetAsync(ctx->vjp_mu, 0, sizeof(float) * 3 * n3, ctx->stream);
+    cudaError_t e = cudaMemsetAsync(ctx->vjp_mu, 0, sizeof(float4) * n3, ctx->stream);
     if (e != cudaSuccess) return e;
     if (ctx->N > 0) {
         float *const nw[3] = {nullptr, nullptr, nullptr};
         VjpParams P = make_params(ctx, L, p, v, nw, nullptr);
-        mu_deposit_kernel<<<(unsigned)((ctx->N + 255) / 256), 256, 0, ctx->stream>>>(P, ctx->vjp_mu);
+        mu_deposit_kernel<<<(unsigned)((ctx->N + 255) / 256), 256, 0, ctx->stream>>>(P, reinterpret_cast<float4 *>(ctx->vjp_mu));
         ctx->launches++;
     }
     const float scale = (float)((double)n3 / (double)(ctx->N > 0 ? ctx->N : 1));
-    div_stencil_kernel<<<(unsigned)((n3 + 255) / 256), 256, 0, ctx->stream>>>(ctx->vjp_mu, L.real, L.n, scale);
+    div_stencil_kernel<<<(unsigned)((n3 + 255) / 256), 256, 0, ctx->stream>>>(
+        reinterpret_cast<const float4 *>(ctx->vjp_mu), L.real, L.n, scale);
     ctx->launches++;
     return cudaGetLastError();
 }

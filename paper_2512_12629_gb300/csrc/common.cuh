@@ -128,9 +128,9 @@ struct cube2_ctx {
     int prof_cap = 0, prof_used = 0;
     int *prof_cls = nullptr;       // [prof_cap] class * CUBE2_MAX_LEVELS + level
     // force vector-Jacobian product scratch (cube2_adjoint_init)
-    float *vjp_mu = nullptr;       // [3][n_max^3] CIC deposit of the cotangent
+    float *vjp_mu = nullptr;       // [n_max^3][4] CIC deposit of the cotangent, the fourth unused
     float *vjp_t = nullptr;        // [3][N] a force product
-    float *vjp_u = nullptr;        // [12][N] reverse-step scratch
+    float *vjp_u = nullptr;        // [6][N] reverse-step scratch
     double *vjp_sq = nullptr;      // [1] loss accumulator
     cube2::PM3 pm3;                // adaptive third level (cfg.pm3_tile > 0)
     float *vel32 = nullptr;        // [3][N] FP32 working momenta of a step (cfg.vel_fp16 = 1 only)
