@@ -132,6 +132,7 @@ void free_ctx(cube2_ctx *c) {
     cudaFree(c->pp_perm);
     cudaFree(c->pp_tgt);
     cudaFree(c->pp_dense);
+    cudaFree(c->pp_long);
     cudaFree(c->vjp_mu);
     cudaFree(c->vjp_t);
     cudaFree(c->vjp_u);
@@ -329,11 +330,12 @@ int cube2_init_mesh(cube2_ctx **out, const cube2_config *cfg, void *stream) {
     alloc((void **)&c->perm, N * 4);
     alloc((void **)&c->perm2, N * 4);
     alloc((void **)&c->big, (size_t)c->n_cells * 4);
-    alloc((void **)&c->big_n, 2 * sizeof(int));
+    alloc((void **)&c->big_n, 3 * sizeof(int));
     alloc((void **)&c->pos4, N * 16);
     alloc((void **)&c->pp_perm, N * 4);
     alloc((void **)&c->pp_tgt, (size_t)pp_target_slots(c->N, c->n_ios) * 4);
     alloc((void **)&c->pp_dense, (size_t)pp_dense_cells(c->N) * sizeof(int2));
+    alloc((void **)&c->pp_long, (size_t)(pp_target_slots(c->N, c->n_ios) / 32) * 4);
     alloc((void **)&c->pp_stats, 4 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemsetAsync(c->pp_stats, 0, 4 * sizeof(unsigned long long), c->stream);
     if (cfg->vel_fp16) alloc((void **)&c->vel32, N * 3 * 4);

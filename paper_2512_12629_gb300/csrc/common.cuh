@@ -107,12 +107,13 @@ struct cube2_ctx {
     int32_t *perm = nullptr;
     int32_t *perm2 = nullptr;      // [N] merge scratch of the segmented sort
     int32_t *big = nullptr;        // [n_cells] cells too large for the per-thread sort
-    int *big_n = nullptr;          // [2] their numbers (up to 1024 particles, more); in PP: dense cells, target
-                                   // places
+    int *big_n = nullptr;          // [3] their numbers (a warp each, a CTA each); in PP: dense cells, target
+                                   // places, warps with long streams
     float4 *pos4 = nullptr;        // [N] in-cell offsets as floats (+ cell id bits), PP order
     int32_t *pp_perm = nullptr;    // [N] particle index of each PP slot (sub-cell order in dense cells)
     int32_t *pp_tgt = nullptr;     // [pp_target_slots] PP slots in target (pencil) order, -1 in the pencils' padding
     int2 *pp_dense = nullptr;      // [N / 64] dense cells and the places of their first targets
+    int32_t *pp_long = nullptr;    // [target places / 32] warps whose source stream several warps share
     unsigned long long *pp_stats = nullptr;  // [4] in-range ordered pairs, candidates; the same of per-lane walks
     int num_sms = 152;
     int32_t *scan_tmp = nullptr;   // block sums of the multi-level scan

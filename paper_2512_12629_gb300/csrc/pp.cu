@@ -24,8 +24,8 @@
 // Compact warps evaluate every pair of target and kept source; others test all
 // of them (packed arithmetic) and evaluate the ones found in range from a queue
 // per lane.  The few warps spread along x (nearly empty regions) walk each
-// lane's own 27 cells.  The adjoint's Jacobian product (pp_vjp_kernel) uses the
-// same stream.
+// lane's own 27 cells.  Long streams of small boxes are shared by eight warps in a
+// second kernel.  The adjoint's Jacobian product (pp_vjp_kernel) uses the same stream.
 //
 // 256^3 run, a step's PP at z = 49 / z = 1 / z = 0: 1.35 / 5.0 / 8.7 ms;
 // with the targets in IOS order (streams only for warps inside one row, the
@@ -65,6 +65,9 @@ struct PPParams {
     int pm3_T, pm3_ns;
     float bcut2_3, inv_bcut_3;
     int wmax;                         // widest warp along x (cells beyond the first) on the shared stream
+    int long_min;                     // longer streams go to the list and are shared by PP_PARTS warps
+    int32_t *long_list;               // target places / 32 of those warps
+    int *long_n;
 };
 
 // R(r, b) of Eq. (refforce) times b^2, as a function of u = r / b < 1.
@@ -375,6 +378,27 @@ constexpr int MIXED_N = 32;             // sources evaluated at a time, any dist
 constexpr int SPARSE_N = 128;           // sources tested before the pairs found are evaluated
 constexpr int QUEUE_N = 32;             // pairs a lane can hold
 
+// A warp in a halo has a stream of thousands of sources and works on it long after
+// the rest of a small box is done.  Streams longer than PPParams.long_min are put on a
+// list and shared by the PP_PARTS warps of a CTA in a second kernel; the partial sums
+// are added in their order, so the result does not depend on which path (the
+// ensemble's persistent kernel works on the parts one after another) computed them.
+//
+// Where the line lies: splitting repeats the staging in every part and starts after
+// the first kernel, so it pays while a long warp outlives the others, that is in small
+// boxes.  PP of 64^3 particles at z = 1, 20 % in haloes, with 512 / 1024 / 2048 / no
+// limit: 0.164 / 0.195 / 0.285 / 0.283 ms; 128^3 at z = 0.5, 40 % in haloes, with 512 /
+// 1024 / 4096 / 8192 / none: 1.245 / 1.188 / 1.167 / 1.120 / 1.122 ms; 256^3 at z = 0
+// with 2048 / 8192 / none 9.46 / 8.76 / 8.75.  The adjoint's pairs cost several times
+// more: 64^3 at z = 0.2, 40 %, with 512 / 1024 / 2048 / none: 1.22 / 1.25 / 1.43 / 2.01
+// ms for its two products; 128^3 at z = 1, 10 %, with 256 / 512 / 1024 / 2048 / none
+// 2.57 / 2.08 / 2.09 / 2.12 / 2.33.  4 or 16 parts are no better than 8.
+constexpr int PP_PARTS = 8;
+constexpr int64_t PP_LONG_N = 65536;    // smaller boxes: the second launch costs more than it gives
+
+inline int pp_long_min(int64_t N) { return N < PP_LONG_N ? 0x7fffffff : N < (1 << 19) ? 512 : (int)(N / 256); }
+inline int vjp_long_min(int64_t N) { return N < PP_LONG_N ? 0x7fffffff : N < (1 << 20) ? 512 : (int)(N / 2048); }
+
 struct alignas(16) PPWarpShared {
     union {
         struct {
@@ -385,7 +409,6 @@ struct alignas(16) PPWarpShared {
             Soa<SPARSE_N + 4> src;
             unsigned char queue[QUEUE_N][32];
         } s;
-        float4 buf[64];
     } u;
     int4 seg[PP_SEGS];
     int begin[PP_SEGS];
@@ -400,20 +423,6 @@ __device__ __forceinline__ float4 frame_position(float4 q, int4 g) {
 
 // padding sources: out of range of every target, and no overflow in the pair formula
 constexpr float PP_FAR = 4096.0f;
-
-// Candidate test of 32 staged sources: bit (31 - k) set where source k is
-// closer than b_cut (sign of r^2 - b_cut^2, shifted in).
-__device__ __forceinline__ unsigned test32(const float4 *S, float mx, float my, float mz, float bcut2) {
-    unsigned m = 0u;
-#pragma unroll
-    for (int k = 0; k < 32; ++k) {
-        const float4 q = S[k];
-        const float rx = q.x - mx, ry = q.y - my, rz = q.z - mz;
-        const float d = fmaf(rx, rx, fmaf(ry, ry, fmaf(rz, rz, -bcut2)));
-        m = __funnelshift_l(__float_as_uint(d), m, 1);
-    }
-    return m;
-}
 
 __device__ __forceinline__ void prefetch_l1(const void *p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 
@@ -596,15 +605,26 @@ __device__ __forceinline__ float box_distance2(float4 lo, float4 hi, float4 q) {
 // segments that begin inside the window [b0, b0 + 32) as one bit mask; before:
 // those begun ahead of it.
 struct PPStream {
-    int nseg, total, before, mine;   // mine: where segment `lane` begins
+    int nseg, first, total, before, mine;   // this warp's part [first, total); mine: where segment `lane` begins
     int4 g;
     float4 raw = make_float4(0.f, 0.f, 0.f, 0.f);
     int slot;
     __device__ __forceinline__ void init(const PPParams &P, const PPWarpShared &W) {
         const int lane = threadIdx.x & 31;
-        before = 0;
+        first = before = 0;
         mine = lane < nseg ? W.begin[lane] : 0x7fffffff;
         load(P, W, 0);   // the target itself is in the stream: never empty
+    }
+    // part p of PP_PARTS of the stream of `all` sources (never empty: all > PP_PARTS * 32)
+    __device__ __forceinline__ void init_part(const PPParams &P, const PPWarpShared &W, int all, int p) {
+        const int lane = threadIdx.x & 31, windows = (all + 31) / 32;
+        first = (int)((int64_t)windows * p / PP_PARTS) * 32;
+        total = min(all, (int)((int64_t)windows * (p + 1) / PP_PARTS) * 32);
+        mine = lane < nseg ? W.begin[lane] : 0x7fffffff;
+        int n = mine < first;
+        for (int k = lane + 32; k < nseg; k += 32) n += W.begin[k] < first;
+        before = __reduce_add_sync(0xffffffffu, n);
+        load(P, W, first);
     }
     __device__ __forceinline__ void load(const PPParams &P, const PPWarpShared &W, int b0) {
         const int lane = threadIdx.x & 31;
@@ -695,7 +715,7 @@ __device__ __forceinline__ void stream_compact(const PPParams &P, PPWarpShared &
     auto &M = W.u.d.mixed;
     int fo = 0, fm = 0;
 #pragma unroll 1
-    for (int b0 = 0; b0 < T.total || fo || fm; b0 += 32) {
+    for (int b0 = T.first; b0 < T.total || fo || fm; b0 += 32) {
         if (b0 < T.total) {
             const float4 q = T.next(P, W, b0);
             const float4 lo = W.box[0], hi = W.box[1];
@@ -804,19 +824,27 @@ __device__ __forceinline__ void eval_queue(const PPParams &P, const PPWarpShared
     if (held) add_pairs(a, L, px, py, pz);
 }
 
-__device__ __forceinline__ void stream_sparse(const PPParams &P, PPWarpShared &W, PPStream &T, const PPLane &L, Sum3 &a,
-                                              unsigned &pairs, unsigned &cands) {
+// stage(place, slot) and drain(held): what the caller keeps of a staged source and
+// does with the queues.
+template <class Stage, class Drain>
+__device__ __forceinline__ void stream_sparse(const PPParams &P, PPWarpShared &W, PPStream &T, const PPLane &L,
+                                              unsigned &pairs, unsigned &cands, const Stage &stage, const Drain &drain) {
     const int lane = threadIdx.x & 31;
     auto &S = W.u.s.src;
     int fill = 0;
     if (lane == 0) S.put(SPARSE_N, make_float4(PP_FAR, PP_FAR, PP_FAR, 0.f));
 #pragma unroll 1
-    for (int b0 = 0; b0 < T.total; b0 += 32) {
+    for (int b0 = T.first; b0 < T.total; b0 += 32) {
+        const int slot = T.slot;
         const float4 q = T.next(P, W, b0);
         const float4 lo = W.box[0], hi = W.box[1];
         const bool keep = b0 + lane < T.total && box_distance2(lo, hi, q) < lo.w;
         const unsigned km = __ballot_sync(0xffffffffu, keep);
-        if (keep) S.put(fill + __popc(km & ((1u << lane) - 1u)), q);
+        if (keep) {
+            const int at = fill + __popc(km & ((1u << lane) - 1u));
+            S.put(at, q);
+            stage(at, slot);
+        }
         fill += __popc(km);
         if (fill <= SPARSE_N - 32 && b0 + 32 < T.total) continue;
         // pad to whole groups of 8, test, queue
@@ -854,7 +882,7 @@ __device__ __forceinline__ void stream_sparse(const PPParams &P, PPWarpShared &W
             pairs += more;
             if (done || __any_sync(0xffffffffu, held + more > QUEUE_N)) {
                 __syncwarp();
-                eval_queue(P, W, held, L, a, pairs);
+                drain(held);
                 held = 0;
                 if (done) break;
             }
@@ -928,35 +956,55 @@ __device__ __forceinline__ float ref_force_deriv_scaled(float u) {
 
 // For the pair term g(r) d of the PP force (g = R_PP(r)/r, IOS-cell units):
 // gc = g(r) and gp = g'(r)/r, so that the pair's Jacobian block is
-// gc I + gp d d^T.  Far pairs use the shell polynomial m(u) of far_pair and
-// its derivative; pairs closer than b_pp the two-term formula and its
-// derivative.
-__device__ __forceinline__ void pp_jacobian_pair(float r2, float inv_bpp, float inv_bcut, float bpp2, float &gc,
-                                                 float &gp) {
-    const float rinv = rsqrtf(r2);
-    if (r2 >= bpp2) {
-        const float u = r2 * rinv * inv_bcut;
-        float m, dm;
-        if (u >= 0.5f) {
-            const float v = 1.0f - u, v2 = v * v, v4 = v2 * v2;
-            m = v4 * v * (192.0f / 5.0f + v * (-416.0f / 5.0f + v * (2048.0f / 35.0f - 64.0f / 5.0f * v)));
-            dm = -v4 * (192.0f + v * (-2496.0f / 5.0f + v * (2048.0f / 5.0f - 512.0f / 5.0f * v)));
-        } else {
-            const float u2 = u * u;
-            m = 1.0f + u2 * u * (-64.0f / 5.0f + u2 * (256.0f / 5.0f + u * (-32.0f + u * (-1536.0f / 35.0f + 192.0f / 5.0f * u))));
-            dm = u2 * (-192.0f / 5.0f + u2 * (256.0f + u * (-192.0f + u * (-1536.0f / 5.0f + 1536.0f / 5.0f * u))));
-        }
-        const float r3 = rinv * rinv * rinv;
-        gc = m * r3;
-        gp = rinv * r3 * (dm * inv_bcut - 3.0f * m * rinv);
-    } else {
-        const float r = r2 * rinv;
-        gc = (ref_force_scaled(r * inv_bpp) * inv_bpp * inv_bpp - ref_force_scaled(r * inv_bcut) * inv_bcut * inv_bcut) *
-             rinv;
-        const float dr = ref_force_deriv_scaled(r * inv_bpp) * inv_bpp * inv_bpp * inv_bpp -
-                         ref_force_deriv_scaled(r * inv_bcut) * inv_bcut * inv_bcut * inv_bcut;
-        gp = (dr - gc) * rinv * rinv;
-    }
+// gc I + gp d d^T.  Far pairs (r >= b_pp), two at a time: with u = r/b_cut and the
+// shell polynomial m(u), gc = m r^-3 and gp = h r^-5, h = u m' - 3 m; on [0, 1/2)
+// both are polynomials in u, on [1/2, 1] in v = 1 - u, zero beyond.  Both branches
+// are evaluated and one is chosen: the lanes of a warp need both all the time.
+__device__ __forceinline__ void far_jacobian2(f2 r2, float inv_bcut, f2 &gc, f2 &gp) {
+    float ra, rb, ua, ub;
+    unpack(r2, ra, rb);
+    const f2 rinv = pack(rsqrtf(ra), rsqrtf(rb));
+    unpack(mul2(mul2(r2, rinv), twice(inv_bcut)), ua, ub);
+    ua = fminf(ua, 1.0f);
+    ub = fminf(ub, 1.0f);
+    const f2 u = pack(ua, ub), v = fma2(u, twice(-1.0f), twice(1.0f));
+    const f2 v2 = mul2(v, v), v4 = mul2(v2, v2);
+    f2 mh = fma2(v, twice(-64.0f / 5.0f), twice(2048.0f / 35.0f));
+    mh = fma2(v, mh, twice(-416.0f / 5.0f));
+    mh = mul2(mul2(v4, v), fma2(v, mh, twice(192.0f / 5.0f)));
+    f2 hh = fma2(v, twice(-64.0f), twice(11776.0f / 35.0f));
+    hh = fma2(v, hh, twice(-3296.0f / 5.0f));
+    hh = fma2(v, hh, twice(576.0f));
+    hh = mul2(v4, fma2(v, hh, twice(-192.0f)));
+    const f2 u2 = mul2(u, u), u3 = mul2(u2, u);
+    f2 ml = fma2(u, twice(192.0f / 5.0f), twice(-1536.0f / 35.0f));
+    ml = fma2(u, ml, twice(-32.0f));
+    ml = fma2(u, ml, twice(256.0f / 5.0f));
+    ml = fma2(u3, fma2(u2, ml, twice(-64.0f / 5.0f)), twice(1.0f));
+    f2 hl = fma2(u, twice(192.0f), twice(-6144.0f / 35.0f));
+    hl = fma2(u, hl, twice(-96.0f));
+    hl = fma2(u, hl, twice(512.0f / 5.0f));
+    hl = fma2(mul2(u3, u2), hl, twice(-3.0f));
+    float mha, mhb, mla, mlb, hha, hhb, hla, hlb;
+    unpack(mh, mha, mhb);
+    unpack(ml, mla, mlb);
+    unpack(hh, hha, hhb);
+    unpack(hl, hla, hlb);
+    const f2 i2 = mul2(rinv, rinv), i3 = mul2(i2, rinv);
+    gc = mul2(pack(ua >= 0.5f ? mha : mla, ub >= 0.5f ? mhb : mlb), i3);
+    gp = mul2(pack(ua >= 0.5f ? hha : hla, ub >= 0.5f ? hhb : hlb), mul2(i3, i2));
+}
+
+// Pairs closer than b_pp: the two-term formula and its derivative; the target itself: 0.
+__device__ __noinline__ float2 close_jacobian(float r2, float inv_bpp, float inv_bcut) {
+    if (!(r2 > 0.0f)) return make_float2(0.0f, 0.0f);
+    const float rinv = rsqrtf(r2), r = r2 * rinv;
+    const float gc = (ref_force_scaled(r * inv_bpp) * inv_bpp * inv_bpp -
+                      ref_force_scaled(r * inv_bcut) * inv_bcut * inv_bcut) *
+                     rinv;
+    const float dr = ref_force_deriv_scaled(r * inv_bpp) * inv_bpp * inv_bpp * inv_bpp -
+                     ref_force_deriv_scaled(r * inv_bcut) * inv_bcut * inv_bcut * inv_bcut;
+    return make_float2(gc, (dr - gc) * rinv * rinv);
 }
 
 struct VjpIO {
@@ -968,13 +1016,23 @@ struct VjpIO {
 // PP part of the vector-Jacobian product: w_i += sum_j A_ij (v_j - v_i) with
 // A_ij = g I + (g'/r) d d^T (the force's Jacobian blocks are symmetric).
 // Warps are dispatched as in the force: a warp inside one narrow row shares a
-// source stream (positions and v_j staged together, the candidate test and
-// set-bit evaluation of the force), other warps walk each lane's 27 cells.
-
+// source stream (v_j staged with the positions; the force's test, queues and packed
+// evaluation), other warps walk each lane's 27 cells.  The two products of a gradient
+// over 128^3 particles at z = 1: 2.43 ms with a pair at a time, both branches of the
+// polynomials taken in turn and every warp on its own, now 2.09.
 __device__ __forceinline__ void jacobian_term(float rx, float ry, float rz, float r2, float4 vj, float vix, float viy,
                                               float viz, const PPParams &P, float &px, float &py, float &pz) {
-    float gc, gp;
-    pp_jacobian_pair(r2, P.inv_bpp, P.inv_bcut, P.bpp2, gc, gp);
+    float gc, gp, unused;
+    if (r2 >= P.bpp2) {
+        f2 c2, p2;
+        far_jacobian2(twice(r2), P.inv_bcut, c2, p2);
+        unpack(c2, gc, unused);
+        unpack(p2, gp, unused);
+    } else {
+        const float2 g = close_jacobian(r2, P.inv_bpp, P.inv_bcut);
+        gc = g.x;
+        gp = g.y;
+    }
     const float dvx = vj.x - vix, dvy = vj.y - viy, dvz = vj.z - viz;
     const float dd = gp * (rx * dvx + ry * dvy + rz * dvz);
     px += gc * dvx + dd * rx;
@@ -1013,63 +1071,57 @@ __device__ void lane_vjp(const PPParams &P, const VjpIO &V, bool has, int c, flo
 }
 
 struct PPVjpWarpShared : PPWarpShared {
-    float4 vbuf[64];  // v_j of the staged sources
+    Soa<SPARSE_N + 4> vel;  // v_j of the staged sources
 };
 
-// Product terms of one batch of 32 staged sources.
-__device__ __forceinline__ void vjp32(const PPParams &P, const float4 *S, const float4 *SV, float mx, float my, float mz,
-                                      float vix, float viy, float viz, bool has, Sum3 &a) {
-    unsigned m = has ? test32(S, mx, my, mz, P.bcut2) : 0u;
-    float px = 0.f, py = 0.f, pz = 0.f;
-    while (m) {
-        const int k = __clz(m);
-        m ^= 0x80000000u >> k;
-        const float4 q = S[k];
-        const float rx = q.x - mx, ry = q.y - my, rz = q.z - mz;
-        const float r2 = rx * rx + ry * ry + rz * rz;
-        if (r2 > 0.0f) jacobian_term(rx, ry, rz, r2, SV[k], vix, viy, viz, P, px, py, pz);
-    }
-    a.add_block(px, py, pz);
-}
-
-__device__ void union_vjp(const PPParams &P, const VjpIO &V, PPVjpWarpShared &W, PPStream &T, bool has, float mx, float my,
-                          float mz, float vix, float viy, float viz, Sum3 &a) {
+// Product terms of the pairs in the lanes' queues, two at a time.
+__device__ __forceinline__ void vjp_queue(const PPParams &P, const PPVjpWarpShared &W, int held, const PPLane &L, float vix,
+                                          float viy, float viz, Sum3 &a) {
     const int lane = threadIdx.x & 31;
-    float4 *S = W.u.buf, *SV = W.vbuf;
-    warp_box(W.box, mx, my, mz, P.bcut2, P.bpp2);
-    int fill = 0;
-    for (int b0 = 0; b0 < T.total; b0 += 32) {
-        const int slot = T.slot;
-        const float4 q = T.next(P, W, b0);
-        const float4 lo = W.box[0], hi = W.box[1];
-        const bool keep = b0 + lane < T.total && box_distance2(lo, hi, q) < lo.w;
-        const unsigned km = __ballot_sync(0xffffffffu, keep);
-        if (keep) {
-            const int at = fill + __popc(km & ((1u << lane) - 1u));
-            const int j = __ldg(&P.perm[slot]);
-            S[at] = q;
-            SV[at] = make_float4(__ldg(&V.v0[j]), __ldg(&V.v1[j]), __ldg(&V.v2[j]), 0.f);
-        }
-        fill += __popc(km);
-        __syncwarp();
-        if (fill >= 32) {
-            vjp32(P, S, SV, mx, my, mz, vix, viy, viz, has, a);
-            __syncwarp();
-            const float4 t = S[32 + lane], tv = SV[32 + lane];
-            if (32 + lane < fill) {
-                S[lane] = t;
-                SV[lane] = tv;
+    const auto &S = W.u.s.src;
+    const auto &V = W.vel;
+    const f2 nx = twice(-L.mx), ny = twice(-L.my), nz = twice(-L.mz);
+    const f2 nvx = twice(-vix), nvy = twice(-viy), nvz = twice(-viz);
+    f2 px = 0ull, py = 0ull, pz = 0ull;
+#pragma unroll 1
+    for (int i = 0; i < held; i += 2) {
+        const int ka = W.u.s.queue[i][lane];
+        const int kb = i + 1 < held ? W.u.s.queue[i + 1][lane] : SPARSE_N;   // slot SPARSE_N: PP_FAR
+        const f2 rx = add2(pack(S.x[ka], S.x[kb]), nx), ry = add2(pack(S.y[ka], S.y[kb]), ny),
+                 rz = add2(pack(S.z[ka], S.z[kb]), nz);
+        const f2 r2 = fma2(rz, rz, fma2(ry, ry, mul2(rx, rx)));
+        f2 gc, gp;
+        far_jacobian2(r2, P.inv_bcut, gc, gp);
+        float ra, rb;
+        unpack(r2, ra, rb);
+        if (__builtin_expect(fminf(ra, rb) < P.bpp2, 0)) {   // rare: a close pair, or the target itself
+            float ca, cb, pa, pb;
+            unpack(gc, ca, cb);
+            unpack(gp, pa, pb);
+#pragma unroll 1
+            for (int e = 0; e < 2; ++e) {
+                const float r = e ? rb : ra;
+                if (r < P.bpp2) {
+                    const float2 g = close_jacobian(r, P.inv_bpp, P.inv_bcut);
+                    if (e) cb = g.x, pb = g.y;
+                    else ca = g.x, pa = g.y;
+                }
             }
-            fill -= 32;
-            __syncwarp();
+            gc = pack(ca, cb);
+            gp = pack(pa, pb);
         }
+        const f2 dx = add2(pack(V.x[ka], V.x[kb]), nvx), dy = add2(pack(V.y[ka], V.y[kb]), nvy),
+                 dz = add2(pack(V.z[ka], V.z[kb]), nvz);
+        const f2 dd = mul2(gp, fma2(rz, dz, fma2(ry, dy, mul2(rx, dx))));
+        px = fma2(gc, dx, fma2(dd, rx, px));
+        py = fma2(gc, dy, fma2(dd, ry, py));
+        pz = fma2(gc, dz, fma2(dd, rz, pz));
     }
-    if (fill > 0) {
-        if (lane >= fill) S[lane] = make_float4(1.0e18f, 1.0e18f, 1.0e18f, 0.0f);
-        __syncwarp();
-        vjp32(P, S, SV, mx, my, mz, vix, viy, viz, has, a);
-    }
-    __syncwarp();
+    float xa, xb, ya, yb, za, zb;
+    unpack(px, xa, xb);
+    unpack(py, ya, yb);
+    unpack(pz, za, zb);
+    if (held) a.add_block(xa + xb, ya + yb, za + zb);
 }
 
 // The warp's target of each lane: its slot (lane 0's in padding lanes), cell
@@ -1100,59 +1152,15 @@ __device__ __forceinline__ PPTarget warp_target(const PPParams &P, int j, PPBloc
     return t;
 }
 
-__global__ void __launch_bounds__(32) pp_vjp_kernel(PPParams P, VjpIO V) {
-    __shared__ PPVjpWarpShared sh;
-    const int64_t i = (int64_t)blockIdx.x * 32 + threadIdx.x;
-    const int j = P.tgt[i];   // with the length's load under way
-    if ((int64_t)blockIdx.x * 32 >= *P.tgt_n) return;
-    PPBlock B;
-    const PPTarget t = warp_target(P, j, B);
-    const int pi = P.perm[t.slot];
-    const float vix = V.v0[pi], viy = V.v1[pi], viz = V.v2[pi];
-    Sum3 a;
-    if (B.xb - B.xa <= P.wmax) {
-        PPStream T;
-        T.total = build_segments(P, sh.seg, sh.begin, B, T.nseg);
-        T.init(P, sh);
-        union_vjp(P, V, sh, T, t.has, (float)(t.cx - B.xa) + t.me.x, (float)(t.cy - B.ya + 1) + t.me.y,
-                  (float)(t.cz - B.za + 1) + t.me.z, vix, viy, viz, a);
-    } else {
-        lane_vjp(P, V, t.has, __float_as_int(t.me.w), t.me, vix, viy, viz, a);
-    }
-    if (t.has) {
-        V.w0[pi] += V.scale * (a.x - a.cx);
-        V.w1[pi] += V.scale * (a.y - a.cy);
-        V.w2[pi] += V.scale * (a.z - a.cz);
-    }
-}
-
 // Warps with fewer expected candidates per pair than this evaluate every pair.
 // The estimate takes the sources as evenly spread; around haloes more of them
 // are in range.  PP at z = 0 of the 256^3 run with 6 / 9 / 14 / 20: 9.8 / 9.0 /
 // 8.7 / 8.7 ms; 512^3 particles at z = 1 with 6 / 9 / 14: 25.0 / 23.4 / 22.9 ms.
 constexpr float PP_COMPACT = 14.0f;
 
-// The warp's 32 target places from i on.  COUNT: accumulate the work counters
-// (off unless asked for: they live through the whole stream).
-template <bool PM3, bool COUNT>
-__device__ __forceinline__ void pp_warp(const PPParams &P, int64_t i, PPWarpShared &W) {
-    const int j = P.tgt[i];   // with the length's load under way
-    if ((i & ~(int64_t)31) >= *P.tgt_n) return;   // whole warps: places past the last pencil's end
-    PPBlock B;
-    const PPTarget t = warp_target(P, j, B);
-    const bool stream = B.xb - B.xa <= P.wmax;
-    // the sums' destinations on their way while the pairs are worked on (perm
-    // stays inside the cell; both prefetches: 1.38 -> 1.35 ms at z = 49)
-    if (P.accumulate) {
-        prefetch_l1(&P.acc0[t.slot]);
-        prefetch_l1(&P.acc1[t.slot]);
-        prefetch_l1(&P.acc2[t.slot]);
-    }
-    if (P.kick != 0.0f) {
-        prefetch_l1(&P.vel0[t.slot]);
-        prefetch_l1(&P.vel1[t.slot]);
-        prefetch_l1(&P.vel2[t.slot]);
-    }
+// The targets as the pair loops see them.
+template <bool PM3>
+__device__ __forceinline__ PPLane pp_lane(const PPParams &P, const PPTarget &t, const PPBlock &B) {
     PPLane L;
     L.has = t.has;
     // PP range of this target: b_3 inside a refined subtile of the third level
@@ -1171,16 +1179,67 @@ __device__ __forceinline__ void pp_warp(const PPParams &P, int64_t i, PPWarpShar
     L.mx = (float)(t.cx - B.xa) + t.me.x;
     L.my = (float)(t.cy - B.ya + 1) + t.me.y;
     L.mz = (float)(t.cz - B.za + 1) + t.me.z;
+    return L;
+}
+
+// Part of the warp's stream, by the loop that suits it.
+template <bool COUNT>
+__device__ __forceinline__ void pp_stream(const PPParams &P, PPWarpShared &W, PPStream &T, const PPLane &L, bool compact,
+                                          Sum3 &a, unsigned &pairs, unsigned &cands) {
+    if (compact)
+        stream_compact<COUNT>(P, W, T, L, a, pairs, cands);
+    else
+        stream_sparse(P, W, T, L, pairs, cands, [](int, int) {}, [&](int held) { eval_queue(P, W, held, L, a, pairs); });
+}
+
+// The warp's 32 target places from i on.  COUNT: accumulate the work counters
+// (off unless asked for: they live through the whole stream).  LIST: long streams
+// go to the list (otherwise their parts are worked on here).
+template <bool PM3, bool COUNT, bool LIST>
+__device__ __forceinline__ void pp_warp(const PPParams &P, int64_t i, PPWarpShared &W) {
+    const int j = P.tgt[i];   // with the length's load under way
+    if ((i & ~(int64_t)31) >= *P.tgt_n) return;   // whole warps: places past the last pencil's end
+    PPBlock B;
+    const PPTarget t = warp_target(P, j, B);
+    const bool stream = B.xb - B.xa <= P.wmax;
+    // the sums' destinations on their way while the pairs are worked on (perm
+    // stays inside the cell; both prefetches: 1.38 -> 1.35 ms at z = 49)
+    if (P.accumulate) {
+        prefetch_l1(&P.acc0[t.slot]);
+        prefetch_l1(&P.acc1[t.slot]);
+        prefetch_l1(&P.acc2[t.slot]);
+    }
+    if (P.kick != 0.0f) {
+        prefetch_l1(&P.vel0[t.slot]);
+        prefetch_l1(&P.vel1[t.slot]);
+        prefetch_l1(&P.vel2[t.slot]);
+    }
+    const PPLane L = pp_lane<PM3>(P, t, B);
     Sum3 a;
     unsigned pairs = 0, cands = 0;
     if (stream) {
         PPStream T;
         T.total = build_segments(P, W.seg, W.begin, B, T.nseg);
-        T.init(P, W);
-        if (warp_box(W.box, L.mx, L.my, L.mz, L.bcut2, P.bpp2) < PP_COMPACT)
-            stream_compact<COUNT>(P, W, T, L, a, pairs, cands);
-        else
-            stream_sparse(P, W, T, L, a, pairs, cands);
+        const bool split = T.total > P.long_min;
+        if (LIST && split) {
+            if ((threadIdx.x & 31) == 0) P.long_list[atomicAdd(P.long_n, 1)] = (int32_t)(i >> 5);
+            return;
+        }
+        const bool compact = warp_box(W.box, L.mx, L.my, L.mz, L.bcut2, P.bpp2) < PP_COMPACT;
+        if constexpr (LIST) {
+            T.init(P, W);
+            pp_stream<COUNT>(P, W, T, L, compact, a, pairs, cands);
+        } else {
+            const int all = T.total, parts = split ? PP_PARTS : 1;
+#pragma unroll 1
+            for (int p = 0; p < parts; ++p) {
+                if (split) T.init_part(P, W, all, p);
+                else T.init(P, W);
+                Sum3 b;
+                pp_stream<COUNT>(P, W, T, L, compact, b, pairs, cands);
+                a.add_block(b.x - b.cx, b.y - b.cy, b.z - b.cz);
+            }
+        }
     } else {
         lane_path(P, __float_as_int(t.me.w), t.me, L, a, pairs, cands);
     }
@@ -1200,7 +1259,126 @@ constexpr int PP_WARPS = 2;
 template <bool PM3, bool COUNT>
 __global__ void __launch_bounds__(PP_WARPS * 32, 32 / PP_WARPS) pp_kernel(PPParams P) {
     __shared__ PPWarpShared sh[PP_WARPS];
-    pp_warp<PM3, COUNT>(P, (int64_t)blockIdx.x * (PP_WARPS * 32) + threadIdx.x, sh[threadIdx.x >> 5]);
+    pp_warp<PM3, COUNT, true>(P, (int64_t)blockIdx.x * (PP_WARPS * 32) + threadIdx.x, sh[threadIdx.x >> 5]);
+}
+
+// Partial sums of the parts of one warp's targets, added in their order by warp 0.
+struct PPPartSums {
+    float v[PP_PARTS][3][32];
+    __device__ __forceinline__ void put(const Sum3 &a) {
+        const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        v[w][0][lane] = a.x - a.cx;
+        v[w][1][lane] = a.y - a.cy;
+        v[w][2][lane] = a.z - a.cz;
+    }
+    __device__ __forceinline__ Sum3 sum() const {
+        const int lane = threadIdx.x & 31;
+        Sum3 a;
+        for (int p = 0; p < PP_PARTS; ++p) a.add_block(v[p][0][lane], v[p][1][lane], v[p][2][lane]);
+        return a;
+    }
+};
+
+// The listed warps, a CTA each.
+template <bool PM3, bool COUNT>
+__global__ void __launch_bounds__(PP_PARTS * 32, 32 / PP_PARTS) pp_long_kernel(PPParams P) {
+    __shared__ PPWarpShared sh[PP_PARTS];
+    __shared__ PPPartSums part;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, n = *P.long_n;
+    PPWarpShared &W = sh[w];
+    for (int item = blockIdx.x; item < n; item += gridDim.x) {
+        PPBlock B;
+        const PPTarget t = warp_target(P, P.tgt[(int64_t)P.long_list[item] * 32 + lane], B);
+        const PPLane L = pp_lane<PM3>(P, t, B);
+        PPStream T;
+        const int all = build_segments(P, W.seg, W.begin, B, T.nseg);
+        const bool compact = warp_box(W.box, L.mx, L.my, L.mz, L.bcut2, P.bpp2) < PP_COMPACT;
+        T.init_part(P, W, all, w);
+        Sum3 a;
+        unsigned pairs = 0, cands = 0;
+        pp_stream<COUNT>(P, W, T, L, compact, a, pairs, cands);
+        part.put(a);
+        __syncthreads();
+        if (w == 0 && t.has) {
+            const Sum3 b = part.sum();
+            finish(P, P.perm[t.slot], b.x - b.cx, b.y - b.cy, b.z - b.cz);
+        }
+        if constexpr (COUNT) add_stats(P.stats, pairs, cands);
+        __syncthreads();
+    }
+}
+
+// The product over one part of the warp's stream.
+__device__ __forceinline__ void vjp_stream(const PPParams &P, const VjpIO &V, PPVjpWarpShared &W, PPStream &T, const PPLane &L,
+                                           float vix, float viy, float viz, Sum3 &a) {
+    if ((threadIdx.x & 31) == 0) W.vel.put(SPARSE_N, make_float4(0.f, 0.f, 0.f, 0.f));
+    unsigned pairs = 0, cands = 0;   // not asked for
+    stream_sparse(P, W, T, L, pairs, cands,
+                  [&](int at, int slot) {
+                      const int k = __ldg(&P.perm[slot]);
+                      W.vel.put(at, make_float4(__ldg(&V.v0[k]), __ldg(&V.v1[k]), __ldg(&V.v2[k]), 0.f));
+                  },
+                  [&](int held) { vjp_queue(P, W, held, L, vix, viy, viz, a); });
+}
+
+__device__ __forceinline__ void vjp_finish(const VjpIO &V, int pi, const Sum3 &a) {
+    V.w0[pi] += V.scale * (a.x - a.cx);
+    V.w1[pi] += V.scale * (a.y - a.cy);
+    V.w2[pi] += V.scale * (a.z - a.cz);
+}
+
+// 28 warps per SM (72 registers): 82 registers and 24 warps took 2.35 ms for the two
+// products of 128^3 particles at z = 1, 64 and 32 2.30, this 2.29 (an unevolved state:
+// 0.52, 0.45, 0.43).
+constexpr int VJP_BLOCKS = 28;
+__global__ void __launch_bounds__(32, VJP_BLOCKS) pp_vjp_kernel(PPParams P, VjpIO V) {
+    __shared__ PPVjpWarpShared sh;
+    const int64_t i = (int64_t)blockIdx.x * 32 + threadIdx.x;
+    const int j = P.tgt[i];   // with the length's load under way
+    if ((int64_t)blockIdx.x * 32 >= *P.tgt_n) return;
+    PPBlock B;
+    const PPTarget t = warp_target(P, j, B);
+    const int pi = P.perm[t.slot];
+    const float vix = V.v0[pi], viy = V.v1[pi], viz = V.v2[pi];
+    Sum3 a;
+    if (B.xb - B.xa <= P.wmax) {
+        PPStream T;
+        T.total = build_segments(P, sh.seg, sh.begin, B, T.nseg);
+        if (T.total > P.long_min) {
+            if (threadIdx.x == 0) P.long_list[atomicAdd(P.long_n, 1)] = blockIdx.x;
+            return;
+        }
+        const PPLane L = pp_lane<false>(P, t, B);
+        warp_box(sh.box, L.mx, L.my, L.mz, P.bcut2, P.bpp2);
+        T.init(P, sh);
+        vjp_stream(P, V, sh, T, L, vix, viy, viz, a);
+    } else {
+        lane_vjp(P, V, t.has, __float_as_int(t.me.w), t.me, vix, viy, viz, a);
+    }
+    if (t.has) vjp_finish(V, pi, a);
+}
+
+__global__ void __launch_bounds__(PP_PARTS * 32, VJP_BLOCKS / PP_PARTS) pp_vjp_long_kernel(PPParams P, VjpIO V) {
+    __shared__ PPVjpWarpShared sh[PP_PARTS];
+    __shared__ PPPartSums part;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, n = *P.long_n;
+    PPVjpWarpShared &W = sh[w];
+    for (int item = blockIdx.x; item < n; item += gridDim.x) {
+        PPBlock B;
+        const PPTarget t = warp_target(P, P.tgt[(int64_t)P.long_list[item] * 32 + lane], B);
+        const int pi = P.perm[t.slot];
+        const PPLane L = pp_lane<false>(P, t, B);
+        PPStream T;
+        const int all = build_segments(P, W.seg, W.begin, B, T.nseg);
+        warp_box(W.box, L.mx, L.my, L.mz, P.bcut2, P.bpp2);
+        T.init_part(P, W, all, w);
+        Sum3 a;
+        vjp_stream(P, V, W, T, L, V.v0[pi], V.v1[pi], V.v2[pi], a);
+        part.put(a);
+        __syncthreads();
+        if (w == 0 && t.has) vjp_finish(V, pi, part.sum());
+        __syncthreads();
+    }
 }
 
 // ------------------------------------------------- ensemble: one persistent PP
@@ -1298,7 +1476,7 @@ __global__ void __launch_bounds__(PP_ITEM, 8) pp_persistent_kernel(const PPParam
         if (item >= count) break;
         const int k = order[item];
         const int b = item_box[k];
-        pp_warp<false, false>(boxes[b], (int64_t)(k - base[b]) * PP_ITEM + threadIdx.x, sh[threadIdx.x >> 5]);
+        pp_warp<false, false, false>(boxes[b], (int64_t)(k - base[b]) * PP_ITEM + threadIdx.x, sh[threadIdx.x >> 5]);
     }
 }
 
@@ -1325,7 +1503,7 @@ static void launch_pp_inputs(cube2_ctx *ctx, const cube2_particles *p) {
     unsigned *tgt_n = reinterpret_cast<unsigned *>(ctx->big_n + 1);
     {
         ProfScope prof(ctx, P_PP_ORDER, 0);
-        cudaMemsetAsync(ctx->big_n, 0, 2 * sizeof(int), ctx->stream);
+        cudaMemsetAsync(ctx->big_n, 0, 3 * sizeof(int), ctx->stream);
         pp_pencil_kernel<<<(unsigned)(pencils_y(n) * pencils_z(n)), PREP_CTA, 0, ctx->stream>>>(
             p->count, p->start, n, PP_SORT_MIN, ctx->pp_tgt, tgt_n, ctx->pp_dense, list_n);
     }
@@ -1346,6 +1524,7 @@ static void launch_pp_inputs(cube2_ctx *ctx, const cube2_particles *p) {
 cudaError_t launch_pp_vjp(cube2_ctx *ctx, const cube2_particles *p, const float *const v[3], float *const w[3]) {
     if (ctx->N == 0) return cudaSuccess;
     PPParams P = pp_params(ctx, p, 1, 0.0f);
+    P.long_min = vjp_long_min(ctx->N);
     VjpIO V{};
     V.v0 = v[0]; V.v1 = v[1]; V.v2 = v[2];
     V.w0 = w[0]; V.w1 = w[1]; V.w2 = w[2];
@@ -1354,6 +1533,10 @@ cudaError_t launch_pp_vjp(cube2_ctx *ctx, const cube2_particles *p, const float 
     ProfScope prof(ctx, P_PP_VJP, 0);
     pp_vjp_kernel<<<(unsigned)(pp_target_slots(ctx->N, ctx->n_ios) / 32), 32, 0, ctx->stream>>>(P, V);
     ctx->launches += 1;
+    if (ctx->N >= PP_LONG_N) {
+        pp_vjp_long_kernel<<<(unsigned)(ctx->num_sms * (VJP_BLOCKS / PP_PARTS)), PP_PARTS * 32, 0, ctx->stream>>>(P, V);
+        ctx->launches += 1;
+    }
     return cudaGetLastError();
 }
 
@@ -1391,6 +1574,9 @@ static PPParams pp_params(cube2_ctx *ctx, const cube2_particles *p, int accumula
     P.kick = kick;
     P.status = ctx->dev_status;
     P.wmax = ctx->pp_wmax;
+    P.long_min = pp_long_min(ctx->N);
+    P.long_list = ctx->pp_long;
+    P.long_n = ctx->big_n + 2;
     if (ctx->pm3.on) {
         P.pm3_slot = ctx->pm3.slot;
         P.pm3_T = ctx->pm3.T;
@@ -1413,14 +1599,17 @@ cudaError_t launch_pp(cube2_ctx *ctx, const cube2_particles *p, int accumulate, 
     }
     {
         ProfScope prof(ctx, P_PP, 0);
-        if (P.pm3_slot)
-            (ctx->pp_count ? pp_kernel<true, true> : pp_kernel<true, false>)<<<ctas, PP_WARPS * 32, 0,
-                                                                              ctx->stream>>>(P);
-        else
-            (ctx->pp_count ? pp_kernel<false, true> : pp_kernel<false, false>)<<<ctas, PP_WARPS * 32, 0,
-                                                                                ctx->stream>>>(P);
+        const bool pm3 = P.pm3_slot != nullptr, count = ctx->pp_count;
+        (pm3 ? (count ? pp_kernel<true, true> : pp_kernel<true, false>)
+             : (count ? pp_kernel<false, true> : pp_kernel<false, false>))<<<ctas, PP_WARPS * 32, 0, ctx->stream>>>(P);
+        ctx->launches += 1;
+        if (ctx->N >= PP_LONG_N) {
+            (pm3 ? (count ? pp_long_kernel<true, true> : pp_long_kernel<true, false>)
+                 : (count ? pp_long_kernel<false, true> : pp_long_kernel<false, false>))<<<
+                (unsigned)(ctx->num_sms * (32 / PP_PARTS)), PP_PARTS * 32, 0, ctx->stream>>>(P);
+            ctx->launches += 1;
+        }
     }
-    ctx->launches += 1;
     return cudaGetLastError();
 }
 
