@@ -482,7 +482,8 @@ int cube2_ensemble_create(cube2_ensemble **out, cube2_ctx *const *ctxs, cube2_pa
  *                   (cube2_ensemble_check) and returns.  Boxes with the third
  *                   level or FP16 velocities are refused (CUBE2_ERR_STATE).
  *   pp_ctas_per_sm  persistent grid: CTAs per SM (1..16)
- *   pp_wmax         PP shared-stream width along x for every box (0: each context's own, 64)
+ *   pp_wmax         0..64, accepted and without effect: the widest shared PP stream is
+ *                   the same everywhere, so that every option gives the same bits
  *   timeout_ms      bound of the persistent kernel's wait (> 0)                  */
 typedef struct {
     int32_t n_streams;
@@ -510,7 +511,7 @@ int cube2_ensemble_publish(cube2_ensemble *ens, int on);
 
 /* Autotuner of the runtime knobs: starting from *best (persistent_pp and
  * timeout_ms kept), a coordinate search over pp_ctas_per_sm in {4, 8, 16}
- * (persistent only), pp_wmax in {8, 16, 24} and n_streams in {8, 16, 32}; each
+ * (persistent only) and n_streams in {8, 16, 32} (pp_wmax is left as it is); each
  * candidate is recorded and timed with CUDA events on `stream` (the fastest of
  * `trials` launches after one warm-up launch), every launch starting from the
  * boxes' states at the call (snapshotted in scratch that this call allocates

@@ -135,8 +135,6 @@ struct cube2_ctx {
     double *vjp_sq = nullptr;      // [1] loss accumulator
     cube2::PM3 pm3;                // adaptive third level (cfg.pm3_tile > 0)
     float *vel32 = nullptr;        // [3][N] FP32 working momenta of a step (cfg.vel_fp16 = 1 only)
-    // shared-stream width of the PP kernel (warps spanning at most pp_wmax + 1 cells along x)
-    int pp_wmax = 64;
     // PP work counters (cube2_pp_count): off unless asked for
     bool pp_count = false;
     // ensemble recording: launch_pp prepares the PP inputs and leaves the PP

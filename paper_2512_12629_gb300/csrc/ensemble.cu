@@ -194,11 +194,6 @@ int cube2_ensemble_create_ex(cube2_ensemble **out, cube2_ctx *const *ctxs, cube2
     }
     int num_sms = 152;
     cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, ctxs[0]->device);
-    std::vector<int> wmax_saved(n_boxes);
-    for (int b = 0; b < n_boxes; ++b) {
-        wmax_saved[b] = ctxs[b]->pp_wmax;
-        if (opts->pp_wmax > 0) ctxs[b]->pp_wmax = opts->pp_wmax;
-    }
 
     int status = CUBE2_OK;
     e = cudaStreamBeginCapture(E->origin, cudaStreamCaptureModeThreadLocal);
@@ -250,10 +245,7 @@ int cube2_ensemble_create_ex(cube2_ensemble **out, cube2_ctx *const *ctxs, cube2
                     timeout_ns, num_sms * opts->pp_ctas_per_sm);
         }
     }
-    for (int b = 0; b < n_boxes; ++b) {
-        ctxs[b]->pp_wmax = wmax_saved[b];
-        ctxs[b]->defer_pp = false;
-    }
+    for (int b = 0; b < n_boxes; ++b) ctxs[b]->defer_pp = false;
     for (int b = 0; b < n_boxes; ++b) E->particle_steps += (int64_t)n_steps * ctxs[b]->N;
     cudaGraph_t g = nullptr;
     const cudaError_t ec = cudaStreamEndCapture(E->origin, &g);
@@ -391,16 +383,14 @@ int cube2_ensemble_autotune(cube2_ctx *const *ctxs, cube2_particles *const *part
     cube2_ensemble_opts cur = *best;
     double cur_ms = 0.0;
     if (status == CUBE2_OK) status = measure(cur, &cur_ms);
-    const int ctas[] = {4, 8, 16}, wmax[] = {8, 16, 24}, streams[] = {8, 16, 32};
-    for (int knob = 0; knob < 3 && status == CUBE2_OK; ++knob) {
+    const int ctas[] = {4, 8, 16}, streams[] = {8, 16, 32};
+    for (int knob = 0; knob < 2 && status == CUBE2_OK; ++knob) {
         if (knob == 0 && !cur.persistent_pp) continue;
         for (int i = 0; i < 3 && status == CUBE2_OK; ++i) {
             cube2_ensemble_opts t = cur;
             if (knob == 0) t.pp_ctas_per_sm = ctas[i];
-            if (knob == 1) t.pp_wmax = wmax[i];
-            if (knob == 2) t.n_streams = streams[i];
-            if (t.pp_ctas_per_sm == cur.pp_ctas_per_sm && t.pp_wmax == cur.pp_wmax && t.n_streams == cur.n_streams)
-                continue;
+            if (knob == 1) t.n_streams = streams[i];
+            if (t.pp_ctas_per_sm == cur.pp_ctas_per_sm && t.n_streams == cur.n_streams) continue;
             double ms = 0.0;
             status = measure(t, &ms);
             if (status == CUBE2_OK && ms < cur_ms) {

@@ -64,7 +64,6 @@ struct PPParams {
     const int32_t *pm3_slot;
     int pm3_T, pm3_ns;
     float bcut2_3, inv_bcut_3;
-    int wmax;                         // widest warp along x (cells beyond the first) on the shared stream
     int long_min;                     // longer streams go to the list and are shared by PP_PARTS warps
     int32_t *long_list;               // target places / 32 of those warps
     int *long_n;
@@ -354,9 +353,11 @@ struct Sum3 {
 constexpr int PP_ROWS = (PEN_Y + 2) * (PEN_Z + 2);
 constexpr int PP_SEGS = 3 * PP_ROWS;
 
-// A warp is on the shared stream when it spans at most wmax + 1 cells along x
-// (PPParams.wmax, the context's pp_wmax); the few wider ones (fewer than 32
-// particles in that many slabs) walk each lane's own 27 cells.
+// A warp is on the shared stream when it spans at most PP_WIDEST + 1 cells along x;
+// the few wider ones (fewer than 32 particles in that many slabs) walk each lane's own
+// 27 cells.  The line is the same for every launch: the two paths add in different
+// orders, and an ensemble gives its boxes the bits of their own steps.
+constexpr int PP_WIDEST = 64;
 
 struct PPBlock {
     int xa, xb, ya, yb, za, zb;
@@ -1201,7 +1202,7 @@ __device__ __forceinline__ void pp_warp(const PPParams &P, int64_t i, PPWarpShar
     if ((i & ~(int64_t)31) >= *P.tgt_n) return;   // whole warps: places past the last pencil's end
     PPBlock B;
     const PPTarget t = warp_target(P, j, B);
-    const bool stream = B.xb - B.xa <= P.wmax;
+    const bool stream = B.xb - B.xa <= PP_WIDEST;
     // the sums' destinations on their way while the pairs are worked on (perm
     // stays inside the cell; both prefetches: 1.38 -> 1.35 ms at z = 49)
     if (P.accumulate) {
@@ -1341,7 +1342,7 @@ __global__ void __launch_bounds__(32, VJP_BLOCKS) pp_vjp_kernel(PPParams P, VjpI
     const int pi = P.perm[t.slot];
     const float vix = V.v0[pi], viy = V.v1[pi], viz = V.v2[pi];
     Sum3 a;
-    if (B.xb - B.xa <= P.wmax) {
+    if (B.xb - B.xa <= PP_WIDEST) {
         PPStream T;
         T.total = build_segments(P, sh.seg, sh.begin, B, T.nseg);
         if (T.total > P.long_min) {
@@ -1573,7 +1574,6 @@ static PPParams pp_params(cube2_ctx *ctx, const cube2_particles *p, int accumula
     P.coef = (float)(vp / (4.0 * 3.14159265358979323846) / (s * s));
     P.kick = kick;
     P.status = ctx->dev_status;
-    P.wmax = ctx->pp_wmax;
     P.long_min = pp_long_min(ctx->N);
     P.long_list = ctx->pp_long;
     P.long_n = ctx->big_n + 2;

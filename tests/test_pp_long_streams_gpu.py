@@ -108,3 +108,25 @@ def test_persistent_kernel_gives_the_same_bits(case):
     ens.close()
     for c in ctxs:
         c.close()
+
+
+@pytest.mark.parametrize("width", [8, 16])
+def test_stream_width_option_leaves_the_bits(width):
+    # thin boxes, whose warps span many cells: the option once moved them to the per-lane walk
+    rng = np.random.default_rng(3)
+    w = C1.with_(name="thin", n_ios=N_IOS, box=float(N_IOS), levels=(Level(N_IOS, 1.0),), b_pp=0.1)
+    x = rng.uniform(0, N_IOS, (3, 9000))
+    st = ios_from_positions(x, np.zeros_like(x), N_IOS, w.box)
+    ctx = cube2.init_mesh(cube2.make_config(w, n_particles=9000))
+    ctx.set_green(0)
+    p = cube2.IOSState.from_numpy(st)
+    ctx.force(p)
+    want = p.clone()
+    ctx.kdk_step(want, 0.5, 0.501)
+    ens = cube2.Ensemble([ctx], [p], np.array([[0.5, 0.501]]),
+                         opts=cube2.ensemble_opts(n_streams=1, persistent_pp=True, pp_wmax=width))
+    ens.launch()
+    ens.check()
+    assert torch.equal(p.acc, want.acc) and torch.equal(p.vel, want.vel) and torch.equal(p.off, want.off)
+    ens.close()
+    ctx.close()
