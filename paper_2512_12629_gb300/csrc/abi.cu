@@ -265,6 +265,7 @@ int cube2_init_mesh(cube2_ctx **out, const cube2_config *cfg, void *stream) {
     c->nl = cfg->n_levels;
     c->N = cfg->n_particles;
     c->n_ios = cfg->n_ios;
+    c->chained = cfg->n_particles <= CHAINED_MAX;
     c->n_cells = (int64_t)cfg->n_ios * cfg->n_ios * cfg->n_ios;
     c->s_ios = cfg->box / cfg->n_ios;
     double prev_b = -1.0;  // softening of the coarser level [Mpc/h]

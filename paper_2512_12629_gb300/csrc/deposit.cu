@@ -408,6 +408,7 @@ __device__ __forceinline__ void coarse_brick(const DepParams &P, int brick, unsi
 
 template <int UP, int BI>
 __global__ void __launch_bounds__(DEP_THREADS, 4) deposit_kernel(DepParams fine) {
+    chain();
     extern __shared__ __align__(16) unsigned int dep_words[];
     fine_brick<UP, BI>(fine, blockIdx.x, dep_words);
 }
@@ -419,12 +420,14 @@ __global__ void __launch_bounds__(DEP_THREADS, 4) deposit_kernel(DepParams fine)
 // fine ones' shared memory).  Figures with 256 threads.
 template <int UP, int BI>
 __global__ void __launch_bounds__(DEP_THREADS) deposit_both_kernel(DepParams fine, DepParams coarse, int n_coarse) {
+    chain();
     extern __shared__ __align__(16) unsigned int dep_words[];
     if ((int)blockIdx.x < n_coarse) coarse_brick(coarse, blockIdx.x, dep_words);
     else fine_brick<UP, BI>(fine, (int)blockIdx.x - n_coarse, dep_words);
 }
 
 __global__ void __launch_bounds__(DEP_THREADS) deposit_coarse_kernel(DepParams coarse) {
+    chain();
     extern __shared__ __align__(16) unsigned int dep_words[];
     coarse_brick(coarse, blockIdx.x, dep_words);
 }
@@ -432,7 +435,7 @@ __global__ void __launch_bounds__(DEP_THREADS) deposit_coarse_kernel(DepParams c
 int64_t bricks(const DepParams &P) { return (int64_t)P.nbx * P.nbx * P.nbx; }
 
 cudaError_t launch_coarse(cube2_ctx *ctx, const DepParams &coarse) {
-    deposit_coarse_kernel<<<(unsigned)bricks(coarse), DEP_THREADS, COARSE_SMEM, ctx->stream>>>(coarse);
+    launch_chained(ctx->chained, deposit_coarse_kernel, (unsigned)bricks(coarse), DEP_THREADS, COARSE_SMEM, ctx->stream, coarse);
     ctx->launches++;
     return cudaGetLastError();
 }
@@ -450,12 +453,12 @@ cudaError_t launch_fine(cube2_ctx *ctx, DepParams fine, const DepParams *coarse)
     }
     fine.nbx = (fine.n_ios + BI - 1) / BI;
     if (coarse && bricks(fine) <= BOTH_BRICKS) {
-        deposit_both_kernel<UP, BI><<<(unsigned)(bricks(*coarse) + bricks(fine)), DEP_THREADS, BOTH, ctx->stream>>>(
+        launch_chained(ctx->chained, deposit_both_kernel<UP, BI>, (unsigned)(bricks(*coarse) + bricks(fine)), DEP_THREADS, BOTH, ctx->stream,
             fine, *coarse, (int)bricks(*coarse));
     } else {
         const cudaError_t e = coarse ? launch_coarse(ctx, *coarse) : cudaSuccess;
         if (e != cudaSuccess) return e;
-        deposit_kernel<UP, BI><<<(unsigned)bricks(fine), DEP_THREADS, SMEM, ctx->stream>>>(fine);
+        launch_chained(ctx->chained, deposit_kernel<UP, BI>, (unsigned)bricks(fine), DEP_THREADS, SMEM, ctx->stream, fine);
     }
     ctx->launches++;
     return cudaGetLastError();

@@ -194,6 +194,11 @@ int cube2_ensemble_create_ex(cube2_ensemble **out, cube2_ctx *const *ctxs, cube2
     }
     int num_sms = 152;
     cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, ctxs[0]->device);
+    std::vector<char> chained(n_boxes);
+    for (int b = 0; b < n_boxes; ++b) {
+        chained[b] = ctxs[b]->chained;
+        ctxs[b]->chained = false;
+    }
 
     int status = CUBE2_OK;
     e = cudaStreamBeginCapture(E->origin, cudaStreamCaptureModeThreadLocal);
@@ -245,7 +250,10 @@ int cube2_ensemble_create_ex(cube2_ensemble **out, cube2_ctx *const *ctxs, cube2
                     timeout_ns, num_sms * opts->pp_ctas_per_sm);
         }
     }
-    for (int b = 0; b < n_boxes; ++b) ctxs[b]->defer_pp = false;
+    for (int b = 0; b < n_boxes; ++b) {
+        ctxs[b]->defer_pp = false;
+        ctxs[b]->chained = chained[b];
+    }
     for (int b = 0; b < n_boxes; ++b) E->particle_steps += (int64_t)n_steps * ctxs[b]->N;
     cudaGraph_t g = nullptr;
     const cudaError_t ec = cudaStreamEndCapture(E->origin, &g);

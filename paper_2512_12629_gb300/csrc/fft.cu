@@ -480,6 +480,7 @@ template <int N, bool BATCH>
 __global__ void __launch_bounds__(XLine<N>::CTA, XLine<N>::MINB) fft_x_r2c(const float *__restrict__ in, float2 *__restrict__ out,
                                                               int64_t nlines, int kxp, const float2 *__restrict__ tw,
                                                               const int *__restrict__ active) {
+    chain();
     extern __shared__ __align__(16) float2 S[];
     if constexpr (BATCH) {
         nlines = (int64_t)*active * N * N / 2;
@@ -496,6 +497,7 @@ template <int N, bool BATCH>
 __global__ void __launch_bounds__(XLine<N>::CTA, XLine<N>::MINB) fft_x_c2r(const float2 *__restrict__ in, float *__restrict__ out,
                                                               int64_t nlines, int kxp, const float2 *__restrict__ tw,
                                                               const int *__restrict__ active) {
+    chain();
     extern __shared__ __align__(16) float2 S[];
     if constexpr (BATCH) {
         nlines = (int64_t)*active * N * N / 2;
@@ -526,6 +528,7 @@ template <int N, bool INV, bool BATCH>
 __global__ void __launch_bounds__(Tile<N, false>::T, Tile<N, false>::MINB) fft_y(float2 *__restrict__ data, int kxp,
                                                                    const float2 *__restrict__ tw,
                                                                    const int *__restrict__ active) {
+    chain();
     extern __shared__ __align__(16) float2 S[];
     if constexpr (BATCH) {
         const int64_t nvb = (int64_t)*active * N * (kxp / Tile<N, false>::L);
@@ -585,6 +588,7 @@ __device__ __forceinline__ void z_block(float2 *S, float2 *__restrict__ data, co
 template <int N, int GMODE, bool BATCH>
 __global__ void __launch_bounds__(Tile<N, true>::T, Tile<N, true>::MINB) fft_z(float2 *__restrict__ data, const float *__restrict__ green,
                                                    int kxp, const float2 *__restrict__ tw, const int *__restrict__ active) {
+    chain();
     extern __shared__ __align__(16) float2 S[];
     if constexpr (BATCH) {
         const int64_t nvb = (int64_t)*active * N * (kxp / Tile<N, true>::L);
@@ -614,13 +618,13 @@ struct Launcher {
         const unsigned bx = pass_grid(ctx, Lv, (nlines + XLine<N>::LINES - 1) / XLine<N>::LINES);
         {
             ProfScope prof(ctx, B ? -1 : P_FFT_X_FWD, Lv.index);   // batched meshes: profiled as one group by the caller
-            fft_x_r2c<N, B><<<bx, XLine<N>::CTA, XLine<N>::SMEM, ctx->stream>>>(Lv.real, Lv.spec, nlines, Lv.kxp, Lv.tw,
+            launch_chained(ctx->chained, fft_x_r2c<N, B>, bx, XLine<N>::CTA, XLine<N>::SMEM, ctx->stream, Lv.real, Lv.spec, nlines, Lv.kxp, Lv.tw,
                                                                             Lv.active);
         }
         const unsigned by = pass_grid(ctx, Lv, (int64_t)Lv.batch * N * (Lv.kxp / Tile<N, false>::L));
         {
             ProfScope prof(ctx, B ? -1 : P_FFT_Y_FWD, Lv.index);
-            fft_y<N, false, B><<<by, Tile<N, false>::T, Tile<N, false>::SMEM, ctx->stream>>>(Lv.spec, Lv.kxp, Lv.tw, Lv.active);
+            launch_chained(ctx->chained, fft_y<N, false, B>, by, Tile<N, false>::T, Tile<N, false>::SMEM, ctx->stream, Lv.spec, Lv.kxp, Lv.tw, Lv.active);
         }
         ctx->launches += 2;
         return cudaGetLastError();
@@ -630,12 +634,12 @@ struct Launcher {
         const unsigned bz = pass_grid(ctx, Lv, (int64_t)Lv.batch * N * (Lv.kxp / Tile<N, true>::L));
         ProfScope prof(ctx, B ? -1 : P_FFT_Z_GREEN, Lv.index);
         if (green && !B && Lv.green2)
-            fft_z<N, 3, false><<<bz, Tile<N, true>::T, Tile<N, true>::SMEM, ctx->stream>>>(Lv.spec, Lv.green2, Lv.kxp, Lv.tw,
+            launch_chained(ctx->chained, fft_z<N, 3, false>, bz, Tile<N, true>::T, Tile<N, true>::SMEM, ctx->stream, Lv.spec, Lv.green2, Lv.kxp, Lv.tw,
                                                                               Lv.active);
         else if (green)
-            fft_z<N, 2, B><<<bz, Tile<N, true>::T, Tile<N, true>::SMEM, ctx->stream>>>(Lv.spec, Lv.green, Lv.kxp, Lv.tw, Lv.active);
+            launch_chained(ctx->chained, fft_z<N, 2, B>, bz, Tile<N, true>::T, Tile<N, true>::SMEM, ctx->stream, Lv.spec, Lv.green, Lv.kxp, Lv.tw, Lv.active);
         else
-            fft_z<N, 0, B><<<bz, Tile<N, true>::T, Tile<N, true>::SMEM, ctx->stream>>>(Lv.spec, nullptr, Lv.kxp, Lv.tw, Lv.active);
+            launch_chained(ctx->chained, fft_z<N, 0, B>, bz, Tile<N, true>::T, Tile<N, true>::SMEM, ctx->stream, Lv.spec, nullptr, Lv.kxp, Lv.tw, Lv.active);
         ctx->launches += 1;
         return cudaGetLastError();
     }
@@ -644,13 +648,13 @@ struct Launcher {
         const unsigned by = pass_grid(ctx, Lv, (int64_t)Lv.batch * N * (Lv.kxp / Tile<N, false>::L));
         {
             ProfScope prof(ctx, B ? -1 : P_FFT_Y_INV, Lv.index);
-            fft_y<N, true, B><<<by, Tile<N, false>::T, Tile<N, false>::SMEM, ctx->stream>>>(Lv.spec, Lv.kxp, Lv.tw, Lv.active);
+            launch_chained(ctx->chained, fft_y<N, true, B>, by, Tile<N, false>::T, Tile<N, false>::SMEM, ctx->stream, Lv.spec, Lv.kxp, Lv.tw, Lv.active);
         }
         const int64_t nlines = (int64_t)Lv.batch * N * N / 2;
         const unsigned bx = pass_grid(ctx, Lv, (nlines + XLine<N>::LINES - 1) / XLine<N>::LINES);
         {
             ProfScope prof(ctx, B ? -1 : P_FFT_X_INV, Lv.index);
-            fft_x_c2r<N, B><<<bx, XLine<N>::CTA, XLine<N>::SMEM, ctx->stream>>>(Lv.spec, Lv.real, nlines, Lv.kxp, Lv.tw,
+            launch_chained(ctx->chained, fft_x_c2r<N, B>, bx, XLine<N>::CTA, XLine<N>::SMEM, ctx->stream, Lv.spec, Lv.real, nlines, Lv.kxp, Lv.tw,
                                                                             Lv.active);
         }
         ctx->launches += 2;

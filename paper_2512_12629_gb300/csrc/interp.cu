@@ -70,6 +70,7 @@ __device__ __forceinline__ void fd7_coeffs(const float w[3], float c[7]) {
 // the same tile as the CIC corner pair's 4-point difference.
 template <int NL, int DA, int DB, int ORD>
 __global__ void __launch_bounds__(INTERP_THREADS) interp_kernel(InterpParams P) {
+    chain();
     extern __shared__ __align__(16) float tiles[];
     __shared__ int row_pre[INTERP_MAX_ROWS + 1], row_start[INTERP_MAX_ROWS];
     const int n_ios = P.n_ios, bi = P.bi;
@@ -308,6 +309,7 @@ __global__ void __launch_bounds__(INTERP_THREADS) interp_kernel(InterpParams P) 
 template <int CELLID_GROUPS>
 __global__ void __launch_bounds__(256) cellid_kernel(const int32_t *__restrict__ count, const int32_t *__restrict__ start,
                                                      int32_t *__restrict__ cellid, int64_t n_cells) {
+    chain();
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - lane) * CELLID_GROUPS;
     int cnt[CELLID_GROUPS], s[CELLID_GROUPS];
@@ -347,8 +349,8 @@ cudaError_t launch_cellid(cube2_ctx *ctx, const cube2_particles *p) {
     const bool many = ctx->n_cells >= (int64_t)ctx->num_sms * 64 * 32 * 4;
     const int64_t per = many ? 1024 : 256;
     const unsigned blocks = (unsigned)((ctx->n_cells + per - 1) / per);
-    if (many) cellid_kernel<4><<<blocks, 256, 0, ctx->stream>>>(p->count, p->start, ctx->cellid, ctx->n_cells);
-    else cellid_kernel<1><<<blocks, 256, 0, ctx->stream>>>(p->count, p->start, ctx->cellid, ctx->n_cells);
+    if (many) launch_chained(ctx->chained, cellid_kernel<4>, blocks, 256, 0, ctx->stream, p->count, p->start, ctx->cellid, ctx->n_cells);
+    else launch_chained(ctx->chained, cellid_kernel<1>, blocks, 256, 0, ctx->stream, p->count, p->start, ctx->cellid, ctx->n_cells);
     ctx->launches++;
     return cudaGetLastError();
 }
@@ -397,7 +399,7 @@ cudaError_t launch_interp(cube2_ctx *ctx, int level, const cube2_particles *p, i
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);           \
             attr = true;                                                                            \
         }                                                                                           \
-        interp_kernel<NL_, A_, B_, O_><<<(unsigned)blocks, INTERP_THREADS, smem, ctx->stream>>>(P); \
+        launch_chained(ctx->chained, interp_kernel<NL_, A_, B_, O_>, (unsigned)blocks, INTERP_THREADS, smem, ctx->stream, P); \
         e = cudaGetLastError();                                                                     \
     }
 #define CUBE2_INTERP_CASE(NL_, A_, B_) CUBE2_INTERP_CASE_O(NL_, A_, B_, 2) CUBE2_INTERP_CASE_O(NL_, A_, B_, 3)

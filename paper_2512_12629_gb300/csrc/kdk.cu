@@ -90,6 +90,7 @@ struct DriftParams {
 };
 
 __global__ void __launch_bounds__(256) kick_drift_kernel(DriftParams P) {
+    chain();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const unsigned mask = __ballot_sync(0xffffffffu, i < P.N);
     if (i >= P.N) return;
@@ -252,6 +253,7 @@ __device__ __forceinline__ void scan_load(const int32_t *in, int64_t base, int64
 }
 
 __global__ void __launch_bounds__(SCAN_THREADS) scan_reduce_kernel(const int32_t *in, int32_t *sums, int64_t n, bool wide) {
+    chain();
     __shared__ int ws[33];
     const int64_t base = (int64_t)blockIdx.x * SCAN_CHUNK + (int64_t)threadIdx.x * SCAN_ITEMS;
     int v[SCAN_ITEMS], s = 0;
@@ -266,6 +268,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_reduce_kernel(const int32_t
 // exclusive scan of in[0, n) into out, adding offsets[blockIdx] (if non-null)
 __global__ void __launch_bounds__(SCAN_THREADS) scan_apply_kernel(const int32_t *in, int32_t *out, int64_t n,
                                                                   const int32_t *offsets, bool wide) {
+    chain();
     __shared__ int ws[33];
     const int64_t base = (int64_t)blockIdx.x * SCAN_CHUNK + (int64_t)threadIdx.x * SCAN_ITEMS;
     int v[SCAN_ITEMS], s = 0;
@@ -294,6 +297,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_apply_kernel(const int32_t 
 // ------------------------------------------------------------- rebin
 __global__ void __launch_bounds__(256) scatter_kernel(Moved from, const int32_t *__restrict__ start, int32_t *perm,
                                                       int64_t n) {
+    chain();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     perm[__ldg(&start[from.cell_off[i].x]) + from.slot[i]] = (int32_t)i;
@@ -403,6 +407,7 @@ __device__ void sort_warp(int32_t *seg, int n, int32_t *s) {
 __global__ void __launch_bounds__(SORT_THREADS) sort_cells_kernel(const int32_t *count, const int32_t *start,
                                                                   int32_t *perm, int32_t *scratch, const int32_t *big,
                                                                   const int *big_n, int64_t n_cells) {
+    chain();
     __shared__ int32_t s[BIG_SORT_SMEM];
     static_assert(SORT_WARPS * WARP_SORT <= BIG_SORT_SMEM, "a buffer per warp");
     const int n_cta = big_n[1];
@@ -452,6 +457,7 @@ struct GatherParams {
 // run at z = 0 (512^3 at z = 1: 1.91 and 2.01); together they took 0.34
 // (2.63), with the packed records 0.23 (1.67).
 __global__ void __launch_bounds__(256) gather_kernel(GatherParams P) {
+    chain();
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= P.N) return;
     const int j = P.slots[s];
@@ -497,6 +503,7 @@ vel_encode_kernel(const float *__restrict__ v0, const float *__restrict__ v1, co
                   const int32_t *__restrict__ cellid, const int32_t *__restrict__ count,
                   const int32_t *__restrict__ start, float *__restrict__ vscale, uint16_t *__restrict__ c0,
                   uint16_t *__restrict__ c1, uint16_t *__restrict__ c2, int64_t n_cells) {
+    chain();
     __shared__ int top[ENCODE_CELLS];
     const int64_t first = (int64_t)blockIdx.x * ENCODE_CELLS;
     const int cells = (int)min((int64_t)ENCODE_CELLS, n_cells - first);
@@ -573,7 +580,7 @@ __global__ void vel_decode_kernel(const uint16_t *__restrict__ c0, const uint16_
 cudaError_t launch_vel_encode(cube2_ctx *ctx, const cube2_particles *p, const float *const v[3]) {
     if (ctx->N == 0) return cudaMemsetAsync(p->vscale, 0, sizeof(float) * ctx->n_cells, ctx->stream);
     ProfScope prof(ctx, P_KICK, 0);
-    vel_encode_kernel<<<(unsigned)((ctx->n_cells + ENCODE_CELLS - 1) / ENCODE_CELLS), ENCODE_THREADS, 0, ctx->stream>>>(
+    launch_chained(ctx->chained, vel_encode_kernel, (unsigned)((ctx->n_cells + ENCODE_CELLS - 1) / ENCODE_CELLS), ENCODE_THREADS, 0, ctx->stream,
         v[0], v[1], v[2], ctx->cellid, p->count, p->start, p->vscale, p->vel16[0], p->vel16[1], p->vel16[2],
         ctx->n_cells);
     ctx->launches++;
@@ -602,7 +609,7 @@ cudaError_t launch_scan(cube2_ctx *ctx, const int32_t *in, int32_t *out, int64_t
     // the callers' arrays may lie anywhere (4-byte words): wide loads only where both allow them
     const bool wide = ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
     if (n <= SCAN_CHUNK) {
-        scan_apply_kernel<<<1, SCAN_THREADS, 0, ctx->stream>>>(in, out, n, nullptr, wide);
+        launch_chained(ctx->chained, scan_apply_kernel, 1, SCAN_THREADS, 0, ctx->stream, in, out, n, nullptr, wide);
         ctx->launches++;
         return cudaGetLastError();
     }
@@ -610,14 +617,14 @@ cudaError_t launch_scan(cube2_ctx *ctx, const int32_t *in, int32_t *out, int64_t
     const int64_t nb = (n + SCAN_CHUNK - 1) / SCAN_CHUNK;
     int32_t *sums = ctx->scan_tmp;
     // reserve this level's sums, recurse on the remainder of the scratch
-    scan_reduce_kernel<<<(unsigned)nb, SCAN_THREADS, 0, ctx->stream>>>(in, sums, n, wide);
+    launch_chained(ctx->chained, scan_reduce_kernel, (unsigned)nb, SCAN_THREADS, 0, ctx->stream, in, sums, n, wide);
     ctx->launches++;
     int32_t *saved = ctx->scan_tmp;
     ctx->scan_tmp = saved + nb;
     cudaError_t e = launch_scan(ctx, sums, sums, nb);
     ctx->scan_tmp = saved;
     if (e != cudaSuccess) return e;
-    scan_apply_kernel<<<(unsigned)nb, SCAN_THREADS, 0, ctx->stream>>>(in, out, n, sums, wide);
+    launch_chained(ctx->chained, scan_apply_kernel, (unsigned)nb, SCAN_THREADS, 0, ctx->stream, in, out, n, sums, wide);
     ctx->launches++;
     return cudaGetLastError();
 }
@@ -658,7 +665,7 @@ cudaError_t launch_kick_drift(cube2_ctx *ctx, const cube2_particles *p, float ki
     if (e != cudaSuccess) return e;
     const int64_t blocks = (ctx->N + 255) / 256;
     if (blocks == 0) return cudaSuccess;
-    kick_drift_kernel<<<(unsigned)blocks, 256, 0, ctx->stream>>>(P);
+    launch_chained(ctx->chained, kick_drift_kernel, (unsigned)blocks, 256, 0, ctx->stream, P);
     ctx->launches++;
     return cudaGetLastError();
 }
@@ -695,7 +702,7 @@ cudaError_t launch_rebin(cube2_ctx *ctx, const cube2_particles *p) {
     if (pb > 0) {
         {
             ProfScope prof(ctx, P_SCATTER, 0);
-            scatter_kernel<<<(unsigned)pb, 256, 0, ctx->stream>>>(moved(ctx), p->start, ctx->perm2, ctx->N);
+            launch_chained(ctx->chained, scatter_kernel, (unsigned)pb, 256, 0, ctx->stream, moved(ctx), p->start, ctx->perm2, ctx->N);
         }
         e = cudaMemsetAsync(ctx->big_n, 0, 2 * sizeof(int), ctx->stream);
         if (e != cudaSuccess) return e;
@@ -706,7 +713,7 @@ cudaError_t launch_rebin(cube2_ctx *ctx, const cube2_particles *p) {
         }
         {
             ProfScope prof(ctx, P_SORT_BIG, 0);
-            sort_cells_kernel<<<(unsigned)(ctx->num_sms * (1536 / SORT_THREADS)), SORT_THREADS, 0, ctx->stream>>>(
+            launch_chained(ctx->chained, sort_cells_kernel, (unsigned)(ctx->num_sms * (1536 / SORT_THREADS)), SORT_THREADS, 0, ctx->stream,
                 p->count, p->start, ctx->perm2, ctx->perm, ctx->big, ctx->big_n, ctx->n_cells);
         }
         GatherParams G{};
@@ -725,7 +732,7 @@ cudaError_t launch_rebin(cube2_ctx *ctx, const cube2_particles *p) {
         G.N = ctx->N;
         {
             ProfScope prof(ctx, P_GATHER, 0);
-            gather_kernel<<<(unsigned)pb, 256, 0, ctx->stream>>>(G);
+            launch_chained(ctx->chained, gather_kernel, (unsigned)pb, 256, 0, ctx->stream, G);
         }
         ctx->launches += 4;
     }

@@ -282,6 +282,7 @@ __global__ void __launch_bounds__(256) pp_dense_sort_kernel(const uint16_t *off0
                                                             const uint16_t *off2, const int32_t *count,
                                                             const int32_t *start, const int2 *list, const int *list_n,
                                                             float4 *pos, int32_t *perm, int32_t *tgt) {
+    chain();
     __shared__ int hist[8][64], run[8][64];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int nwarps_total = gridDim.x * (blockDim.x >> 5);
@@ -1259,6 +1260,7 @@ __device__ __forceinline__ void pp_warp(const PPParams &P, int64_t i, PPWarpShar
 constexpr int PP_WARPS = 2;
 template <bool PM3, bool COUNT>
 __global__ void __launch_bounds__(PP_WARPS * 32, 32 / PP_WARPS) pp_kernel(PPParams P) {
+    chain();
     __shared__ PPWarpShared sh[PP_WARPS];
     pp_warp<PM3, COUNT, true>(P, (int64_t)blockIdx.x * (PP_WARPS * 32) + threadIdx.x, sh[threadIdx.x >> 5]);
 }
@@ -1283,6 +1285,7 @@ struct PPPartSums {
 // The listed warps, a CTA each.
 template <bool PM3, bool COUNT>
 __global__ void __launch_bounds__(PP_PARTS * 32, 32 / PP_PARTS) pp_long_kernel(PPParams P) {
+    chain();
     __shared__ PPWarpShared sh[PP_PARTS];
     __shared__ PPPartSums part;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, n = *P.long_n;
@@ -1333,6 +1336,7 @@ __device__ __forceinline__ void vjp_finish(const VjpIO &V, int pi, const Sum3 &a
 // 0.52, 0.45, 0.43).
 constexpr int VJP_BLOCKS = 28;
 __global__ void __launch_bounds__(32, VJP_BLOCKS) pp_vjp_kernel(PPParams P, VjpIO V) {
+    chain();
     __shared__ PPVjpWarpShared sh;
     const int64_t i = (int64_t)blockIdx.x * 32 + threadIdx.x;
     const int j = P.tgt[i];   // with the length's load under way
@@ -1360,6 +1364,7 @@ __global__ void __launch_bounds__(32, VJP_BLOCKS) pp_vjp_kernel(PPParams P, VjpI
 }
 
 __global__ void __launch_bounds__(PP_PARTS * 32, VJP_BLOCKS / PP_PARTS) pp_vjp_long_kernel(PPParams P, VjpIO V) {
+    chain();
     __shared__ PPVjpWarpShared sh[PP_PARTS];
     __shared__ PPPartSums part;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, n = *P.long_n;
@@ -1515,7 +1520,7 @@ static void launch_pp_inputs(cube2_ctx *ctx, const cube2_particles *p) {
     }
     {
         ProfScope prof(ctx, P_PP_ORDER, 0);
-        pp_dense_sort_kernel<<<(unsigned)(ctx->num_sms * 8), 256, 0, ctx->stream>>>(
+        launch_chained(ctx->chained, pp_dense_sort_kernel, (unsigned)(ctx->num_sms * 8), 256, 0, ctx->stream,
             p->off[0], p->off[1], p->off[2], p->count, p->start, ctx->pp_dense, list_n, ctx->pos4, ctx->pp_perm,
             ctx->pp_tgt);
     }
@@ -1532,10 +1537,10 @@ cudaError_t launch_pp_vjp(cube2_ctx *ctx, const cube2_particles *p, const float 
     V.scale = (float)((double)P.coef / ctx->s_ios);
     launch_pp_inputs(ctx, p);
     ProfScope prof(ctx, P_PP_VJP, 0);
-    pp_vjp_kernel<<<(unsigned)(pp_target_slots(ctx->N, ctx->n_ios) / 32), 32, 0, ctx->stream>>>(P, V);
+    launch_chained(ctx->chained, pp_vjp_kernel, (unsigned)(pp_target_slots(ctx->N, ctx->n_ios) / 32), 32, 0, ctx->stream, P, V);
     ctx->launches += 1;
     if (ctx->N >= PP_LONG_N) {
-        pp_vjp_long_kernel<<<(unsigned)(ctx->num_sms * (VJP_BLOCKS / PP_PARTS)), PP_PARTS * 32, 0, ctx->stream>>>(P, V);
+        launch_chained(ctx->chained, pp_vjp_long_kernel, (unsigned)(ctx->num_sms * (VJP_BLOCKS / PP_PARTS)), PP_PARTS * 32, 0, ctx->stream, P, V);
         ctx->launches += 1;
     }
     return cudaGetLastError();
@@ -1600,13 +1605,14 @@ cudaError_t launch_pp(cube2_ctx *ctx, const cube2_particles *p, int accumulate, 
     {
         ProfScope prof(ctx, P_PP, 0);
         const bool pm3 = P.pm3_slot != nullptr, count = ctx->pp_count;
-        (pm3 ? (count ? pp_kernel<true, true> : pp_kernel<true, false>)
-             : (count ? pp_kernel<false, true> : pp_kernel<false, false>))<<<ctas, PP_WARPS * 32, 0, ctx->stream>>>(P);
+        launch_chained(ctx->chained, pm3 ? (count ? pp_kernel<true, true> : pp_kernel<true, false>)
+                           : (count ? pp_kernel<false, true> : pp_kernel<false, false>),
+                       ctas, PP_WARPS * 32, 0, ctx->stream, P);
         ctx->launches += 1;
         if (ctx->N >= PP_LONG_N) {
-            (pm3 ? (count ? pp_long_kernel<true, true> : pp_long_kernel<true, false>)
-                 : (count ? pp_long_kernel<false, true> : pp_long_kernel<false, false>))<<<
-                (unsigned)(ctx->num_sms * (32 / PP_PARTS)), PP_PARTS * 32, 0, ctx->stream>>>(P);
+            launch_chained(ctx->chained, pm3 ? (count ? pp_long_kernel<true, true> : pp_long_kernel<true, false>)
+                               : (count ? pp_long_kernel<false, true> : pp_long_kernel<false, false>),
+                           (unsigned)(ctx->num_sms * (32 / PP_PARTS)), PP_PARTS * 32, 0, ctx->stream, P);
             ctx->launches += 1;
         }
     }
