@@ -236,7 +236,10 @@ __device__ __forceinline__ void set_status(int *status, int bit) { atomicOr(stat
 // serialisation (cube2_ctx.chained): the next one's CTAs are placed while the last of
 // this one's still run, and wait in chain() for all its writes.  Every kernel launched
 // so calls chain() first, in every thread, before it touches memory; then it completes
-// only after its predecessor has, and any kernel may follow it.
+// only after its predecessor has, and any kernel may follow it.  It is resident while
+// the predecessor writes, and read-only loads are for what nobody writes meanwhile (and
+// may be moved above the wait): particles and meshes are read with ordinary loads, only
+// tables fixed before (twiddles, Green's function) with __ldg or through const __restrict__.
 //
 // It saves the start of each of a small box's dozen short kernels: the force of 32^3
 // particles 72.7 -> 58.2 us, a step of 64^3 425 -> 405, placing 128^3 positions 178 ->

@@ -210,10 +210,15 @@ struct Tile {
 
 // Tiles are read and written once a pass: streaming loads and stores (512^3: z
 // 0.41 -> 0.38 ms); past 512 the plain L2 ones (z at 1024: 3.85 against 4.00 ms).
+// volatile: not moved above chain().
 template <int N>
 __device__ __forceinline__ float2 tile_load(const float2 *p) {
-    if constexpr (N <= 512) return __ldcs(p);
-    return __ldcg(p);
+    float2 v;
+    if constexpr (N <= 512)
+        asm volatile("ld.global.cs.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(__cvta_generic_to_global(p)) : "memory");
+    else
+        asm volatile("ld.global.cg.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(__cvta_generic_to_global(p)) : "memory");
+    return v;
 }
 template <int N>
 __device__ __forceinline__ void tile_store(float2 *p, float2 v) {
@@ -351,7 +356,7 @@ __device__ __forceinline__ void line_stages(float2 *S, int t, int line, const fl
 }
 
 template <int N>
-__device__ __forceinline__ void x_r2c_block(float2 *smem, const float *__restrict__ in, float2 *__restrict__ out,
+__device__ __forceinline__ void x_r2c_block(float2 *smem, const float *in, float2 *__restrict__ out,
                                             int64_t nlines, int kxp, const float2 *__restrict__ tw, int64_t vb) {
     using X = XLine<N>;
     constexpr int R = X::R1, NB = X::NB1, TL = X::TL, LAST = Plan<N, false, true>::S - 1;
@@ -359,7 +364,7 @@ __device__ __forceinline__ void x_r2c_block(float2 *smem, const float *__restric
     const int64_t want = vb * X::LINES + line, l = want < nlines ? want : nlines - 1;   // spare threads repeat the last
     const float *a = in + 2 * l * N, *b = a + N;
     float2 *S = smem + line * X::PITCH;
-    line_stages<N, false, 0, LAST>(S, t, line, tw, [&](int x) { return make_float2(__ldg(&a[x]), __ldg(&b[x])); },
+    line_stages<N, false, 0, LAST>(S, t, line, tw, [&](int x) { return make_float2(a[x], b[x]); },
                                    [](int, float2) {});
     float2 *A = out + 2 * l * kxp, *B = A + kxp;
 #pragma unroll
@@ -388,7 +393,7 @@ __device__ __forceinline__ void x_r2c_block(float2 *smem, const float *__restric
 }
 
 template <int N>
-__device__ __forceinline__ void x_c2r_block(float2 *smem, const float2 *__restrict__ in, float *__restrict__ out,
+__device__ __forceinline__ void x_c2r_block(float2 *smem, const float2 *in, float *__restrict__ out,
                                             int64_t nlines, int kxp, const float2 *__restrict__ tw, int64_t vb) {
     using X = XLine<N>;
     constexpr int R = X::R1, NB = X::NB1, TL = X::TL;
@@ -439,9 +444,9 @@ __device__ __forceinline__ void x_c2r_block(float2 *smem, const float2 *__restri
 }
 
 template <int N, bool BATCH>
-__global__ void __launch_bounds__(XLine<N>::CTA, XLine<N>::MINB) fft_x_r2c(const float *__restrict__ in, float2 *__restrict__ out,
+__global__ void __launch_bounds__(XLine<N>::CTA, XLine<N>::MINB) fft_x_r2c(const float *in, float2 *__restrict__ out,
                                                               int64_t nlines, int kxp, const float2 *__restrict__ tw,
-                                                              const int *__restrict__ active) {
+                                                              const int *active) {
     chain();
     extern __shared__ __align__(16) float2 S[];
     if constexpr (BATCH) {
@@ -456,9 +461,9 @@ __global__ void __launch_bounds__(XLine<N>::CTA, XLine<N>::MINB) fft_x_r2c(const
 }
 
 template <int N, bool BATCH>
-__global__ void __launch_bounds__(XLine<N>::CTA, XLine<N>::MINB) fft_x_c2r(const float2 *__restrict__ in, float *__restrict__ out,
+__global__ void __launch_bounds__(XLine<N>::CTA, XLine<N>::MINB) fft_x_c2r(const float2 *in, float *__restrict__ out,
                                                               int64_t nlines, int kxp, const float2 *__restrict__ tw,
-                                                              const int *__restrict__ active) {
+                                                              const int *active) {
     chain();
     extern __shared__ __align__(16) float2 S[];
     if constexpr (BATCH) {
@@ -489,7 +494,7 @@ __device__ __forceinline__ void y_block(float2 *S, float2 *__restrict__ data, in
 template <int N, bool INV, bool BATCH>
 __global__ void __launch_bounds__(Tile<N, false>::T, Tile<N, false>::MINB) fft_y(float2 *__restrict__ data, int kxp,
                                                                    const float2 *__restrict__ tw,
-                                                                   const int *__restrict__ active) {
+                                                                   const int *active) {
     chain();
     extern __shared__ __align__(16) float2 S[];
     if constexpr (BATCH) {
@@ -549,7 +554,7 @@ __device__ __forceinline__ void z_block(float2 *S, float2 *__restrict__ data, co
 
 template <int N, int GMODE, bool BATCH>
 __global__ void __launch_bounds__(Tile<N, true>::T, Tile<N, true>::MINB) fft_z(float2 *__restrict__ data, const float *__restrict__ green,
-                                                   int kxp, const float2 *__restrict__ tw, const int *__restrict__ active) {
+                                                   int kxp, const float2 *__restrict__ tw, const int *active) {
     chain();
     extern __shared__ __align__(16) float2 S[];
     if constexpr (BATCH) {

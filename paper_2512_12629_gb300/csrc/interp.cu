@@ -307,8 +307,8 @@ __global__ void __launch_bounds__(INTERP_THREADS) interp_kernel(InterpParams P) 
 // a warp for every slot of the chip one group each is better (64^3: 0.0104 against
 // 0.0135 ms).  More than 256 particles are written cell by cell, without the search.
 template <int CELLID_GROUPS>
-__global__ void __launch_bounds__(256) cellid_kernel(const int32_t *__restrict__ count, const int32_t *__restrict__ start,
-                                                     int32_t *__restrict__ cellid, int64_t n_cells) {
+__global__ void __launch_bounds__(256) cellid_kernel(const int32_t *count, const int32_t *start, int32_t *__restrict__ cellid,
+                                                     int64_t n_cells) {
     chain();
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - lane) * CELLID_GROUPS;

@@ -295,12 +295,12 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_apply_kernel(const int32_t 
 }
 
 // ------------------------------------------------------------- rebin
-__global__ void __launch_bounds__(256) scatter_kernel(Moved from, const int32_t *__restrict__ start, int32_t *perm,
+__global__ void __launch_bounds__(256) scatter_kernel(Moved from, const int32_t *start, int32_t *perm,
                                                       int64_t n) {
     chain();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    perm[__ldg(&start[from.cell_off[i].x]) + from.slot[i]] = (int32_t)i;
+    perm[start[from.cell_off[i].x] + from.slot[i]] = (int32_t)i;
 }
 
 // Cells of more than RANK_MAX particles, whose segments are sorted ascending
@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(256) sort_list_kernel(const int32_t *__restric
                                                         int *big_n, bool wide) {
     const int64_t c0 = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
     int4 v = make_int4(0, 0, 0, 0);
-    if (wide && c0 + 3 < n_cells) v = __ldg(reinterpret_cast<const int4 *>(count + c0));
+    if (wide && c0 + 3 < n_cells) v = *reinterpret_cast<const int4 *>(count + c0);
     else
         for (int k = 0; c0 + k < n_cells && k < 4; ++k) (&v.x)[k] = count[c0 + k];
     if (max(max(v.x, v.y), max(v.z, v.w)) <= RANK_MAX) return;
@@ -461,15 +461,15 @@ __global__ void __launch_bounds__(256) gather_kernel(GatherParams P) {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= P.N) return;
     const int j = P.slots[s];
-    const int2 co = __ldg(&P.from.cell_off[j]);
-    const float4 vo = __ldg(&P.from.vel_off[j]);
+    const int2 co = P.from.cell_off[j];
+    const float4 vo = P.from.vel_off[j];
     const int c = co.x;
-    const int cnt = __ldg(&P.count[c]);
+    const int cnt = P.count[c];
     int64_t i = s;
     if (cnt > 1 && cnt <= RANK_MAX) {
-        const int st = __ldg(&P.start[c]);
+        const int st = P.start[c];
         int rank = 0;
-        for (int k = 0; k < cnt; ++k) rank += __ldg(&P.slots[st + k]) < j;
+        for (int k = 0; k < cnt; ++k) rank += P.slots[st + k] < j;
         i = st + rank;
     }
     const unsigned off01 = __float_as_uint(vo.w);
@@ -499,10 +499,9 @@ __device__ __forceinline__ uint16_t velocity_code(float v, float s) {
 }
 
 __global__ void __launch_bounds__(ENCODE_THREADS)
-vel_encode_kernel(const float *__restrict__ v0, const float *__restrict__ v1, const float *__restrict__ v2,
-                  const int32_t *__restrict__ cellid, const int32_t *__restrict__ count,
-                  const int32_t *__restrict__ start, float *__restrict__ vscale, uint16_t *__restrict__ c0,
-                  uint16_t *__restrict__ c1, uint16_t *__restrict__ c2, int64_t n_cells) {
+vel_encode_kernel(const float *v0, const float *v1, const float *v2, const int32_t *cellid, const int32_t *count,
+                  const int32_t *start, float *__restrict__ vscale, uint16_t *__restrict__ c0, uint16_t *__restrict__ c1,
+                  uint16_t *__restrict__ c2, int64_t n_cells) {
     chain();
     __shared__ int top[ENCODE_CELLS];
     const int64_t first = (int64_t)blockIdx.x * ENCODE_CELLS;
@@ -555,10 +554,10 @@ vel_encode_kernel(const float *__restrict__ v0, const float *__restrict__ v1, co
         }
     }
     for (int64_t i = rest + threadIdx.x; i < e; i += ENCODE_THREADS) {
-        const float s = __int_as_float(top[cellid[i] - (int)first]);
-        c0[i] = velocity_code(v0[i], s);
-        c1[i] = velocity_code(v1[i], s);
-        c2[i] = velocity_code(v2[i], s);
+        const float s = __int_as_float(top[cellid[i] - (int)first]), vx = v0[i], vy = v1[i], vz = v2[i];
+        c0[i] = velocity_code(vx, s);
+        c1[i] = velocity_code(vy, s);
+        c2[i] = velocity_code(vz, s);
     }
 }
 

@@ -132,31 +132,31 @@ struct RowRanges {
         const int BIG = 0x7fffffff;
         if (cx > 0 && cx < n - 1) {
             nseg = 1;
-            beg[0] = __ldg(&P.start[r + cx - 1]);
-            b1[0] = __ldg(&P.start[r + cx]);
-            b2[0] = __ldg(&P.start[r + cx + 1]);
-            end[0] = b2[0] + __ldg(&P.count[r + cx + 1]);
+            beg[0] = P.start[r + cx - 1];
+            b1[0] = P.start[r + cx];
+            b2[0] = P.start[r + cx + 1];
+            end[0] = b2[0] + P.count[r + cx + 1];
             base[0] = -1;
         } else if (cx == 0) {
             nseg = 2;
-            beg[0] = __ldg(&P.start[r]);
-            b1[0] = __ldg(&P.start[r + 1]);
+            beg[0] = P.start[r];
+            b1[0] = P.start[r + 1];
             b2[0] = BIG;
-            end[0] = b1[0] + __ldg(&P.count[r + 1]);
+            end[0] = b1[0] + P.count[r + 1];
             base[0] = 0;
-            beg[1] = __ldg(&P.start[r + n - 1]);
-            end[1] = beg[1] + __ldg(&P.count[r + n - 1]);
+            beg[1] = P.start[r + n - 1];
+            end[1] = beg[1] + P.count[r + n - 1];
             b1[1] = b2[1] = BIG;
             base[1] = -1;
         } else {
             nseg = 2;
-            beg[0] = __ldg(&P.start[r + n - 2]);
-            b1[0] = __ldg(&P.start[r + n - 1]);
+            beg[0] = P.start[r + n - 2];
+            b1[0] = P.start[r + n - 1];
             b2[0] = BIG;
-            end[0] = b1[0] + __ldg(&P.count[r + n - 1]);
+            end[0] = b1[0] + P.count[r + n - 1];
             base[0] = -1;
-            beg[1] = __ldg(&P.start[r]);
-            end[1] = beg[1] + __ldg(&P.count[r]);
+            beg[1] = P.start[r];
+            end[1] = beg[1] + P.count[r];
             b1[1] = b2[1] = BIG;
             base[1] = 1;
         }
@@ -444,12 +444,12 @@ __device__ __forceinline__ int build_segments(const PPParams &P, int4 *seg, int 
         if (lane < rows) {
             if (g == 0) {
                 const int lo = max(B.xa - 1, 0), hi = min(B.xb + 1, n - 1);
-                beg = __ldg(&P.start[rb + lo]);
-                len = __ldg(&P.start[rb + hi]) + __ldg(&P.count[rb + hi]) - beg;
+                beg = P.start[rb + lo];
+                len = P.start[rb + hi] + P.count[rb + hi] - beg;
             } else {
                 const int c = g == 1 ? rb + n - 1 : rb;
-                beg = __ldg(&P.start[c]);
-                len = __ldg(&P.count[c]);
+                beg = P.start[c];
+                len = P.count[c];
                 adj += g == 1 ? n : -n;
             }
         }
@@ -639,7 +639,7 @@ struct PPStream {
         g = W.seg[before + __popc(mask & (0xffffffffu >> (31 - lane))) - 1];
         before += __popc(mask);
         slot = b0 + lane + g.x;
-        if (b0 + lane < total) raw = __ldg(&P.pos[slot]);
+        if (b0 + lane < total) raw = P.pos[slot];
     }
     // the source at b0 + lane in the warp's frame (of no meaning past the end)
     __device__ __forceinline__ float4 next(const PPParams &P, const PPWarpShared &W, int b0) {
@@ -926,7 +926,7 @@ __device__ void lane_path(const PPParams &P, int c, float4 me, const PPLane &L, 
             for (int sgi = 0; sgi < rr.nseg; ++sgi) {
 #pragma unroll 1
                 for (int j = rr.beg[sgi]; j < rr.end[sgi]; ++j) {
-                    const float4 q = __ldg(&P.pos[j]);
+                    const float4 q = P.pos[j];
                     const float fdx = (float)(rr.base[sgi] + (j >= rr.b1[sgi]) + (j >= rr.b2[sgi]));
                     const float rx = (fdx + q.x) - me.x;
                     const float ry = (fdy + q.y) - me.y;
@@ -1055,15 +1055,15 @@ __device__ void lane_vjp(const PPParams &P, const VjpIO &V, bool has, int c, flo
             float px = 0.f, py = 0.f, pz = 0.f;
             for (int sgi = 0; sgi < rr.nseg; ++sgi) {
                 for (int j = rr.beg[sgi]; j < rr.end[sgi]; ++j) {
-                    const float4 q = __ldg(&P.pos[j]);
+                    const float4 q = P.pos[j];
                     const float fdx = (float)(rr.base[sgi] + (j >= rr.b1[sgi]) + (j >= rr.b2[sgi]));
                     const float rx = (fdx + q.x) - me.x;
                     const float ry = (fdy + q.y) - me.y;
                     const float rz = (fdz + q.z) - me.z;
                     const float r2 = rx * rx + ry * ry + rz * rz;
                     if (r2 < P.bcut2 && r2 > 0.0f) {
-                        const int pj = __ldg(&P.perm[j]);
-                        const float4 vj = make_float4(__ldg(&V.v0[pj]), __ldg(&V.v1[pj]), __ldg(&V.v2[pj]), 0.f);
+                        const int pj = P.perm[j];
+                        const float4 vj = make_float4(V.v0[pj], V.v1[pj], V.v2[pj], 0.f);
                         jacobian_term(rx, ry, rz, r2, vj, vix, viy, viz, P, px, py, pz);
                     }
                 }
@@ -1139,7 +1139,7 @@ __device__ __forceinline__ PPTarget warp_target(const PPParams &P, int j, PPBloc
     t.has = j >= 0;
     const int j0 = __shfl_sync(0xffffffffu, j, 0);   // a warp's first target is never padding
     t.slot = t.has ? j : j0;
-    t.me = __ldg(&P.pos[t.slot]);
+    t.me = P.pos[t.slot];
     const int n = P.n_ios, c = __float_as_int(t.me.w);
     const int row = (int)(__umulhi((unsigned)c, P.div_mul) >> P.div_shift);
     t.cx = c - row * n;
@@ -1171,7 +1171,7 @@ __device__ __forceinline__ PPLane pp_lane(const PPParams &P, const PPTarget &t, 
     if (PM3) {
         const int T = P.pm3_T;
         const int s = (t.cz / T * P.pm3_ns + t.cy / T) * P.pm3_ns + t.cx / T;
-        if (__ldg(&P.pm3_slot[s]) >= 0) {
+        if (P.pm3_slot[s] >= 0) {
             L.bcut2 = P.bcut2_3;
             ibc = P.inv_bcut_3;
         }
@@ -1319,8 +1319,8 @@ __device__ __forceinline__ void vjp_stream(const PPParams &P, const VjpIO &V, PP
     unsigned pairs = 0, cands = 0;   // not asked for
     stream_sparse(P, W, T, L, pairs, cands,
                   [&](int at, int slot) {
-                      const int k = __ldg(&P.perm[slot]);
-                      W.vel.put(at, make_float4(__ldg(&V.v0[k]), __ldg(&V.v1[k]), __ldg(&V.v2[k]), 0.f));
+                      const int k = P.perm[slot];
+                      W.vel.put(at, make_float4(V.v0[k], V.v1[k], V.v2[k], 0.f));
                   },
                   [&](int held) { vjp_queue(P, W, held, L, vix, viy, viz, a); });
 }
@@ -1423,7 +1423,7 @@ __global__ void __launch_bounds__(256) pp_item_cost_kernel(const PPParams *__res
     unsigned s = 0;
     for (int64_t i = i0; i < i1; ++i) {
         const int j = P.tgt[i];
-        if (j >= 0) s += (unsigned)__ldg(&P.count[__float_as_int(__ldg(&P.pos[j]).w)]);
+        if (j >= 0) s += (unsigned)P.count[__float_as_int(P.pos[j].w)];
     }
     cost[k] = s;
 }
