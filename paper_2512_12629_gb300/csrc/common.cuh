@@ -5,9 +5,11 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <initializer_list>
 #include <string>
 
 #include "../../include/cube2.h"
+#include "per_device.cuh"
 
 namespace cube2 {
 
@@ -267,6 +269,24 @@ inline void launch_chained(bool on, void (*kernel)(P...), unsigned grid, unsigne
     cfg.attrs = &attr;
     cfg.numAttrs = on ? 1 : 0;
     cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);   // the caller reads cudaGetLastError()
+}
+
+// f() once on the current device: the opt-ins that a launch needs.
+template <class F>
+inline cudaError_t once_per_device(PerDevice &made, F f) {
+    int device = 0;
+    const cudaError_t e = cudaGetDevice(&device);
+    return e == cudaSuccess ? made.once(device, f) : e;
+}
+
+template <class K>
+inline cudaError_t allow_shared(K *kernel, size_t bytes) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+inline cudaError_t first_error(std::initializer_list<cudaError_t> all) {
+    for (const cudaError_t e : all)
+        if (e != cudaSuccess) return e;
+    return cudaSuccess;
 }
 
 __device__ __forceinline__ int wrap(int j, int n) { return j < 0 ? j + n : (j >= n ? j - n : j); }

@@ -445,12 +445,11 @@ constexpr int64_t BOTH_BRICKS = 8192;   // most fine bricks with which the coars
 template <int UP, int BI>
 cudaError_t launch_fine(cube2_ctx *ctx, DepParams fine, const DepParams *coarse) {
     constexpr size_t SMEM = DepTile<(BI << UP)>::SMEM, BOTH = SMEM > COARSE_SMEM ? SMEM : COARSE_SMEM;
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(deposit_kernel<UP, BI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
-        cudaFuncSetAttribute(deposit_both_kernel<UP, BI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BOTH);
-        attr = true;
-    }
+    static PerDevice made;
+    const cudaError_t opt = once_per_device(made, [] {
+        return first_error({allow_shared(deposit_kernel<UP, BI>, SMEM), allow_shared(deposit_both_kernel<UP, BI>, BOTH)});
+    });
+    if (opt != cudaSuccess) return opt;
     fine.nbx = (fine.n_ios + BI - 1) / BI;
     if (coarse && bricks(fine) <= BOTH_BRICKS) {
         launch_chained(ctx->chained, deposit_both_kernel<UP, BI>, (unsigned)(bricks(*coarse) + bricks(fine)), DEP_THREADS, BOTH, ctx->stream,

@@ -628,44 +628,45 @@ struct Launcher {
         return cudaGetLastError();
     }
     static cudaError_t forward(cube2_ctx *ctx, Level &Lv) {
-        setup();
+        const cudaError_t e = setup();
+        if (e != cudaSuccess) return e;
         if constexpr (N <= BATCH_MAX_N)
             if (Lv.active) return forward_v<true>(ctx, Lv);
         if (Lv.active) return cudaErrorInvalidValue;
         return forward_v<false>(ctx, Lv);
     }
     static cudaError_t z_pass(cube2_ctx *ctx, Level &Lv, bool green) {
-        setup();
+        const cudaError_t e = setup();
+        if (e != cudaSuccess) return e;
         if constexpr (N <= BATCH_MAX_N)
             if (Lv.active) return z_pass_v<true>(ctx, Lv, green);
         if (Lv.active) return cudaErrorInvalidValue;
         return z_pass_v<false>(ctx, Lv, green);
     }
     static cudaError_t inverse(cube2_ctx *ctx, Level &Lv) {
-        setup();
+        const cudaError_t e = setup();
+        if (e != cudaSuccess) return e;
         if constexpr (N <= BATCH_MAX_N)
             if (Lv.active) return inverse_v<true>(ctx, Lv);
         if (Lv.active) return cudaErrorInvalidValue;
         return inverse_v<false>(ctx, Lv);
     }
     template <bool B>
-    static void setup_v() {
-        const int smem = (int)std::max(Tile<N, false>::SMEM, Tile<N, true>::SMEM), xmem = (int)XLine<N>::SMEM;
-        cudaFuncSetAttribute(fft_x_r2c<N, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, xmem);
-        cudaFuncSetAttribute(fft_x_c2r<N, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, xmem);
-        cudaFuncSetAttribute(fft_y<N, false, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaFuncSetAttribute(fft_y<N, true, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaFuncSetAttribute(fft_z<N, 0, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaFuncSetAttribute(fft_z<N, 2, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    static cudaError_t setup_v() {
+        constexpr size_t y = Tile<N, false>::SMEM, z = Tile<N, true>::SMEM, x = XLine<N>::SMEM;
+        return first_error({allow_shared(fft_x_r2c<N, B>, x), allow_shared(fft_x_c2r<N, B>, x),
+                            allow_shared(fft_y<N, false, B>, y), allow_shared(fft_y<N, true, B>, y),
+                            allow_shared(fft_z<N, 0, B>, z), allow_shared(fft_z<N, 2, B>, z)});
     }
-    static void setup() {
-        static bool done = false;
-        if (done) return;
-        setup_v<false>();
-        cudaFuncSetAttribute(fft_z<N, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Tile<N, true>::SMEM);
-        cudaFuncSetAttribute(fft_z<N, 3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Tile<N, true>::SMEM);
-        if constexpr (N <= BATCH_MAX_N) setup_v<true>();
-        done = true;
+    static cudaError_t setup() {
+        static PerDevice made;
+        return once_per_device(made, [] {
+            cudaError_t e = first_error({setup_v<false>(), allow_shared(fft_z<N, 1, false>, Tile<N, true>::SMEM),
+                                         allow_shared(fft_z<N, 3, false>, Tile<N, true>::SMEM)});
+            if constexpr (N <= BATCH_MAX_N)
+                if (e == cudaSuccess) e = setup_v<true>();
+            return e;
+        });
     }
 };
 
@@ -769,7 +770,8 @@ void *g_noalloc_ptr[NOALLOC_MAX_DEVICES] = {};
 template <int N>
 cudaError_t noalloc_passes(const float *rho, float2 *spec, const float *gpad, float *phi, const float2 *tw, int kxp,
                            cudaStream_t st) {
-    Launcher<N>::setup();
+    const cudaError_t opt = Launcher<N>::setup();
+    if (opt != cudaSuccess) return opt;
     constexpr int L = Tile<N, true>::L;
     static_assert(L == Tile<N, false>::L, "one grid for y and z");
     static_assert(twiddle_entries(N) <= NOALLOC_TWIDDLES && (size_t)N * N * ((N / 2 + 16) / 16 * 16) <= NOALLOC_HALF,

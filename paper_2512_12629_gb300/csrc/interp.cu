@@ -393,12 +393,9 @@ cudaError_t launch_interp(cube2_ctx *ctx, int level, const cube2_particles *p, i
     // tile edges are 8, 10, 14 or 22 (brick 8 or 4, shifts -2..1); the coarse level has the smaller edge
 #define CUBE2_INTERP_CASE_O(NL_, A_, B_, O_)                                                        \
     if (P.nl == NL_ && d0 == A_ && d1 == B_ && ord == O_) {                                         \
-        static bool attr = false;                                                                   \
-        if (!attr) {                                                                                \
-            cudaFuncSetAttribute(interp_kernel<NL_, A_, B_, O_>,                                     \
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);           \
-            attr = true;                                                                            \
-        }                                                                                           \
+        static PerDevice made;                                                                      \
+        e = once_per_device(made, [] { return allow_shared(interp_kernel<NL_, A_, B_, O_>, 200 * 1024); }); \
+        if (e != cudaSuccess) return e;                                                             \
         launch_chained(ctx->chained, interp_kernel<NL_, A_, B_, O_>, (unsigned)blocks, INTERP_THREADS, smem, ctx->stream, P); \
         e = cudaGetLastError();                                                                     \
     }

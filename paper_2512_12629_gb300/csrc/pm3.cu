@@ -329,11 +329,9 @@ cudaError_t launch_pm3(cube2_ctx *ctx, const cube2_particles *p) {
         ProfScope prof(ctx, P_PM3_DEPOSIT, 0);
         const int slab = pm3_slab_planes(g.m);
         const size_t smem = (size_t)2 * slab * g.m * g.m * sizeof(unsigned int);
-        static bool attr = false;
-        if (!attr) {
-            cudaFuncSetAttribute(pm3_slab_deposit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
-            attr = true;
-        }
+        static PerDevice made;
+        e = once_per_device(made, [] { return allow_shared(pm3_slab_deposit_kernel, 100 * 1024); });
+        if (e != cudaSuccess) return e;
         pm3_slab_deposit_kernel<<<dim3((unsigned)((g.m + slab - 1) / slab), (unsigned)M.max_tiles), 256, smem,
                                   ctx->stream>>>(p->off[0], p->off[1], p->off[2], p->count, p->start, M.list, M.count,
                                                  g, slab, M.lev.real, M.dens_scale, ctx->dev_status);
