@@ -36,7 +36,10 @@
 // reproducible.
 #include "common.cuh"
 
+#include <math.h>
 #include <string.h>
+
+#include <algorithm>
 
 namespace cube2 {
 namespace {
@@ -1570,11 +1573,15 @@ static PPParams pp_params(cube2_ctx *ctx, const cube2_particles *p, int accumula
     }
     P.accumulate = accumulate;
     const double s = ctx->s_ios;
-    P.inv_bpp = (float)(s / ctx->cfg.b_pp);
-    P.inv_bcut = (float)(s / ctx->b_range);
-    P.bcut2 = (float)((ctx->b_range / s) * (ctx->b_range / s));
-    P.bpp2 = (float)((ctx->cfg.b_pp / s) * (ctx->cfg.b_pp / s));
-    P.ratio2 = (float)((s / ctx->cfg.b_pp) * (s / ctx->cfg.b_pp));
+    // Separations are 0 or at least 2^-16 cells: shorter lengths all act like these, whose
+    // powers stay within FP32 (the square of a softening that underflowed to 0 would no
+    // longer tell the target itself from a far pair).
+    const double b_cut = std::max(ctx->b_range, ldexp(s, -17)), b_pp = std::max(ctx->cfg.b_pp, ldexp(s, -18));
+    P.inv_bpp = (float)(s / b_pp);
+    P.inv_bcut = (float)(s / b_cut);
+    P.bcut2 = (float)((b_cut / s) * (b_cut / s));
+    P.bpp2 = (float)((b_pp / s) * (b_pp / s));
+    P.ratio2 = (float)((s / b_pp) * (s / b_pp));
     const double vp = ctx->cfg.box * ctx->cfg.box * ctx->cfg.box / (double)ctx->N;
     P.coef = (float)(vp / (4.0 * 3.14159265358979323846) / (s * s));
     P.kick = kick;
@@ -1586,8 +1593,9 @@ static PPParams pp_params(cube2_ctx *ctx, const cube2_particles *p, int accumula
         P.pm3_slot = ctx->pm3.slot;
         P.pm3_T = ctx->pm3.T;
         P.pm3_ns = ctx->pm3.ns;
-        P.bcut2_3 = (float)((ctx->pm3.b3 / s) * (ctx->pm3.b3 / s));
-        P.inv_bcut_3 = (float)(s / ctx->pm3.b3);
+        const double b3 = std::max(ctx->pm3.b3, ldexp(s, -17));
+        P.bcut2_3 = (float)((b3 / s) * (b3 / s));
+        P.inv_bcut_3 = (float)(s / b3);
     }
     return P;
 }
