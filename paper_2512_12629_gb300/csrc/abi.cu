@@ -133,6 +133,7 @@ void free_ctx(cube2_ctx *c) {
     cudaFree(c->pp_tgt);
     cudaFree(c->pp_dense);
     cudaFree(c->pp_long);
+    cudaFree(c->pp_work);
     cudaFree(c->vjp_mu);
     cudaFree(c->vjp_t);
     cudaFree(c->vjp_u);
@@ -331,7 +332,8 @@ int cube2_init_mesh(cube2_ctx **out, const cube2_config *cfg, void *stream) {
     alloc((void **)&c->perm, N * 4);
     alloc((void **)&c->perm2, N * 4);
     alloc((void **)&c->big, (size_t)c->n_cells * 4);
-    alloc((void **)&c->big_n, 3 * sizeof(int));
+    alloc((void **)&c->big_n, 2 * sizeof(int));
+    alloc(&c->pp_work, pp_work_bytes());
     alloc((void **)&c->pos4, N * 16);
     alloc((void **)&c->pp_perm, N * 4);
     alloc((void **)&c->pp_tgt, (size_t)pp_target_slots(c->N, c->n_ios) * 4);

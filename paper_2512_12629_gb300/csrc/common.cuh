@@ -107,15 +107,15 @@ struct cube2_ctx {
     void *moved8 = nullptr;
     int32_t *tslot = nullptr;
     int32_t *perm = nullptr;
-    int32_t *perm2 = nullptr;      // [N] merge scratch of the segmented sort
-    int32_t *big = nullptr;        // [n_cells] cells too large for the per-thread sort
-    int *big_n = nullptr;          // [3] their numbers (a warp each, a CTA each); in PP: dense cells, target
-                                   // places, warps with long streams
+    int32_t *perm2 = nullptr;      // [N] old indices by provisional slot (their sort has perm for scratch)
+    int32_t *big = nullptr;        // [n_cells] cells whose slots are sorted: a warp each from the front, a CTA each from the back
+    int *big_n = nullptr;          // [2] their numbers
     float4 *pos4 = nullptr;        // [N] in-cell offsets as floats (+ cell id bits), PP order
     int32_t *pp_perm = nullptr;    // [N] particle index of each PP slot (sub-cell order in dense cells)
     int32_t *pp_tgt = nullptr;     // [pp_target_slots] PP slots in target (pencil) order, -1 in the pencils' padding
     int2 *pp_dense = nullptr;      // [N / 64] dense cells and the places of their first targets
     int32_t *pp_long = nullptr;    // [target places / 32] warps whose source stream several warps share
+    void *pp_work = nullptr;       // PP's counters (PPWork)
     unsigned long long *pp_stats = nullptr;  // [4] in-range ordered pairs, candidates; the same of per-lane walks
     int num_sms = 152;
     int32_t *scan_tmp = nullptr;   // block sums of the multi-level scan
@@ -197,6 +197,7 @@ cudaError_t launch_fft_batched_solve(cube2_ctx *ctx, Level &L);     // forward, 
 cudaError_t launch_pm3(cube2_ctx *ctx, const cube2_particles *p);    // map, local deposit + solve, gather (acc +=)
 cudaError_t launch_pm3_map(cube2_ctx *ctx, const cube2_particles *p);  // refinement map only
 cudaError_t launch_vel_encode(cube2_ctx *ctx, const cube2_particles *p, const float *const v[3]);
+size_t pp_work_bytes();
 int64_t pp_dense_cells(int64_t N);
 int64_t pp_target_slots(int64_t N, int n_ios);
 int64_t pp_target_items(int64_t N, int n_ios);

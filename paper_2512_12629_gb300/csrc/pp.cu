@@ -44,16 +44,23 @@
 namespace cube2 {
 namespace {
 
+// Counters of one PP evaluation (zeroed before it).
+struct PPWork {
+    int dense;          // cells reordered by sub-cell
+    unsigned places;    // target places in use
+    int crowd;          // targets with long streams, by the cells around them
+    int n;              // warps with long streams, listed
+};
+
 struct PPParams {
     const float4 *pos;          // [N] (off_x, off_y, off_z)/2^16, .w = cell id bits, in PP slot order
     const int32_t *perm;        // [N] particle index of each slot
     const int32_t *tgt;         // slot of each target, pencil by pencil, padded to whole warps with -1
-    const unsigned *tgt_n;      // length of tgt (device)
+    PPWork *work;
     const int32_t *count, *start;
     float *acc0, *acc1, *acc2;
     float *vel0, *vel1, *vel2;
-    unsigned long long *stats;  // [2]: in-range ordered pairs, candidates
-    int64_t N;
+    unsigned long long *stats;  // [4]: in-range ordered pairs, candidates; the same of per-lane walks
     int n_ios, accumulate;
     unsigned div_mul;           // c / n_ios = umulhi(c, div_mul) >> div_shift for 0 <= c < 2^31
     int div_shift;
@@ -69,7 +76,7 @@ struct PPParams {
     float bcut2_3, inv_bcut_3;
     int long_min;                     // longer streams go to the list and are shared by PP_PARTS warps
     int32_t *long_list;               // target places / 32 of those warps
-    int *long_n;
+    int long_crowd;                   // most targets with long streams with which that is done
 };
 
 // R(r, b) of Eq. (refforce) times b^2, as a function of u = r / b < 1.
@@ -180,18 +187,47 @@ constexpr int PREP_WARPS = 4, PREP_CTA = PREP_WARPS * 32;   // input kernels
 // starts on a whole warp (its tail is padded with -1): a warp never spans two.
 constexpr int PEN_Y = 2, PEN_Z = 2, PEN = PEN_Y * PEN_Z;
 
+constexpr int PP_ROWS = (PEN_Y + 2) * (PEN_Z + 2);   // rows of cells that a warp's targets see
+
+// A warp in a halo has a stream of thousands of sources and works on it long after
+// the rest of a small box is done.  Streams longer than PPParams.long_min are put on a
+// list and shared by the PP_PARTS warps of a CTA in a second kernel; the partial sums
+// are added in their order, so the result does not depend on which path (the
+// ensemble's persistent kernel works on the parts one after another) computed them.
+//
+// Splitting repeats the staging in every part and starts after the first kernel: it
+// pays while a few long warps outlive the others, that is in small boxes and where the
+// long warps would not fill the chip by themselves.  PP with / without, 64^3 particles
+// 20 % or 40 % in haloes (600 and 1300 long warps): 0.23 / 0.30 and 0.34 / 0.44 ms;
+// 500000 in 32^3 cells, 262144 in 24^3 or a tenth of 64^3 cells, all evenly (8000 to
+// 16000): 0.63 / 0.39, 0.40 / 0.27 and 0.27 / 0.19 ms.  96^3 particles, 20 % or 55 %
+// in haloes: 0.49 / 0.50 and 0.87 / 0.82 ms, larger boxes less.  The limit of 512
+// against 1024 and 2048: 0.22 / 0.25 / 0.33 ms (64^3, 20 % in haloes).  The adjoint's
+// pairs cost several times more: two products of 128^3 particles, 10 % or 40 % in
+// haloes, 2.07 / 2.20 and 4.06 / 3.82 ms.  4 or 16 parts are no better than 8.
+// What decides is counted from the cells before the first warp runs (pp_pencil_kernel),
+// so that every launch of a state decides the same.
+constexpr int PP_PARTS = 8;
+constexpr int PP_UNSPLIT = 0x7fffffff;
+constexpr int64_t PP_LONG_N = 65536;    // smaller boxes: the second launch costs more than it gives
+
+inline int pp_long_min(int64_t N) { return N < PP_LONG_N || N >= (1 << 19) ? PP_UNSPLIT : 512; }
+inline int vjp_long_min(int64_t N) { return N < PP_LONG_N || N >= (1 << 22) ? PP_UNSPLIT : N < (1 << 20) ? 512 : (int)(N / 2048); }
+
 __host__ __device__ __forceinline__ int pencils_y(int n) { return (n + PEN_Y - 1) / PEN_Y; }
 __host__ __device__ __forceinline__ int pencils_z(int n) { return (n + PEN_Z - 1) / PEN_Z; }
 
 // One CTA per pencil: the target places of its cells (cells of sort_min
 // particles or more are listed with their first place for pp_dense_sort_kernel,
 // which writes them with a warp each) and the padding of the pencil's tail.
-// Pencils take their places in tgt by an atomic on tgt_n: their order varies,
-// the warps of a pencil and so the results do not.
+// Pencils take their places in tgt by an atomic on their number: their order varies,
+// the warps of a pencil and so the results do not.  LONG: counts the targets whose
+// streams are longer than long_min, about.
+template <bool LONG>
 __global__ void __launch_bounds__(PREP_CTA) pp_pencil_kernel(const int32_t *__restrict__ count,
                                                              const int32_t *__restrict__ start, int n, int sort_min,
-                                                             int32_t *__restrict__ tgt, unsigned *tgt_n,
-                                                             int2 *__restrict__ list, int *list_n) {
+                                                             int long_min, int32_t *__restrict__ tgt,
+                                                             int2 *__restrict__ list, PPWork *work) {
     __shared__ unsigned s_base;   // places are unsigned: N plus the padding may pass 2^31
     __shared__ int s_warp[PREP_WARPS];
     const int npy = pencils_y(n);
@@ -208,7 +244,7 @@ __global__ void __launch_bounds__(PREP_CTA) pp_pencil_kernel(const int32_t *__re
         total = __reduce_add_sync(0xffffffffu, total);
         const int padded = (total + 31) & ~31;
         unsigned base = 0;
-        if (lane == 0 && padded) base = atomicAdd(tgt_n, (unsigned)padded);
+        if (lane == 0 && padded) base = atomicAdd(&work->places, (unsigned)padded);
         base = __shfl_sync(0xffffffffu, base, 0);
         if (lane < padded - total) tgt[base + total + lane] = -1;
         if (lane == 0) s_base = base;
@@ -239,12 +275,25 @@ __global__ void __launch_bounds__(PREP_CTA) pp_pencil_kernel(const int32_t *__re
             run += s_warp[k];
         }
         __syncthreads();
+        if (LONG) {   // a stream: the rows around the pencil's, over the slabs of 32 targets and one on each side
+            int near = 0;
+            if (sum > 0) {
+#pragma unroll 4
+                for (int k = 0; k < PP_ROWS; ++k) {
+                    const int64_t r = ((int64_t)wrap(z0 - 1 + k / (PEN_Y + 2), n) * n + wrap(y0 - 1 + k % (PEN_Y + 2), n)) * n;
+                    near += count[r + wrap(x - 1, n)] + count[r + x] + count[r + wrap(x + 1, n)];
+                }
+            }
+            if (sum > 0) near += (int)((int64_t)near * 32 / (3 * sum));
+            const int crowd = __reduce_add_sync(0xffffffffu, near > long_min ? sum : 0);
+            if (lane == 0 && crowd) atomicAdd(&work->crowd, crowd);
+        }
 #pragma unroll
         for (int k = 0; k < PEN; ++k) {
             const int64_t r = row_of(k);
             if (x < n && r >= 0) {
                 if (cnt[k] >= sort_min) {
-                    list[atomicAdd(list_n, 1)] = make_int2((int)(r + x), (int)at);
+                    list[atomicAdd(&work->dense, 1)] = make_int2((int)(r + x), (int)at);
                 } else if (cnt[k]) {
                     const int st = start[r + x];
                     for (int j = 0; j < cnt[k]; ++j) tgt[at + j] = st + j;
@@ -354,7 +403,6 @@ struct Sum3 {
 // coordinates in the warp's frame (cell (xa, ya - 1, za - 1) at 0) are (cell id
 // - seg[s].y) + off_x, row_y + off_y, row_z + off_z with the row's offsets as
 // floats in seg[s].z and .w: exact in FP32 for blocks of up to 128 cells.
-constexpr int PP_ROWS = (PEN_Y + 2) * (PEN_Z + 2);
 constexpr int PP_SEGS = 3 * PP_ROWS;
 
 // A warp is on the shared stream when it spans at most PP_WIDEST + 1 cells along x;
@@ -382,27 +430,6 @@ constexpr int OUTER_N = 64;             // sources evaluated at a time, no pair 
 constexpr int MIXED_N = 32;             // sources evaluated at a time, any distance
 constexpr int SPARSE_N = 128;           // sources tested before the pairs found are evaluated
 constexpr int QUEUE_N = 32;             // pairs a lane can hold
-
-// A warp in a halo has a stream of thousands of sources and works on it long after
-// the rest of a small box is done.  Streams longer than PPParams.long_min are put on a
-// list and shared by the PP_PARTS warps of a CTA in a second kernel; the partial sums
-// are added in their order, so the result does not depend on which path (the
-// ensemble's persistent kernel works on the parts one after another) computed them.
-//
-// Where the line lies: splitting repeats the staging in every part and starts after
-// the first kernel, so it pays while a long warp outlives the others, that is in small
-// boxes.  PP of 64^3 particles at z = 1, 20 % in haloes, with 512 / 1024 / 2048 / no
-// limit: 0.164 / 0.195 / 0.285 / 0.283 ms; 128^3 at z = 0.5, 40 % in haloes, with 512 /
-// 1024 / 4096 / 8192 / none: 1.245 / 1.188 / 1.167 / 1.120 / 1.122 ms; 256^3 at z = 0
-// with 2048 / 8192 / none 9.46 / 8.76 / 8.75.  The adjoint's pairs cost several times
-// more: 64^3 at z = 0.2, 40 %, with 512 / 1024 / 2048 / none: 1.22 / 1.25 / 1.43 / 2.01
-// ms for its two products; 128^3 at z = 1, 10 %, with 256 / 512 / 1024 / 2048 / none
-// 2.57 / 2.08 / 2.09 / 2.12 / 2.33.  4 or 16 parts are no better than 8.
-constexpr int PP_PARTS = 8;
-constexpr int64_t PP_LONG_N = 65536;    // smaller boxes: the second launch costs more than it gives
-
-inline int pp_long_min(int64_t N) { return N < PP_LONG_N ? 0x7fffffff : N < (1 << 19) ? 512 : (int)(N / 256); }
-inline int vjp_long_min(int64_t N) { return N < PP_LONG_N ? 0x7fffffff : N < (1 << 20) ? 512 : (int)(N / 2048); }
 
 struct alignas(16) PPWarpShared {
     union {
@@ -1020,9 +1047,10 @@ struct VjpIO {
 
 // PP part of the vector-Jacobian product: w_i += sum_j A_ij (v_j - v_i) with
 // A_ij = g I + (g'/r) d d^T (the force's Jacobian blocks are symmetric).
-// Warps are dispatched as in the force: a warp inside one narrow row shares a
-// source stream (v_j staged with the positions; the force's test, queues and packed
-// evaluation), other warps walk each lane's 27 cells.  The two products of a gradient
+// Warps are dispatched as in the force: targets in pencil order, one source stream per
+// warp (v_j staged with the positions; the force's test, queues and packed evaluation
+// in compact warps too), long streams shared by eight warps, and each lane's 27 cells for
+// the few warps wider than a stream.  The two products of a gradient
 // over 128^3 particles at z = 1: 2.43 ms with a pair at a time, both branches of the
 // polynomials taken in turn and every warp on its own, now 2.09.
 __device__ __forceinline__ void jacobian_term(float rx, float ry, float rz, float r2, float4 vj, float vix, float viy,
@@ -1203,7 +1231,7 @@ __device__ __forceinline__ void pp_stream(const PPParams &P, PPWarpShared &W, PP
 template <bool PM3, bool COUNT, bool LIST>
 __device__ __forceinline__ void pp_warp(const PPParams &P, int64_t i, PPWarpShared &W) {
     const int j = P.tgt[i];   // with the length's load under way
-    if ((i & ~(int64_t)31) >= *P.tgt_n) return;   // whole warps: places past the last pencil's end
+    if ((i & ~(int64_t)31) >= P.work->places) return;   // whole warps: places past the last pencil's end
     PPBlock B;
     const PPTarget t = warp_target(P, j, B);
     const bool stream = B.xb - B.xa <= PP_WIDEST;
@@ -1225,9 +1253,9 @@ __device__ __forceinline__ void pp_warp(const PPParams &P, int64_t i, PPWarpShar
     if (stream) {
         PPStream T;
         T.total = build_segments(P, W.seg, W.begin, B, T.nseg);
-        const bool split = T.total > P.long_min;
+        const bool split = T.total > P.long_min && P.work->crowd <= P.long_crowd;
         if (LIST && split) {
-            if ((threadIdx.x & 31) == 0) P.long_list[atomicAdd(P.long_n, 1)] = (int32_t)(i >> 5);
+            if ((threadIdx.x & 31) == 0) P.long_list[atomicAdd(&P.work->n, 1)] = (int32_t)(i >> 5);
             return;
         }
         const bool compact = warp_box(W.box, L.mx, L.my, L.mz, L.bcut2, P.bpp2) < PP_COMPACT;
@@ -1291,7 +1319,7 @@ __global__ void __launch_bounds__(PP_PARTS * 32, 32 / PP_PARTS) pp_long_kernel(P
     chain();
     __shared__ PPWarpShared sh[PP_PARTS];
     __shared__ PPPartSums part;
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, n = *P.long_n;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, n = P.work->n;
     PPWarpShared &W = sh[w];
     for (int item = blockIdx.x; item < n; item += gridDim.x) {
         PPBlock B;
@@ -1343,7 +1371,7 @@ __global__ void __launch_bounds__(32, VJP_BLOCKS) pp_vjp_kernel(PPParams P, VjpI
     __shared__ PPVjpWarpShared sh;
     const int64_t i = (int64_t)blockIdx.x * 32 + threadIdx.x;
     const int j = P.tgt[i];   // with the length's load under way
-    if ((int64_t)blockIdx.x * 32 >= *P.tgt_n) return;
+    if ((int64_t)blockIdx.x * 32 >= P.work->places) return;
     PPBlock B;
     const PPTarget t = warp_target(P, j, B);
     const int pi = P.perm[t.slot];
@@ -1352,8 +1380,8 @@ __global__ void __launch_bounds__(32, VJP_BLOCKS) pp_vjp_kernel(PPParams P, VjpI
     if (B.xb - B.xa <= PP_WIDEST) {
         PPStream T;
         T.total = build_segments(P, sh.seg, sh.begin, B, T.nseg);
-        if (T.total > P.long_min) {
-            if (threadIdx.x == 0) P.long_list[atomicAdd(P.long_n, 1)] = blockIdx.x;
+        if (T.total > P.long_min && P.work->crowd <= P.long_crowd) {
+            if (threadIdx.x == 0) P.long_list[atomicAdd(&P.work->n, 1)] = blockIdx.x;
             return;
         }
         const PPLane L = pp_lane<false>(P, t, B);
@@ -1370,7 +1398,7 @@ __global__ void __launch_bounds__(PP_PARTS * 32, VJP_BLOCKS / PP_PARTS) pp_vjp_l
     chain();
     __shared__ PPVjpWarpShared sh[PP_PARTS];
     __shared__ PPPartSums part;
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, n = *P.long_n;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, n = P.work->n;
     PPVjpWarpShared &W = sh[w];
     for (int item = blockIdx.x; item < n; item += gridDim.x) {
         PPBlock B;
@@ -1422,7 +1450,7 @@ __global__ void __launch_bounds__(256) pp_item_cost_kernel(const PPParams *__res
     const int b = item_box[k];
     const PPParams &P = boxes[b];
     const int64_t i0 = (int64_t)(k - base[b]) * PP_ITEM;
-    const int64_t i1 = min(i0 + PP_ITEM, (int64_t)*P.tgt_n);
+    const int64_t i1 = min(i0 + PP_ITEM, (int64_t)P.work->places);
     unsigned s = 0;
     for (int64_t i = i0; i < i1; ++i) {
         const int j = P.tgt[i];
@@ -1500,21 +1528,22 @@ int64_t pp_target_items(int64_t N, int n_ios) {
 
 int64_t pp_target_slots(int64_t N, int n_ios) { return pp_target_items(N, n_ios) * PP_ITEM; }
 
+size_t pp_work_bytes() { return sizeof(PPWork); }
+
 // Cells that can hold PP_SORT_MIN particles.
 int64_t pp_dense_cells(int64_t N) { return N / PP_SORT_MIN; }
 
 static PPParams pp_params(cube2_ctx *ctx, const cube2_particles *p, int accumulate, float kick);
 
 // PP inputs: target order, float positions, dense cells sorted by sub-cell.
-static void launch_pp_inputs(cube2_ctx *ctx, const cube2_particles *p) {
+static void launch_pp_inputs(cube2_ctx *ctx, const cube2_particles *p, const PPParams &P) {
     const int n = ctx->n_ios;
-    int *list_n = ctx->big_n;
-    unsigned *tgt_n = reinterpret_cast<unsigned *>(ctx->big_n + 1);
     {
         ProfScope prof(ctx, P_PP_ORDER, 0);
-        cudaMemsetAsync(ctx->big_n, 0, 3 * sizeof(int), ctx->stream);
-        pp_pencil_kernel<<<(unsigned)(pencils_y(n) * pencils_z(n)), PREP_CTA, 0, ctx->stream>>>(
-            p->count, p->start, n, PP_SORT_MIN, ctx->pp_tgt, tgt_n, ctx->pp_dense, list_n);
+        cudaMemsetAsync(P.work, 0, sizeof(PPWork), ctx->stream);
+        auto *pencils = P.long_min < PP_UNSPLIT ? pp_pencil_kernel<true> : pp_pencil_kernel<false>;
+        pencils<<<(unsigned)(pencils_y(n) * pencils_z(n)), PREP_CTA, 0, ctx->stream>>>(
+            p->count, p->start, n, PP_SORT_MIN, P.long_min, ctx->pp_tgt, ctx->pp_dense, P.work);
     }
     {
         ProfScope prof(ctx, P_PREP, 0);
@@ -1524,7 +1553,7 @@ static void launch_pp_inputs(cube2_ctx *ctx, const cube2_particles *p) {
     {
         ProfScope prof(ctx, P_PP_ORDER, 0);
         launch_chained(ctx->chained, pp_dense_sort_kernel, (unsigned)(ctx->num_sms * 8), 256, 0, ctx->stream,
-            p->off[0], p->off[1], p->off[2], p->count, p->start, ctx->pp_dense, list_n, ctx->pos4, ctx->pp_perm,
+            p->off[0], p->off[1], p->off[2], p->count, p->start, ctx->pp_dense, &P.work->dense, ctx->pos4, ctx->pp_perm,
             ctx->pp_tgt);
     }
     ctx->launches += 3;
@@ -1538,11 +1567,11 @@ cudaError_t launch_pp_vjp(cube2_ctx *ctx, const cube2_particles *p, const float 
     V.v0 = v[0]; V.v1 = v[1]; V.v2 = v[2];
     V.w0 = w[0]; V.w1 = w[1]; V.w2 = w[2];
     V.scale = (float)((double)P.coef / ctx->s_ios);
-    launch_pp_inputs(ctx, p);
+    launch_pp_inputs(ctx, p, P);
     ProfScope prof(ctx, P_PP_VJP, 0);
     launch_chained(ctx->chained, pp_vjp_kernel, (unsigned)(pp_target_slots(ctx->N, ctx->n_ios) / 32), 32, 0, ctx->stream, P, V);
     ctx->launches += 1;
-    if (ctx->N >= PP_LONG_N) {
+    if (P.long_min < PP_UNSPLIT) {
         launch_chained(ctx->chained, pp_vjp_long_kernel, (unsigned)(ctx->num_sms * (VJP_BLOCKS / PP_PARTS)), PP_PARTS * 32, 0, ctx->stream, P, V);
         ctx->launches += 1;
     }
@@ -1554,7 +1583,7 @@ static PPParams pp_params(cube2_ctx *ctx, const cube2_particles *p, int accumula
     P.pos = ctx->pos4;
     P.perm = ctx->pp_perm;
     P.tgt = ctx->pp_tgt;
-    P.tgt_n = reinterpret_cast<unsigned *>(ctx->big_n + 1);
+    P.work = reinterpret_cast<PPWork *>(ctx->pp_work);
     P.count = p->count; P.start = p->start;
     P.acc0 = p->acc[0]; P.acc1 = p->acc[1]; P.acc2 = p->acc[2];
     if (ctx->vel32) {   // FP16 storage: the second kick updates the step's FP32 working copy
@@ -1563,7 +1592,6 @@ static PPParams pp_params(cube2_ctx *ctx, const cube2_particles *p, int accumula
         P.vel0 = p->vel[0]; P.vel1 = p->vel[1]; P.vel2 = p->vel[2];
     }
     P.stats = ctx->pp_stats;
-    P.N = ctx->N;
     P.n_ios = ctx->n_ios;
     {   // ceil(2^(31 + l) / n) with 2^(l-1) < n <= 2^l: exact quotients below 2^31
         int l = 1;
@@ -1588,7 +1616,7 @@ static PPParams pp_params(cube2_ctx *ctx, const cube2_particles *p, int accumula
     P.status = ctx->dev_status;
     P.long_min = pp_long_min(ctx->N);
     P.long_list = ctx->pp_long;
-    P.long_n = ctx->big_n + 2;
+    P.long_crowd = ctx->num_sms * 32 * 32 * 3 / 5;   // 0.6 of the resident warps' targets
     if (ctx->pm3.on) {
         P.pm3_slot = ctx->pm3.slot;
         P.pm3_T = ctx->pm3.T;
@@ -1604,7 +1632,7 @@ cudaError_t launch_pp(cube2_ctx *ctx, const cube2_particles *p, int accumulate, 
     PPParams P = pp_params(ctx, p, accumulate, kick);
     if (ctx->N == 0) return cudaSuccess;
     const unsigned ctas = (unsigned)(pp_target_slots(ctx->N, ctx->n_ios) / (PP_WARPS * 32));
-    launch_pp_inputs(ctx, p);
+    launch_pp_inputs(ctx, p, P);
     if (ctx->defer_pp) {   // an ensemble's persistent kernel runs this box's PP later
         static_assert(sizeof(PPParams) <= sizeof(ctx->pp_deferred), "deferred PP parameters");
         memcpy(ctx->pp_deferred, &P, sizeof P);
@@ -1617,7 +1645,7 @@ cudaError_t launch_pp(cube2_ctx *ctx, const cube2_particles *p, int accumulate, 
                            : (count ? pp_kernel<false, true> : pp_kernel<false, false>),
                        ctas, PP_WARPS * 32, 0, ctx->stream, P);
         ctx->launches += 1;
-        if (ctx->N >= PP_LONG_N) {
+        if (P.long_min < PP_UNSPLIT) {
             launch_chained(ctx->chained, pm3 ? (count ? pp_long_kernel<true, true> : pp_long_kernel<true, false>)
                                : (count ? pp_long_kernel<false, true> : pp_long_kernel<false, false>),
                            (unsigned)(ctx->num_sms * (32 / PP_PARTS)), PP_PARTS * 32, 0, ctx->stream, P);
