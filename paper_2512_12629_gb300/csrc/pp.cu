@@ -402,14 +402,18 @@ struct Sum3 {
 // ranges.  Positions p from begin[s] on are slots p + seg[s].x; a source's
 // coordinates in the warp's frame (cell (xa, ya - 1, za - 1) at 0) are (cell id
 // - seg[s].y) + off_x, row_y + off_y, row_z + off_z with the row's offsets as
-// floats in seg[s].z and .w: exact in FP32 for blocks of up to 128 cells.
+// floats in seg[s].z and .w: exact in FP32, and so are their differences, while they
+// are below 256 cells.
 constexpr int PP_SEGS = 3 * PP_ROWS;
 
-// A warp is on the shared stream when it spans at most PP_WIDEST + 1 cells along x;
-// the few wider ones (fewer than 32 particles in that many slabs) walk each lane's own
-// 27 cells.  The line is the same for every launch: the two paths add in different
-// orders, and an ensemble gives its boxes the bits of their own steps.
-constexpr int PP_WIDEST = 64;
+// A warp is on the shared stream when it spans at most PP_WIDEST + 1 cells along x, as
+// far as its frame is exact; the few wider ones (fewer than 32 particles in that many
+// slabs) walk each lane's own 27 cells.  A lane of a halo at the end of a wide warp
+// walks alone: 70000 particles in 96^3 cells, half of them in 64 clumps, 0.21 ms with
+// streams of up to 65 cells, now 0.16; 10^6 evenly in 256^3 cells 0.24 -> 0.22.  The line
+// is the same for every launch: the two paths add in different orders, and an ensemble
+// gives its boxes the bits of their own steps.
+constexpr int PP_WIDEST = 250;
 
 struct PPBlock {
     int xa, xb, ya, yb, za, zb;

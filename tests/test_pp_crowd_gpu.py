@@ -1,5 +1,7 @@
-"""PP in boxes in which as many targets have long streams as are still split between
-warps, and more (each stream then stays with its warp).  Force and adjoint product against the FP64 oracle, and the
+"""PP where the paths of the source streams change: boxes in which as many targets have
+long streams as are still split between warps, and more (each stream then stays with its
+warp); warps wider than a stream may be, which walk each lane's own cells, beside ones
+that are just not.  Force and adjoint product against the FP64 oracle, and the
 persistent kernel bit for bit against the box's own launches.
 
 Tolerances as in the other PP tests: |F_gpu - F_or| <= 1e-5 (scale + |F_or|) with the
@@ -28,13 +30,21 @@ from paper_2512_12629_gb300 import cube2  # noqa: E402
 
 def _case(name):
     rng = np.random.default_rng(29)
-    n, mesh = 16, Level(32, 2.0)             # 16^3 cells, evenly: every stream is long
-    x = rng.uniform(0, 16, (3, int(name)))
+    if name == "wide":       # 256 cells a side: pencils whose particles lie at both ends, 251, 252 and 253 cells apart
+        n, mesh = 256, Level(128, 0.5)
+        x = rng.uniform(0, 256, (3, 600))
+        for k, gap in enumerate((250, 251, 252, 255)):
+            x[0, 40 * k:40 * k + 20] = 0.5 + 0.2 * rng.normal(size=20) % 0.5
+            x[0, 40 * k + 20:40 * k + 40] = gap + rng.uniform(0, 1, 20)
+            x[1:, 40 * k:40 * k + 40] = np.array([[10.0], [20.0 * k + 2]]) + rng.uniform(0, 1, (2, 40))
+    else:                    # 16^3 cells, evenly: every stream is long
+        n, mesh = 16, Level(32, 2.0)
+        x = rng.uniform(0, 16, (3, int(name)))
     w = C1.with_(name=f"crowd-{name}", n_ios=n, box=float(n), levels=(mesh,), b_pp=0.1)
     return w, ios_from_positions(x, np.zeros_like(x), n, w.box)
 
 
-NAMES = ["90000", "100000"]
+NAMES = ["90000", "100000", "wide"]
 
 
 @pytest.mark.parametrize("name", NAMES)
@@ -56,6 +66,9 @@ def test_force(name):
     ctx.pp_count(True)
     ctx.pp_force(p)
     assert torch.equal(p.acc, first)
+    if name == "wide":
+        lane = ctx.pp_stats_paths()[2:]
+        assert lane[1] > 0                    # some warps walked
     ctx.close()
 
 
