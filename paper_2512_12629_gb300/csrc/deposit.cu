@@ -60,7 +60,13 @@ __device__ __forceinline__ float u64_delta_to_f32(uint64_t acc, uint64_t m, floa
 constexpr int DEP_THREADS = 384;       // four CTAs per SM with 40 registers (256: 0.79 ms, 512: 0.80 against 0.75)
 constexpr int COARSE = 8;              // owned mesh cells per axis of a coarse brick
 constexpr int COARSE_WARP = 96;        // particles from which a coarse block gets a warp
-// mean particles per cell from which a brick's lanes take chunks (always: 0.96 ms at z = 49 instead of 0.81)
+// Mean particles per cell from which a brick's lanes take DENSE_RUN particles in a row
+// (always: 0.96 ms at z = 49 instead of 0.81).  Longer runs than that have a line of
+// every array in use per lane, more than the L1 holds beside four CTAs' tiles: 16
+// particles a cell in 96^3 cells, 192^3 mesh, with runs of 4 / 8 / 16 / 32 / a 32nd of
+// the warp's 0.27 / 0.33 / 0.43 / 0.64 / 0.73 ms, 64 a cell in 32^3 0.23 / 0.27 / 0.34 /
+// 0.52 / 0.86; the 256^3 run at z = 0 1.185 to 1.20 ms.
+constexpr int DENSE_RUN = 4;            // a power of two
 constexpr int DENSE_ITEMS = 3;
 
 // The high word of a weight, with the carry of its low word's addition to old.
@@ -193,14 +199,12 @@ __device__ __forceinline__ void deposit_items(const DepParams &P, const Segments
                                               unsigned int *lo, unsigned int *hi, int ext0, int ext1, int ext2) {
     using Tile = DepTile<(BI << UP)>;
     // Even bricks: lanes on consecutive particles (their loads share lines).
-    // Dense ones: each lane a contiguous chunk of its warp's items, so that the
-    // lanes sit in different cells and fewer of their corners hit the same words.
+    // Dense ones: each lane DENSE_RUN in a row, so that the lanes sit in different
+    // cells or parts of one and fewer of their corners hit the same words.
     const int nwarps = DEP_THREADS / 32, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int per_w = ((total + nwarps - 1) / nwarps + 31) & ~31;
-    const bool chunks = total > DENSE_ITEMS * (BI + 2) * (BI + 2) * (BI + 2);
-    const int step = chunks ? 1 : 32;
-    const int it0 = w * per_w + (chunks ? lane * (per_w >> 5) : lane);
-    const int it1 = min(total, chunks ? it0 + (per_w >> 5) : (w + 1) * per_w);
+    const int last = total > DENSE_ITEMS * (BI + 2) * (BI + 2) * (BI + 2) ? DENSE_RUN - 1 : 0;   // of a run, per_w % 32 == 0
+    const int it0 = w * per_w + lane * (last + 1), it1 = min(total, (w + 1) * per_w);
     if (it0 >= it1) return;
     int sg = 0, hi_s = nseg - 1;   // last segment with pre <= it0
     while (sg < hi_s) {
@@ -209,7 +213,7 @@ __device__ __forceinline__ void deposit_items(const DepParams &P, const Segments
         else hi_s = mid - 1;
     }
     int next = G.pre[sg + 1];
-    for (int t = it0; t < it1; t += step) {
+    for (int t = it0; t < it1; t += (t & last) == last ? 32 + 31 * last : 1) {
         while (next <= t) next = G.pre[++sg + 1];
         const int p = G.first[sg] + t, info = G.info[sg];
         const int hx = P.cellid[p] - G.c0[sg], hy = info & 0xff, hz = info >> 8;
