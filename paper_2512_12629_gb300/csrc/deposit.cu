@@ -59,7 +59,13 @@ __device__ __forceinline__ float u64_delta_to_f32(uint64_t acc, uint64_t m, floa
 
 constexpr int DEP_THREADS = 384;       // four CTAs per SM with 40 registers (256: 0.79 ms, 512: 0.80 against 0.75)
 constexpr int COARSE = 8;              // owned mesh cells per axis of a coarse brick
-constexpr int COARSE_WARP = 96;        // particles from which a coarse block gets a warp
+// Coarse blocks of COARSE_WARP particles get a warp, if they are few.  Of more than
+// COARSE_FEW in a brick the warps take only those of COARSE_MEANS times the average, and
+// threads the others: a warp does its share one after another, about 1.5 us each (16
+// particles a cell, evenly, in 64^3 cells: 0.213 ms with all of them by warps, 0.08 by
+// threads; 64^3 particles, half in clumps, 0.044 against 0.105).
+constexpr int COARSE_WARP = 96, COARSE_FEW = 96, COARSE_MEANS = 4;
+constexpr int COARSE_TOP = 4096;       // always a warp from here on: eight smaller blocks cannot overflow a cell
 // Mean particles per cell from which a brick's lanes take DENSE_RUN particles in a row
 // (always: 0.96 ms at z = 49 instead of 0.81).  Longer runs than that have a line of
 // every array in use per lane, more than the L1 holds beside four CTAs' tiles: 16
@@ -326,18 +332,20 @@ struct CoarseRow {
     __device__ int size() const { return end - beg + end2 - beg2; }
 };
 
-constexpr size_t COARSE_SMEM = DepTile<COARSE>::SMEM + sizeof(int) * (COARSE + 1) * (COARSE + 1) * (COARSE + 1);
+constexpr size_t COARSE_SMEM = DepTile<COARSE>::SMEM + 2 * sizeof(int) * (COARSE + 1) * (COARSE + 1) * (COARSE + 1);
 
 __device__ __forceinline__ void coarse_brick(const DepParams &P, int brick, unsigned int *words) {
     using Tile = DepTile<COARSE>;
     __shared__ int s_n;
+    __shared__ unsigned long long s_sum;
     unsigned int *lo = words, *hi = words + Tile::CELLS;
-    int *s_list = reinterpret_cast<int *>(words + 2 * Tile::CELLS);   // blocks that get a warp
+    int *s_list = reinterpret_cast<int *>(words + 2 * Tile::CELLS);   // large blocks
+    int *s_size = s_list + (COARSE + 1) * (COARSE + 1) * (COARSE + 1);
     const int n = P.n_ios;
     const int ox = brick % P.nbx * COARSE, oy = brick / P.nbx % P.nbx * COARSE, oz = brick / (P.nbx * P.nbx) * COARSE;
     const int ex = min(COARSE, P.n - ox), ey = min(COARSE, P.n - oy), ez = min(COARSE, P.n - oz);
     Tile::zero(words);
-    if (threadIdx.x == 0) s_n = 0;
+    if (threadIdx.x == 0) s_n = 0, s_sum = 0;
     __syncthreads();
     // block (bx, by, bz): lower corner b - 1 (owned-local), IOS cells 2 (o + b) - 1 and 2 (o + b) per axis
     auto rows = [&](int b, int (&r)[4], int &xa, int &xb, int &base) {
@@ -352,18 +360,7 @@ __device__ __forceinline__ void coarse_brick(const DepParams &P, int brick, unsi
     auto take = [&](Moments &m, int j, int dx, int k) {   // fraction: half a cell for the second one, plus half the offset
         m.add((dx << 15) + (P.off0[j] >> 1), ((k & 1) << 15) + (P.off1[j] >> 1), ((k >> 1) << 15) + (P.off2[j] >> 1));
     };
-    const int nblocks = (ex + 1) * (ey + 1) * (ez + 1);
-    for (int b = threadIdx.x; b < nblocks; b += DEP_THREADS) {
-        int r[4], xa, xb, base;
-        rows(b, r, xa, xb, base);
-        int many = 0;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) many += CoarseRow(P, r[k], xa, xb).size();
-        if (many == 0) continue;
-        if (many >= COARSE_WARP) {
-            s_list[atomicAdd(&s_n, 1)] = b;
-            continue;
-        }
+    auto by_thread = [&](const int (&r)[4], int xa, int xb, int base) {
         Moments m;
         m.clear();
 #pragma unroll 1
@@ -373,10 +370,40 @@ __device__ __forceinline__ void coarse_brick(const DepParams &P, int brick, unsi
             for (int j = R.beg2; j < R.end2; ++j) take(m, j, 1, k);
         }
         add_moments<Tile::W, false>(lo, hi, base, m, P.status);
+    };
+    const int nblocks = (ex + 1) * (ey + 1) * (ez + 1);
+    for (int b = threadIdx.x; b < nblocks; b += DEP_THREADS) {
+        int r[4], xa, xb, base;
+        rows(b, r, xa, xb, base);
+        int many = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) many += CoarseRow(P, r[k], xa, xb).size();
+        if (many == 0) continue;
+        if (many >= COARSE_WARP) {
+            const int at = atomicAdd(&s_n, 1);
+            s_list[at] = b;
+            s_size[at] = many;
+            atomicAdd(&s_sum, (unsigned long long)many);
+            continue;
+        }
+        by_thread(r, xa, xb, base);
     }
     __syncthreads();
+    int warp_from = 0;
+    if (s_n > COARSE_FEW) {
+        static_assert(8 * COARSE_TOP < FIX, "no watch on the blocks that threads take");
+        warp_from = (int)min((unsigned long long)COARSE_TOP, COARSE_MEANS * s_sum / s_n);
+        for (int i = threadIdx.x; i < s_n; i += DEP_THREADS) {
+            if (s_size[i] >= warp_from) continue;
+            int r[4], xa, xb, base;
+            rows(s_list[i], r, xa, xb, base);
+            by_thread(r, xa, xb, base);
+        }
+        __syncthreads();   // before the watched additions
+    }
     const int lane = threadIdx.x & 31;
     for (int i = threadIdx.x >> 5; i < s_n; i += DEP_THREADS / 32) {
+        if (s_size[i] < warp_from) continue;
         int r[4], xa, xb, base, many = 0;
         rows(s_list[i], r, xa, xb, base);
         Moments m;
