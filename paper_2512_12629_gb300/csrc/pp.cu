@@ -211,6 +211,8 @@ constexpr int PP_PARTS = 8;
 constexpr int PP_UNSPLIT = 0x7fffffff;
 constexpr int64_t PP_LONG_N = 65536;    // smaller boxes: the second launch costs more than it gives
 
+constexpr int LONG_SLAB = 8;            // targets of a pencil's slab of cells from which its streams are looked at
+
 inline int pp_long_min(int64_t N) { return N < PP_LONG_N || N >= (1 << 19) ? PP_UNSPLIT : 512; }
 inline int vjp_long_min(int64_t N) { return N < PP_LONG_N || N >= (1 << 22) ? PP_UNSPLIT : N < (1 << 20) ? 512 : (int)(N / 2048); }
 
@@ -276,15 +278,17 @@ __global__ void __launch_bounds__(PREP_CTA) pp_pencil_kernel(const int32_t *__re
         }
         __syncthreads();
         if (LONG) {   // a stream: the rows around the pencil's, over the slabs of 32 targets and one on each side
+            // thinner slabs hold few of the targets with long streams, and a nearly empty box hundreds of slabs
+            // for each particle (10^5 evenly in 192^3 cells with them counted: PP 0.094 ms instead of 0.07)
             int near = 0;
-            if (sum > 0) {
+            if (sum >= LONG_SLAB) {
 #pragma unroll 4
                 for (int k = 0; k < PP_ROWS; ++k) {
                     const int64_t r = ((int64_t)wrap(z0 - 1 + k / (PEN_Y + 2), n) * n + wrap(y0 - 1 + k % (PEN_Y + 2), n)) * n;
                     near += count[r + wrap(x - 1, n)] + count[r + x] + count[r + wrap(x + 1, n)];
                 }
+                near += (int)((int64_t)near * 32 / (3 * sum));
             }
-            if (sum > 0) near += (int)((int64_t)near * 32 / (3 * sum));
             const int crowd = __reduce_add_sync(0xffffffffu, near > long_min ? sum : 0);
             if (lane == 0 && crowd) atomicAdd(&work->crowd, crowd);
         }
