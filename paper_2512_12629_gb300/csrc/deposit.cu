@@ -63,8 +63,10 @@ constexpr int COARSE = 8;              // owned mesh cells per axis of a coarse 
 // COARSE_FEW in a brick the warps take only those of COARSE_MEANS times the average, and
 // threads the others: a warp does its share one after another, about 1.5 us each (16
 // particles a cell, evenly, in 64^3 cells: 0.213 ms with all of them by warps, 0.08 by
-// threads; 64^3 particles, half in clumps, 0.044 against 0.105).
-constexpr int COARSE_WARP = 96, COARSE_FEW = 96, COARSE_MEANS = 4;
+// threads; 64^3 particles, half in clumps, 0.044 against 0.105).  Warps from 96 / 128 /
+// 160 particles on: 12 a cell in 32^3 cells 0.091 / 0.056 / 0.054 ms, 64^3 particles,
+// half in clumps, 0.045 / 0.047 / 0.048, the 256^3 run at z = 0 1.178 / 1.186 / 1.194.
+constexpr int COARSE_WARP = 128, COARSE_FEW = 96, COARSE_MEANS = 4;
 constexpr int COARSE_TOP = 4096;       // always a warp from here on: eight smaller blocks cannot overflow a cell
 // Mean particles per cell from which a brick's lanes take DENSE_RUN particles in a row
 // (always: 0.96 ms at z = 49 instead of 0.81).  Longer runs than that have a line of

@@ -1,6 +1,6 @@
 """The CIC deposit in evenly dense boxes, where bricks go from one division of their
 particles to the other: lanes on single particles and on runs of four, coarse blocks by
-threads and by warps (96 particles, four times the brick's mean, 4096), with and without
+threads and by warps (128 particles, four times the average of those, 4096), with and without
 clumps, whole and partial bricks; accumulators and FP32 grids against the oracle's
 integers, bit for bit.
 """
