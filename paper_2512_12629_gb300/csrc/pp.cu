@@ -74,6 +74,7 @@ struct PPParams {
     const int32_t *pm3_slot;
     int pm3_T, pm3_ns;
     float bcut2_3, inv_bcut_3;
+    bool even;                        // dense throughout (pp_compact)
     int long_min;                     // longer streams go to the list and are shared by PP_PARTS warps
     int32_t *long_list;               // target places / 32 of those warps
     int long_crowd;                   // most targets with long streams with which that is done
@@ -1197,7 +1198,26 @@ __device__ __forceinline__ PPTarget warp_target(const PPParams &P, int j, PPBloc
 // The estimate takes the sources as evenly spread; around haloes more of them
 // are in range.  PP at z = 0 of the 256^3 run with 6 / 9 / 14 / 20: 9.8 / 9.0 /
 // 8.7 / 8.7 ms; 512^3 particles at z = 1 with 6 / 9 / 14: 25.0 / 23.4 / 22.9 ms.
-constexpr float PP_COMPACT = 14.0f;
+//
+// Where the sources are as even as the estimate has them, 9 is the better line, which
+// matters in boxes that are dense throughout: 8 / 9 / 11 particles a cell, evenly, in
+// 64^3, 48^3 and 64^3 cells 0.82 / 0.50 / 1.60 ms with 14, 0.71 / 0.44 / 1.48 with 9.
+// Even: the density of the whole stream is PP_EVEN_LO to PP_EVEN_HI times the targets' own (32 in
+// their box).  With about one particle a cell the dense places are haloes, where the
+// rule costs more than it gives (the 256^3 run at z = 0 9.27 -> 9.36 ms): it is for
+// boxes of PP_EVEN_MEAN particles a cell or more.
+constexpr float PP_COMPACT = 14.0f, PP_COMPACT_EVEN = 9.0f;
+constexpr float PP_EVEN_LO = 1.3f, PP_EVEN_HI = 3.0f;
+constexpr int PP_EVEN_MEAN = 4;
+
+__device__ __forceinline__ bool pp_compact(const PPParams &P, const float4 *box, float candidates, int total, const PPBlock &B) {
+    if (!P.even || candidates < PP_COMPACT_EVEN) return candidates < PP_COMPACT;
+    const float4 lo = box[0], hi = box[1];
+    const float own = (hi.x - lo.x) * (hi.y - lo.y) * (hi.z - lo.z) * (1.0f / 32.0f);   // cells a target
+    const float around = (float)((B.xb - B.xa + 3) * (B.yb - B.ya + 3) * (B.zb - B.za + 3));
+    const float ratio = (float)total * own / around;
+    return candidates < (ratio > PP_EVEN_LO && ratio < PP_EVEN_HI ? PP_COMPACT_EVEN : PP_COMPACT);
+}
 
 // The targets as the pair loops see them.
 template <bool PM3>
@@ -1266,7 +1286,7 @@ __device__ __forceinline__ void pp_warp(const PPParams &P, int64_t i, PPWarpShar
             if ((threadIdx.x & 31) == 0) P.long_list[atomicAdd(&P.work->n, 1)] = (int32_t)(i >> 5);
             return;
         }
-        const bool compact = warp_box(W.box, L.mx, L.my, L.mz, L.bcut2, P.bpp2) < PP_COMPACT;
+        const bool compact = pp_compact(P, W.box, warp_box(W.box, L.mx, L.my, L.mz, L.bcut2, P.bpp2), T.total, B);
         if constexpr (LIST) {
             T.init(P, W);
             pp_stream<COUNT>(P, W, T, L, compact, a, pairs, cands);
@@ -1335,7 +1355,7 @@ __global__ void __launch_bounds__(PP_PARTS * 32, 32 / PP_PARTS) pp_long_kernel(P
         const PPLane L = pp_lane<PM3>(P, t, B);
         PPStream T;
         const int all = build_segments(P, W.seg, W.begin, B, T.nseg);
-        const bool compact = warp_box(W.box, L.mx, L.my, L.mz, L.bcut2, P.bpp2) < PP_COMPACT;
+        const bool compact = pp_compact(P, W.box, warp_box(W.box, L.mx, L.my, L.mz, L.bcut2, P.bpp2), all, B);
         T.init_part(P, W, all, w);
         Sum3 a;
         unsigned pairs = 0, cands = 0;
@@ -1608,6 +1628,7 @@ static PPParams pp_params(cube2_ctx *ctx, const cube2_particles *p, int accumula
         P.div_shift = l - 1;
     }
     P.accumulate = accumulate;
+    P.even = ctx->N >= PP_EVEN_MEAN * ctx->n_cells;
     const double s = ctx->s_ios;
     // Separations are 0 or at least 2^-16 cells: shorter lengths all act like these, whose
     // powers stay within FP32 (the square of a softening that underflowed to 0 would no

@@ -1,7 +1,7 @@
 """PP where the paths of the source streams change: boxes in which as many targets have
 long streams as are still split between warps, and more (each stream then stays with its
-warp); warps wider than a stream may be, which walk each lane's own cells, beside ones
-that are just not.  Force and adjoint product against the FP64 oracle, and the
+warp); boxes dense throughout; warps wider than a stream may be, which walk each lane's
+own cells, beside ones that are just not.  Force and adjoint product against the FP64 oracle, and the
 persistent kernel bit for bit against the box's own launches.
 
 Tolerances as in the other PP tests: |F_gpu - F_or| <= 1e-5 (scale + |F_or|) with the
@@ -37,6 +37,9 @@ def _case(name):
             x[0, 40 * k:40 * k + 20] = 0.5 + 0.2 * rng.normal(size=20) % 0.5
             x[0, 40 * k + 20:40 * k + 40] = gap + rng.uniform(0, 1, 20)
             x[1:, 40 * k:40 * k + 40] = np.array([[10.0], [20.0 * k + 2]]) + rng.uniform(0, 1, (2, 40))
+    elif name == "even":     # eight a cell: between the warps that evaluate every pair and those that test first
+        n, mesh = 16, Level(32, 2.0)
+        x = np.concatenate([rng.uniform(0, 16, (3, 33000)), 8 + rng.normal(size=(3, 1000))], 1) % 16
     else:                    # 16^3 cells, evenly: every stream is long
         n, mesh = 16, Level(32, 2.0)
         x = rng.uniform(0, 16, (3, int(name)))
@@ -44,7 +47,7 @@ def _case(name):
     return w, ios_from_positions(x, np.zeros_like(x), n, w.box)
 
 
-NAMES = ["90000", "100000", "wide"]
+NAMES = ["90000", "100000", "even", "wide"]
 
 
 @pytest.mark.parametrize("name", NAMES)
@@ -72,7 +75,7 @@ def test_force(name):
     ctx.close()
 
 
-@pytest.mark.parametrize("name", NAMES[1:])
+@pytest.mark.parametrize("name", NAMES[1:2] + NAMES[3:])
 def test_force_vjp(name):
     w, st = _case(name)
     n_part = int(st["count"].sum())
