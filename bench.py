@@ -232,7 +232,9 @@ def bus_id_of(dev):
 
 # ------------------------------------------------------ algorithmic bytes
 def algorithmic_bytes(w, n_part, cls, level):
-    """Compulsory HBM bytes of one launch group of a kernel class (each array once)."""
+    """Compulsory HBM bytes of one launch group of a kernel class (each array once); None for
+    classes whose work depends on the state: the sorts inside large cells, and the PP order
+    (two kernels, one of them over the dense cells only)."""
     N, C = n_part, w.n_ios ** 3
     meshes = [lv.n_mesh for lv in w.levels]
     n = meshes[level] if level < len(meshes) else meshes[-1]
@@ -249,18 +251,21 @@ def algorithmic_bytes(w, n_part, cls, level):
         "fft_y_inv": 16 * half,
         "fft_x_inv": 8 * half + 4 * n ** 3,
         "interp": 4 * n ** 3 + 22 * N if tsc else sum(4 * m ** 3 for m in meshes) + 22 * N,
-        "pp": 58 * N + 8 * C,
-        "kick": 36 * N,
-        "kick_drift": 68 * N + 4 * C,
+        # positions 16, target and particle of each place 4 + 4, force and momentum in and out 48
+        "pp": 72 * N + 8 * C,
+        # FP16 contexts: the encoder (momenta 12, cell 4, codes 6; a scale per cell)
+        "kick": 22 * N + 4 * C if getattr(w, "vel_fp16", False) else 36 * N,
+        # offsets 6, momenta and forces 24, cell 4; records 24, slot 4; the histogram zeroed
+        "kick_drift": 62 * N + 4 * C,
         "scan": 8 * C,
         "scatter": 16 * N,
-        "sort": 8 * C + 8 * N,
-        "gather": 48 * N,
+        "sort": 4 * C,           # the list of the cells to sort
+        # slots 4, records 24; map 4, offsets 6, momenta 12, cell 4
+        "gather": 54 * N,
         "cellid": 8 * C + 4 * N,
         "green": 4 * green_len,
-        "prep": 26 * N,
-        "pp_order": 4 * C + 26 * N,
-        "sort_big": 8 * N,
+        # offsets 6, cell 4; positions 16, map 4
+        "prep": 30 * N,
     }
     # the third level's classes move data-dependent amounts (the refined
     # subtiles' local boxes): no algorithmic figure
@@ -271,11 +276,13 @@ def algorithmic_bytes(w, n_part, cls, level):
 # counts them: the separation 3, r^2 5, the reciprocal square root and the
 # scaled distance u = r / b 3, one shell polynomial of R_PP in Horner form 14,
 # the 1/r^3 scaling and the product with the force factor 2, accumulation of
-# the three components 3: 30.  The kernel as written also evaluates the second
-# shell polynomial and forms the powers of v = 1 - u (45 in all), and tests
-# every candidate (separation 3 and r^2 - b^2 6); both are reported beside it.
+# the three components 3: 30.  The kernel as written evaluates both shell
+# polynomials of a pair (43 in all); its warps either test every candidate
+# (separation 3 and r^2 - b^2 6) and evaluate the pairs found, or evaluate every
+# candidate without a test (29 or 43 each).  "as written" counts 43 a pair, and
+# with 9 a candidate beside it the work of the warps that test: a lower bound.
 PP_FLOPS_PAIR = 30
-PP_FLOPS_PAIR_AS_WRITTEN = 45
+PP_FLOPS_PAIR_AS_WRITTEN = 43
 PP_FLOPS_CANDIDATE = 9
 
 
@@ -313,7 +320,7 @@ def pp_roofline(pairs, cands, launches, per_launch_ms, peak_tflops, sms, sm_mhz,
     flops = pairs * PP_FLOPS_PAIR / launches
     sec = per_launch_ms / 1e3
     achieved = flops / sec / 1e12
-    return {"bound": "alu", "kernel": "pp_kernel (shared-stream and per-lane paths)", "achieved": achieved,
+    return {"bound": "alu", "kernel": "pp_kernel (source streams; per-lane walk in nearly empty regions)", "achieved": achieved,
             "peak": peak_tflops, "unit": "TFLOP/s", "frac": achieved / peak_tflops,
             "peak_source": f"measured: FP32 FMA probe kernel (cube2_fma_probe), CUDA events, {sms} SMs",
             "peak_derived": fp32_peak_derived(sms, sm_mhz), "peak_derived_note":
@@ -574,7 +581,7 @@ def run_ensemble(args):
                        "recording": "step by step: boxes' steps up to their PP inputs on LPT-placed graph branches, "
                                     "then one persistent PP kernel over all boxes (cost-ordered device queue)",
                        "autotuned": {"n_streams": best.n_streams, "pp_ctas_per_sm": best.pp_ctas_per_sm,
-                                     "pp_wmax": best.pp_wmax, "tuning_s": tune_s, "tuned_ms": tune_ms},
+                                     "tuning_s": tune_s, "tuned_ms": tune_ms},
                        "step": "one graph launch = every box's 20 steps; states reset to the ICs before each",
                        "l2": "inputs larger than L2 (~1 GB of particles and meshes)", "parallelism": "boxes split over ranks"},
             "per_box_graph": {"value": value_b, "unit": UNIT, "ms_per_launch": ms_b / args.steps,
