@@ -156,24 +156,40 @@ struct Plan {
     }
 };
 
-__global__ void twiddle_rows_kernel(float2 *tw, int n) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    for (int k = 0; k < 4; ++k) {
-        const bool xp = k >= 2, inv = k % 2 == 1;
-        const int S = stages_of(n, xp);
-        int span = radix_at(n, inv ? S - 1 : 0, xp);
-        for (int s = 1; s < S; ++s) {
-            const int R = radix_at(n, inv ? S - 1 - s : s, xp), nb = n / R, at = twiddle_row(n, xp, inv, s);
-            if (idx >= at && idx < at + (R - 1) * nb) {
-                const int r = (idx - at) / nb + 1, j = (idx - at) % nb;
-                double si, co;
-                sincospi((inv ? 2.0 : -2.0) * (double)(r * (j % span)) / (double)(span * R), &si, &co);
-                tw[idx] = make_float2((float)co, (float)si);
-                return;
-            }
-            span *= R;
+// The fraction of a turn of entry idx, if it lies in one of a line's rows from stage s on.
+template <int N, bool XP, bool INV, int s>
+__device__ __forceinline__ void twiddle_turn(int idx, int &num, int &den) {
+    if constexpr (s < stages_of(N, XP)) {
+        constexpr int R = Plan<N, INV, XP>::radix(s), NB = N / R, NS = Plan<N, INV, XP>::span(s), at = twiddle_row(N, XP, INV, s);
+        if (idx >= at && idx < at + (R - 1) * NB) {
+            num = (INV ? 1 : -1) * (((idx - at) / NB + 1) * ((idx - at) % NB % NS));
+            den = NS * R;
         }
+        twiddle_turn<N, XP, INV, s + 1>(idx, num, den);
     }
+}
+
+// Sizes are template parameters: with the rows looked up at run time the kernel took
+// longer than the five passes of a small mesh, whose allocation-free solve makes its
+// twiddles in each call (64^3 81 us a call, 96^3 172).
+constexpr int TWIDDLE_THREADS = 64;
+template <int N>
+__global__ void __launch_bounds__(TWIDDLE_THREADS) twiddle_rows_kernel(float2 *tw) {
+    const int idx = blockIdx.x * TWIDDLE_THREADS + threadIdx.x;
+    if (idx >= twiddle_entries(N)) return;
+    int num = 0, den = 1;
+    twiddle_turn<N, false, false, 1>(idx, num, den);
+    twiddle_turn<N, false, true, 1>(idx, num, den);
+    twiddle_turn<N, true, false, 1>(idx, num, den);
+    twiddle_turn<N, true, true, 1>(idx, num, den);
+    double si, co;
+    sincospi(2.0 * (double)num / (double)den, &si, &co);
+    tw[idx] = make_float2((float)co, (float)si);
+}
+template <int N>
+cudaError_t make_twiddles(float2 *tw, cudaStream_t st) {
+    twiddle_rows_kernel<N><<<(twiddle_entries(N) + TWIDDLE_THREADS - 1) / TWIDDLE_THREADS, TWIDDLE_THREADS, 0, st>>>(tw);
+    return cudaGetLastError();
 }
 
 // Values of stage s's butterflies j twiddled and transformed; nothing to twiddle in stage 0.
@@ -670,11 +686,12 @@ struct Launcher {
     }
 };
 
-enum class Op { Forward, ZGreen, ZForward, Inverse };
+enum class Op { Twiddles, Forward, ZGreen, ZForward, Inverse };
 
 template <int N>
 cudaError_t run_op(cube2_ctx *ctx, Level &Lv, Op op) {
     switch (op) {
+        case Op::Twiddles: return make_twiddles<N>(Lv.tw, ctx->stream);
         case Op::Forward: return Launcher<N>::forward(ctx, Lv);
         case Op::ZGreen: return Launcher<N>::z_pass(ctx, Lv, true);
         case Op::ZForward: return Launcher<N>::z_pass(ctx, Lv, false);
@@ -711,9 +728,8 @@ cudaError_t dispatch(cube2_ctx *ctx, Level &Lv, Op op) {
 int64_t fft_twiddle_entries(int n) { return twiddle_entries(n); }
 
 cudaError_t launch_init_twiddles(cube2_ctx *ctx, Level &L) {
-    twiddle_rows_kernel<<<(twiddle_entries(L.n) + 255) / 256, 256, 0, ctx->stream>>>(L.tw, L.n);
     ctx->launches++;
-    return cudaGetLastError();
+    return dispatch(ctx, L, Op::Twiddles);
 }
 
 bool fft_size_supported(int n) {
@@ -768,10 +784,11 @@ std::mutex g_noalloc_mutex;
 void *g_noalloc_ptr[NOALLOC_MAX_DEVICES] = {};
 
 template <int N>
-cudaError_t noalloc_passes(const float *rho, float2 *spec, const float *gpad, float *phi, const float2 *tw, int kxp,
+cudaError_t noalloc_passes(const float *rho, float2 *spec, const float *gpad, float *phi, float2 *tw, int kxp,
                            cudaStream_t st) {
-    const cudaError_t opt = Launcher<N>::setup();
-    if (opt != cudaSuccess) return opt;
+    cudaError_t e = Launcher<N>::setup();
+    if (e == cudaSuccess) e = make_twiddles<N>(tw, st);
+    if (e != cudaSuccess) return e;
     constexpr int L = Tile<N, true>::L;
     static_assert(L == Tile<N, false>::L, "one grid for y and z");
     static_assert(twiddle_entries(N) <= NOALLOC_TWIDDLES && (size_t)N * N * ((N / 2 + 16) / 16 * 16) <= NOALLOC_HALF,
@@ -844,10 +861,6 @@ extern "C" int cube2_solve_pm_noalloc(const float *rho, const float *green, floa
                           (size_t)n * n, cudaMemcpyDeviceToDevice, st);
     if (e == cudaSuccess && (size_t)kxp > nh)
         e = cudaMemset2DAsync(gpad + nh, kxp * sizeof(float), 0, (kxp - nh) * sizeof(float), (size_t)n * n, st);
-    if (e == cudaSuccess) {
-        twiddle_rows_kernel<<<(twiddle_entries(n) + 127) / 128, 128, 0, st>>>(tw, n);
-        e = cudaGetLastError();
-    }
     if (e == cudaSuccess) {
         switch (n) {
             case 8: e = noalloc_passes<8>(rho, spec, gpad, phi, tw, kxp, st); break;
