@@ -481,7 +481,8 @@ int cube2_ensemble_create(cube2_ensemble **out, cube2_ctx *const *ctxs, cube2_pa
  *                   (%globaltimer) and otherwise records CUBE2_ERR_TIMEOUT
  *                   (cube2_ensemble_check) and returns.  Boxes with the third
  *                   level or FP16 velocities are refused (CUBE2_ERR_STATE).
- *   pp_ctas_per_sm  persistent grid: CTAs per SM (1..16)
+ *   pp_ctas_per_sm  persistent grid: CTAs per SM (1..16; eight are resident at
+ *                   a time, the others start as these end and find the queue empty)
  *   pp_wmax         0..64, accepted and without effect: the widest shared PP stream is
  *                   the same everywhere, so that every option gives the same bits
  *   timeout_ms      bound of the persistent kernel's wait (> 0)                  */

@@ -247,8 +247,15 @@ __device__ __forceinline__ void set_status(int *status, int bit) { atomicOr(stat
 // It saves the start of each of a small box's dozen short kernels: the force of 32^3
 // particles 72.7 -> 58.2 us, a step of 64^3 425 -> 405, placing 128^3 positions 178 ->
 // 165.  In large boxes the waiting CTAs only hold places (a 256^3 step: 4.93 -> 5.06
-// ms), and so they do between the branches of an ensemble's graph (1107 -> 1130 us):
-// contexts of more than CHAINED_MAX particles and recordings launch plainly.
+// ms; 4.51 -> 4.60 of two in a row), and so they do between the branches of an
+// ensemble's graph (1107 -> 1130 us): contexts of more than CHAINED_MAX particles and
+// recordings launch plainly.  Between them little changes (192^3: a step 2.137 -> 2.123
+// ms, with haloes 4.22 -> 4.20); the line is the largest size with a clear gain.
+//
+// Launched plainly in every context, and so a link where the next kernel waits:
+// prep_positions (with chain() in it a 256^3 step took 4.99 instead of 4.97 ms) and, not
+// tried, pp_pencil, the placement, the list of cells to sort, the TSC deposit, the third
+// level's own kernels and the adjoint's mesh kernels.
 constexpr int64_t CHAINED_MAX = 1 << 21;
 
 __device__ __forceinline__ void chain() {
